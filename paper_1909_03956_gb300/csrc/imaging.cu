@@ -181,15 +181,26 @@ __global__ void k_image_from_fft(const float2* __restrict__ f, int n, const unsi
 // image above. K_w is tabulated at kWpOversample points per cell over the
 // support S = 2h + 1 cells (h from the largest chirp frequency of the field
 // and the Kaiser-Bessel half-width) for planes uniformly spaced in |w|,
-// from a midpoint sum over kWpSamples^2 points of the field (two complex
-// matrix products per plane), and interpolated linearly in |w| between the
-// two nearest planes; an entry at w < 0 takes conj(K_|w|(-x, -y)). Each
-// entry is spread over the support its own |w| needs (the same rule at that
-// |w|), not the table's.
+// from a midpoint sum over kWpSamples^2 points of the field, and interpolated
+// linearly in |w| between the two nearest planes. Each visibility stands for
+// two entries, V at B and conj(V) at -B; the image takes the real part of the
+// transform, and Re F(G + conj G(-.)) = 2 Re F(G), so one of them is gridded,
+// the one at w >= 0, and the image doubled (exact). Each entry is spread over
+// the support its own |w| needs (the same rule at that |w|), not the table's.
+//
+// The integrand is even in t and in s, and so is the table in x and in y: the
+// midpoint sum runs over the positive quadrant with real cosines, and one
+// quadrant of the table is computed (k_wp_stage1, k_wp_stage2: 16 times less
+// work than complex sums over the whole field, whose two products took 657 +
+// 230 us at 64 planes and h = 11; these take 17 + 17, latency bound, and
+// k_wp_field 19 us where float64 tapers and sincospi at every sample took
+// 420). k_wp_layout writes it out per offset within a cell, so that an entry's
+// taps are whole rows.
 constexpr int kWpWidth = 7;             // Kaiser-Bessel width (cells)
 constexpr double kWpBeta = 16.25;       // its shape parameter
 constexpr int kWpOversample = 8;        // table points per cell
 constexpr int kWpSamples = 128;         // field samples per axis for the kernels
+constexpr int kWpHalf = kWpSamples / 2; // those at t > 0
 constexpr int kWpMaxHalf = 32;          // largest half-support h (cells)
 
 // c(t) / c(0) for the Kaiser-Bessel kernel of width W and shape beta: the
@@ -212,48 +223,131 @@ __host__ __device__ inline double kb_taper(double t)
 
 struct WpPlan {
     int P;          // planes
-    int h, S, T;    // half-support, support (cells), table points per axis (S * oversample + 1)
+    int h, S;       // half-support, support (cells)
+    int Tc;         // table points at x >= 0: x_c = c / oversample, c = 0 .. (h + 1/2) oversample
     double dw;      // plane spacing in |w|
     double ndl;     // n dl: the field width (radians)
     double xc_per_w;   // the field's largest chirp frequency (cells) per unit |w|
 };
 
-// f[p][q][r] = c(t_q) c(t_r) exp(-i 2 pi w_p (n - 1)) at the field's sample
-// points t = (q + 1/2)/M - 1/2 (float64 phase reduced modulo 1).
-__global__ void k_wp_field(WpPlan pl, float2* __restrict__ f)
+__device__ __forceinline__ double wp_sample(int q) { return (q + 0.5) / kWpSamples; }   // t_q > 0
+
+// The tables of one image: ct[r][c] = cos(2 pi x_c t_r); ft[r] = c(t_r), the
+// field samples' taper; gc[i] = 1 / c((i - n/2) / n), the pixels' grid
+// correction, as a double-float.
+__global__ void k_wp_tables(WpPlan pl, int n, float* __restrict__ ct, double* __restrict__ ft, F2* __restrict__ gc)
 {
-    const int M = kWpSamples;
-    const int64_t total = static_cast<int64_t>(pl.P) * M * M;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int r = static_cast<int>(i % M), q = static_cast<int>((i / M) % M), p = static_cast<int>(i / (M * M));
-        const double tq = (q + 0.5) / M - 0.5, tr = (r + 0.5) / M - 0.5;
-        const double l = tq * pl.ndl, m = tr * pl.ndl;
-        const double r2 = l * l + m * m;
-        const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
-        double ph = -(p * pl.dw) * nm1;                // turns
-        ph -= rint(ph);
-        double sn, cs;
-        sincospi(2.0 * ph, &sn, &cs);
-        const double c = kb_taper(tq) * kb_taper(tr);
-        f[i] = make_float2(static_cast<float>(c * cs), static_cast<float>(c * sn));
+    const int nc = pl.Tc * kWpHalf, total = nc + kWpHalf + n;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        if (i < nc) {
+            const int r = i / pl.Tc, c = i % pl.Tc;
+            double ph = static_cast<double>(c) / kWpOversample * wp_sample(r);
+            ph -= rint(ph);
+            ct[i] = static_cast<float>(cospi(2.0 * ph));
+        } else if (i < nc + kWpHalf) {
+            ft[i - nc] = kb_taper(wp_sample(i - nc));
+        } else {
+            const int k = i - nc - kWpHalf;
+            gc[k] = split_f64(1.0 / kb_taper(static_cast<double>(k - n / 2) / n));
+        }
     }
 }
 
-// tw[j][q] = exp(i 2 pi x_j t_q), x_j = j / oversample - (h + 1/2).
-__global__ void k_wp_twiddles(WpPlan pl, float2* __restrict__ tw)
+// f[p][q][r] = c(t_q) c(t_r) exp(-i 2 pi w_p (n - 1)) at the field's sample
+// points t > 0 (float64 phase): a thread per (q, r), the planes of a group of
+// kWpFieldPlanes one after the other (n - 1 and the taper are theirs alike).
+constexpr int kWpFieldPlanes = 8;
+
+__global__ void k_wp_field(WpPlan pl, const double* __restrict__ ft, float2* __restrict__ f)
 {
-    const int M = kWpSamples;
-    const int total = pl.T * M;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int q = i % M, j = i / M;
-        const double x = static_cast<double>(j) / kWpOversample - (pl.h + 0.5);
-        const double t = (q + 0.5) / M - 0.5;
-        double ph = x * t;
-        ph -= rint(ph);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kWpHalf * kWpHalf) return;
+    const int r = i % kWpHalf, q = i / kWpHalf;
+    const double l = wp_sample(q) * pl.ndl, m = wp_sample(r) * pl.ndl;
+    const double r2 = l * l + m * m;
+    const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
+    const double c = ft[q] * ft[r];
+    const int p1 = min(pl.P, static_cast<int>(blockIdx.y + 1) * kWpFieldPlanes);
+    for (int p = blockIdx.y * kWpFieldPlanes; p < p1; ++p) {
         double sn, cs;
-        sincospi(2.0 * ph, &sn, &cs);
-        tw[i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+        sincos_turns_f64(-(p * pl.dw) * nm1, sn, cs);
+        f[static_cast<int64_t>(p) * kWpHalf * kWpHalf + i] =
+            make_float2(static_cast<float>(c * cs), static_cast<float>(c * sn));
+    }
+}
+
+// a[p][q][c] = sum_r f[p][q][r] ct[r][c]: a CTA per (plane, 8 rows q), threads over c.
+constexpr int kWpGroup = 8;
+
+__global__ void __launch_bounds__(128) k_wp_stage1(WpPlan pl, const float2* __restrict__ f,
+                                                   const float* __restrict__ ct, float2* __restrict__ a)
+{
+    __shared__ float2 row[kWpGroup][kWpHalf];
+    const int p = blockIdx.x, q0 = blockIdx.y * kWpGroup;
+    const float2* src = f + (static_cast<int64_t>(p) * kWpHalf + q0) * kWpHalf;
+    for (int i = threadIdx.x; i < kWpGroup * kWpHalf; i += blockDim.x) row[i / kWpHalf][i % kWpHalf] = src[i];
+    __syncthreads();
+    for (int c = threadIdx.x; c < pl.Tc; c += blockDim.x) {
+        float2 acc[kWpGroup];
+#pragma unroll
+        for (int g = 0; g < kWpGroup; ++g) acc[g] = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int r = 0; r < kWpHalf; ++r) {
+            const float2 t = bcast2(__ldg(ct + r * pl.Tc + c));
+#pragma unroll
+            for (int g = 0; g < kWpGroup; ++g) acc[g] = fma2(row[g][r], t, acc[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < kWpGroup; ++g)
+            a[(static_cast<int64_t>(p) * kWpHalf + q0 + g) * pl.Tc + c] = acc[g];
+    }
+}
+
+// K_q[p][i][c] = (4/M^2) sum_q ct[q][i] a[p][q][c], one quadrant of the
+// table: a CTA per (plane, 8 rows i), threads over c.
+__global__ void __launch_bounds__(128) k_wp_stage2(WpPlan pl, const float2* __restrict__ a,
+                                                   const float* __restrict__ ct, float2* __restrict__ Kq)
+{
+    __shared__ float col[kWpHalf][kWpGroup];
+    const int p = blockIdx.x, i0 = blockIdx.y * kWpGroup;
+    for (int k = threadIdx.x; k < kWpGroup * kWpHalf; k += blockDim.x) {
+        const int q = k / kWpGroup, g = k % kWpGroup;
+        col[q][g] = i0 + g < pl.Tc ? ct[q * pl.Tc + i0 + g] : 0.0f;
+    }
+    __syncthreads();
+    const float inv = 4.0f / (static_cast<float>(kWpSamples) * static_cast<float>(kWpSamples));
+    for (int c = threadIdx.x; c < pl.Tc; c += blockDim.x) {
+        float2 acc[kWpGroup];
+#pragma unroll
+        for (int g = 0; g < kWpGroup; ++g) acc[g] = make_float2(0.f, 0.f);
+        const float2* ap = a + static_cast<int64_t>(p) * kWpHalf * pl.Tc + c;
+#pragma unroll 8
+        for (int q = 0; q < kWpHalf; ++q) {
+            const float2 v = __ldg(ap + q * pl.Tc);
+#pragma unroll
+            for (int g = 0; g < kWpGroup; ++g) acc[g] = fma2(v, bcast2(col[q][g]), acc[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < kWpGroup; ++g)
+            if (i0 + g < pl.Tc)
+                Kq[(static_cast<int64_t>(p) * pl.Tc + i0 + g) * pl.Tc + c] =
+                    make_float2(acc[g].x * inv, acc[g].y * inv);
+    }
+}
+
+// The table as the gridding reads it: K[p][oy][ox][ty][tx], ty, tx = 0 .. S,
+// the point x = tx + ox / oversample - (h + 1/2), y likewise (0 beyond the
+// support): a CTA per (p, oy, ox).
+__global__ void k_wp_layout(WpPlan pl, const float2* __restrict__ Kq, float2* __restrict__ K)
+{
+    constexpr int O = kWpOversample;
+    const int R = pl.S + 1, oy = (blockIdx.x / O) % O, ox = blockIdx.x % O;
+    const float2* src = Kq + static_cast<int64_t>(blockIdx.x / (O * O)) * pl.Tc * pl.Tc;
+    float2* dst = K + static_cast<int64_t>(blockIdx.x) * R * R;
+    const int mid = pl.Tc - 1;   // the table index of x = 0
+    for (int i = threadIdx.x; i < R * R; i += blockDim.x) {
+        const int cy = abs(O * (i / R) + oy - mid), cx = abs(O * (i % R) + ox - mid);
+        dst[i] = cy <= mid && cx <= mid ? __ldg(src + cy * pl.Tc + cx) : make_float2(0.f, 0.f);
     }
 }
 
@@ -262,133 +356,167 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-// a[p][q][j] = sum_r f[p][q][r] tw[j][r]: one CTA per (p, q), threads over j.
-__global__ void k_wp_stage1(WpPlan pl, const float2* __restrict__ f, const float2* __restrict__ tw,
-                            float2* __restrict__ a)
+// An entry whose offsets sit within kWpTie of a tie between two table points
+// (in units of the table's spacing): float32 rounds the taps' positions to
+// their nearest points one by one, each entry of the Hermitian pair by itself,
+// and near a tie they need not agree. Three float32 roundings of positions
+// below 2 kWpMaxHalf + 1 cells, 2^-19 each, times the oversampling: below
+// 2^-14.
+constexpr float kWpTie = 1.0f / 8192;
+
+__device__ __forceinline__ float2 wp_mix(float2 k0, float2 k1, float a)
 {
-    const int M = kWpSamples;
-    __shared__ float2 row[kWpSamples];
-    const int64_t pq = blockIdx.x;
-    for (int r = threadIdx.x; r < M; r += blockDim.x) row[r] = f[pq * M + r];
-    __syncthreads();
-    for (int j = threadIdx.x; j < pl.T; j += blockDim.x) {
-        float2 acc = make_float2(0.f, 0.f);
-        const float2* t = tw + static_cast<int64_t>(j) * M;
-        for (int r = 0; r < M; ++r) {
-            const float2 b = cmul(row[r], t[r]);
-            acc.x += b.x;
-            acc.y += b.y;
-        }
-        a[pq * pl.T + j] = acc;
-    }
+    return make_float2(fmaf(a, k1.x - k0.x, k0.x), fmaf(a, k1.y - k0.y, k0.y));
 }
 
-// K[p][i][j] = (1/M^2) sum_q tw[i][q] a[p][q][j]: one CTA per (p, i).
-__global__ void k_wp_stage2(WpPlan pl, const float2* __restrict__ a, const float2* __restrict__ tw,
-                            float2* __restrict__ K)
+// The general form of an entry (V at cell (uc, vc) of the grid, half-support
+// he, offsets fx, fy): every tap finds its table point in both entries of the
+// pair, and where they differ takes their mean, as gridding both would.
+__device__ __noinline__ void wp_spread_ties(const WpPlan& pl, const float2* __restrict__ K0, float a, float2 V,
+                                            int uc, int vc, int he, float fx, float fy, int n,
+                                            float2* __restrict__ grid, int lane)
 {
-    const int M = kWpSamples;
-    __shared__ float2 col[kWpSamples];
-    const int p = blockIdx.x / pl.T, i = blockIdx.x % pl.T;
-    for (int q = threadIdx.x; q < M; q += blockDim.x) col[q] = tw[static_cast<int64_t>(i) * M + q];
-    __syncthreads();
-    const float inv = 1.0f / (static_cast<float>(M) * static_cast<float>(M));
-    for (int j = threadIdx.x; j < pl.T; j += blockDim.x) {
-        float2 acc = make_float2(0.f, 0.f);
-        const float2* ap = a + (static_cast<int64_t>(p) * M) * pl.T + j;
-        for (int q = 0; q < M; ++q) {
-            const float2 b = cmul(col[q], ap[static_cast<int64_t>(q) * pl.T]);
-            acc.x += b.x;
-            acc.y += b.y;
-        }
-        K[(static_cast<int64_t>(p) * pl.T + i) * pl.T + j] = make_float2(acc.x * inv, acc.y * inv);
-    }
-}
-
-// One entry (V at x, y cells and w) into the grid by a warp, lanes over the
-// S x S taps; false if its support leaves the grid (the entry is dropped).
-__device__ __forceinline__ bool wp_entry(const WpPlan& pl, const float2* __restrict__ K, float2 V, double x,
-                                         double y, double w, int n, float2* __restrict__ grid, int lane)
-{
-    const double icd = rint(x), jcd = rint(y);
-    const int half = n / 2;
-    const double lo = -half + pl.h + 1, hi = half - pl.h - 1;
-    if (!(icd >= lo && icd <= hi && jcd >= lo && jcd <= hi && fabs(w) <= 1e30))   // false for NaN too
-        return false;
-    const int ic = static_cast<int>(icd), jc = static_cast<int>(jcd);
-    const float fx = static_cast<float>(x - icd), fy = static_cast<float>(y - jcd);
-    const bool neg = w < 0.0;
-    double pw = fabs(w) / pl.dw;
-    int p0 = static_cast<int>(floor(pw));
-    if (p0 > pl.P - 2) p0 = pl.P - 2;
-    if (p0 < 0) p0 = 0;
-    const float a = static_cast<float>(fmin(fmax(pw - p0, 0.0), 1.0));
-    const int last = pl.S * kWpOversample;                         // the table's last index
-    const float2* K0 = K + static_cast<int64_t>(p0) * pl.T * pl.T;
-    const float2* K1 = K0 + static_cast<int64_t>(pl.T) * pl.T;
-    // this entry's own support: the Kaiser-Bessel half-width and the chirp
-    // frequency of its |w| (the kernel is negligible beyond), within the table's
-    int he = static_cast<int>(ceil(0.5 * kWpWidth + pl.xc_per_w * fabs(w))) + 1;
-    he = he < pl.h ? he : pl.h;
-    const int Se = 2 * he + 1;
-    const int taps = Se * Se;
-    for (int t = lane; t < taps; t += 32) {
+    constexpr int O = kWpOversample;
+    const int R = pl.S + 1, last = pl.S * O, Se = 2 * he + 1;
+    const float2* K1 = K0 + static_cast<int64_t>(O) * O * R * R;
+    auto index = [&](int d, float f) { return __float2int_rn((static_cast<float>(d) - f + pl.h + 0.5f) * O); };
+    auto value = [&](int ix, int iy) {
+        const int at = ((iy % O) * O + ix % O) * R * R + (iy / O) * R + ix / O;
+        return wp_mix(__ldg(K0 + at), __ldg(K1 + at), a);
+    };
+    for (int t = lane; t < Se * Se; t += 32) {
         const int dx = t % Se - he, dy = t / Se - he;
-        int ix = __float2int_rn((static_cast<float>(dx) - fx + pl.h + 0.5f) * kWpOversample);
-        int iy = __float2int_rn((static_cast<float>(dy) - fy + pl.h + 0.5f) * kWpOversample);
-        ix = min(max(ix, 0), last);
-        iy = min(max(iy, 0), last);
-        if (neg) {                                                 // conj(K_|w|(-x, -y))
-            ix = last - ix;
-            iy = last - iy;
-        }
-        const int64_t off = static_cast<int64_t>(ix) * pl.T + iy;  // table [x][y]
-        const float2 k0 = K0[off], k1 = K1[off];
-        float2 k = make_float2(fmaf(a, k1.x - k0.x, k0.x), fmaf(a, k1.y - k0.y, k0.y));
-        if (neg) k.y = -k.y;
-        const int iu = ic + dx + half, iv = jc + dy + half;
-        const float sg = ((iu + iv) & 1) ? -1.0f : 1.0f;            // the index shift (-1)^(iu+iv)
-        const float2 e = cmul(V, k);
-        float* g = reinterpret_cast<float*>(grid + static_cast<int64_t>(iv) * n + iu);
-        atomicAdd(g, sg * e.x);
-        atomicAdd(g + 1, sg * e.y);
+        const float2 k0 = value(index(dx, fx), index(dy, fy));
+        const float2 k1 = value(last - index(-dx, -fx), last - index(-dy, -fy));
+        const float sg = ((uc + dx + vc + dy) & 1) ? -0.5f : 0.5f;
+        const float2 e = cmul(V, make_float2(k0.x + k1.x, k0.y + k1.y));
+        atomicAdd(grid + static_cast<int64_t>(vc + dy) * n + uc + dx, make_float2(sg * e.x, sg * e.y));
     }
-    return true;
 }
 
-// A warp per visibility: the visibility (unit value if vis is null) and its
-// conjugate at -B; counts the entries gridded.
-__global__ void k_grid_wproj(WpPlan pl, const float2* __restrict__ K, const double* __restrict__ uvw,
-                             const float2* __restrict__ vis, int64_t n_vis, int n, double inv_du,
-                             float2* __restrict__ grid, unsigned long long* __restrict__ count)
+// A warp takes `group` visibilities (unit values if vis is null): each of its
+// first `group` lanes plans one (cell, offset, planes, support: float64 work
+// that a whole warp would repeat), then the warp spreads them one after the
+// other, a lane per aligned pair of cells of a row, 32 / L rows at a time
+// (L lanes cover a row). An entry whose support leaves the grid is dropped;
+// counts two entries per visibility gridded.
+// Bound by L2: per tap 16 bytes of table (two planes, rows of the layout) and
+// an 8-byte addition to the grid, two cells per 16-byte atomic. Medium array,
+// 1 008 000 visibilities, 2048 x 2048, 64 planes: 0.51 ms, against 3.0 ms
+// for both entries of each visibility with 4-byte atomics and a table read
+// across its rows.
+__global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __restrict__ K,
+                                                    const double* __restrict__ uvw, const float2* __restrict__ vis,
+                                                    int64_t n_vis, int n, double inv_du, int group,
+                                                    float2* __restrict__ grid, unsigned long long* __restrict__ count)
 {
+    constexpr int O = kWpOversample;
+    __shared__ unsigned int blk;
+    if (threadIdx.x == 0) blk = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x / 32);
-    unsigned long long mine = 0;
-    for (int64_t k = static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5); k < n_vis;
-         k += warps) {
-        const double x = uvw[3 * k] * inv_du, y = uvw[3 * k + 1] * inv_du, w = uvw[3 * k + 2];
-        const float2 V = vis ? vis[k] : make_float2(1.0f, 0.0f);
-        const bool in = wp_entry(pl, K, V, x, y, w, n, grid, lane);
-        if (in) wp_entry(pl, K, make_float2(V.x, -V.y), -x, -y, -w, n, grid, lane);
-        if (in && lane == 0) mine += 2;
+    const int R = pl.S + 1, half = n / 2;
+    const int64_t k = (static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5)) * group + lane;
+    // the plan of this lane's visibility: its cell, half-support, lower plane,
+    // table row and column of the first tap (-1: near a tie), offset from the
+    // cell's centre and weight between the planes
+    int uc = 0, vc = 0, he = -1, p0 = 0, tab = -1;
+    float fx = 0.0f, fy = 0.0f, a = 0.0f;
+    float2 V = make_float2(0.f, 0.f);
+    if (lane < group && k < n_vis) {
+        double x = uvw[3 * k] * inv_du, y = uvw[3 * k + 1] * inv_du, w = uvw[3 * k + 2];
+        V = vis ? vis[k] : make_float2(1.0f, 0.0f);
+        if (w < 0.0) {               // the conjugate entry
+            x = -x;
+            y = -y;
+            w = -w;
+            V.y = -V.y;
+        }
+        const double icd = rint(x), jcd = rint(y);
+        const double lo = -half + pl.h + 1, hi = half - pl.h - 1;
+        if (icd >= lo && icd <= hi && jcd >= lo && jcd <= hi && w <= 1e30) {   // false for NaN too
+            fx = static_cast<float>(x - icd);
+            fy = static_cast<float>(y - jcd);
+            const double pw = w / pl.dw;
+            p0 = static_cast<int>(floor(pw));
+            if (p0 > pl.P - 2) p0 = pl.P - 2;
+            if (p0 < 0) p0 = 0;
+            a = static_cast<float>(fmin(fmax(pw - p0, 0.0), 1.0));
+            // this entry's own support: the Kaiser-Bessel half-width and the
+            // chirp frequency of its |w| (the kernel is negligible beyond),
+            // within the table's
+            he = static_cast<int>(fmin(ceil(0.5 * kWpWidth + pl.xc_per_w * w) + 1.0, static_cast<double>(pl.h)));
+            uc = static_cast<int>(icd) + half;
+            vc = static_cast<int>(jcd) + half;
+            // tap d's nearest table point is at (d - fx + h + 1/2) oversample:
+            // d + h cells and an offset o = 0 .. oversample alike for every tap
+            // (o = oversample: the next cell's 0)
+            const float gx = (0.5f - fx) * O, gy = (0.5f - fy) * O;
+            const int ox = __float2int_rn(gx), oy = __float2int_rn(gy);
+            if (fabsf(fabsf(gx - ox) - 0.5f) > kWpTie && fabsf(fabsf(gy - oy) - 0.5f) > kWpTie)
+                tab = (((oy % O) * O + ox % O) * R + pl.h - he + oy / O) * R + pl.h - he + ox / O;
+        }
     }
-    if (lane == 0 && mine) atomicAdd(count, mine);
+    const unsigned todo = __ballot_sync(0xffffffffu, he >= 0);
+    if (lane == 0 && todo) atomicAdd(&blk, 2u * __popc(todo));
+    const int64_t plane = static_cast<int64_t>(O) * O * R * R;
+    for (unsigned left = todo; left; left &= left - 1) {
+        const int src = __ffs(left) - 1;
+        const int su = __shfl_sync(0xffffffffu, uc, src), sv = __shfl_sync(0xffffffffu, vc, src);
+        const int sh = __shfl_sync(0xffffffffu, he, src), st = __shfl_sync(0xffffffffu, tab, src);
+        const int sp = __shfl_sync(0xffffffffu, p0, src);
+        const float sa = __shfl_sync(0xffffffffu, a, src);
+        const float2 sV = make_float2(__shfl_sync(0xffffffffu, V.x, src), __shfl_sync(0xffffffffu, V.y, src));
+        const float2* K0 = K + sp * plane;
+        if (st < 0) {
+            const float sx = __shfl_sync(0xffffffffu, fx, src), sy = __shfl_sync(0xffffffffu, fy, src);
+            wp_spread_ties(pl, K0, sa, sV, su, sv, sh, sx, sy, n, grid, lane);
+            continue;
+        }
+        K0 += st;
+        const float2* K1 = K0 + plane;
+        const int Se = 2 * sh + 1, u0 = su - sh, v0 = sv - sh;   // the first tap's cell
+        const int ua = u0 & ~1;                            // even: a pair of cells is 16-byte aligned
+        const int pairs = (u0 + Se - ua + 1) >> 1;
+        const int lg = pairs <= 8 ? 3 : pairs <= 16 ? 4 : 5;   // log2 of the lanes per row
+        for (int r = lane >> lg; r < Se; r += 32 >> lg) {
+            const float sg = ((v0 + r) & 1) ? -1.0f : 1.0f;    // the index shift (-1)^(iu+iv), iu even
+            float4* out = reinterpret_cast<float4*>(grid + static_cast<int64_t>(v0 + r) * n + ua);
+            for (int q = lane & ((1 << lg) - 1); q < pairs; q += 1 << lg) {
+                float2 e[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int t = 2 * q + j + ua - u0;         // tap -1 and Se: outside the support
+                    e[j] = make_float2(0.f, 0.f);
+                    if (t >= 0 && t < Se) e[j] = cmul(sV, wp_mix(__ldg(K0 + r * R + t), __ldg(K1 + r * R + t), sa));
+                }
+                atomicAdd(out + q, make_float4(sg * e[0].x, sg * e[0].y, -sg * e[1].x, -sg * e[1].y));
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && blk) atomicAdd(count, static_cast<unsigned long long>(blk));
 }
 
-// Real part of the transformed grid, times (-1)^(ix+iy) / (W c(t) c(s)).
+// Twice the real part of the transformed grid, times
+// (-1)^(ix+iy) / (W c(t) c(s)), the correction's product in double-float.
+// Bound by HBM (12 bytes per pixel); with both tapers evaluated per pixel in
+// float64 714 us at 2048 x 2048, 23 us so.
 __global__ void k_image_from_fft_wp(const float2* __restrict__ f, int n, const unsigned long long* __restrict__ count,
-                                    float* __restrict__ image)
+                                    const F2* __restrict__ gc, float* __restrict__ image)
 {
     const unsigned long long W = *count;
-    const double inv = W ? 1.0 / static_cast<double>(W) : 0.0;
+    const double inv = W ? 2.0 / static_cast<double>(W) : 0.0;
     for (int iy = blockIdx.x; iy < n; iy += gridDim.x) {
         const int64_t row = static_cast<int64_t>(iy) * n;
-        const double cy = kb_taper(static_cast<double>(iy - n / 2) / n);
+        const F2 g = gc[iy];
+        const F2 cy = split_f64((static_cast<double>(g.hi) + static_cast<double>(g.lo)) * inv);
         for (int ix = threadIdx.x; ix < n; ix += blockDim.x) {
             const float sg = ((ix + iy) & 1) ? -1.0f : 1.0f;
-            const double c = kb_taper(static_cast<double>(ix - n / 2) / n) * cy;
-            image[row + ix] = static_cast<float>(sg * f[row + ix].x * inv / c);
+            float p, t;
+            df_product(cy, gc[ix], p, t);
+            const float v = sg * f[row + ix].x;
+            image[row + ix] = fmaf(v, p, v * t);
         }
     }
 }
@@ -941,10 +1069,13 @@ namespace wt {
 namespace {
 
 // The largest |w| of the visibilities as float64 bits (non-negative doubles
-// order as their bits); *out zeroed before the launch.
-__global__ void k_max_abs_w(const double* __restrict__ uvw, int64_t n_vis, unsigned long long* __restrict__ out)
+// order as their bits); *out zeroed before the launch. One atomic per CTA of
+// 256 threads, at most four CTAs per SM (an atomic per warp of a thread per
+// visibility: 28 us against 10 for 1 008 000).
+__global__ void __launch_bounds__(256) k_max_abs_w(const double* __restrict__ uvw, int64_t n_vis, unsigned long long* __restrict__ out)
 {
     unsigned long long m = 0;
+#pragma unroll 4
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_vis;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const double w = fabs(uvw[3 * i + 2]);
@@ -958,7 +1089,13 @@ __global__ void k_max_abs_w(const double* __restrict__ uvw, int64_t n_vis, unsig
         const unsigned long long other = __shfl_xor_sync(0xffffffffu, m, o);
         m = other > m ? other : m;
     }
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+    __shared__ unsigned long long wm[8];
+    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) m = wm[i] > m ? wm[i] : m;
+        if (m) atomicMax(out, m);
+    }
 }
 
 // The batch's largest finite |w| (1 if none is above 0); synchronises s.
@@ -970,7 +1107,7 @@ int max_abs_w(const double* uvw, int64_t n_vis, cudaStream_t s, double* out)
     cudaError_t e = cudaMemsetAsync(d, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess && n_vis > 0) {
         int64_t b = (n_vis + 255) / 256;
-        if (b > 4096) b = 4096;
+        if (b > 4 * num_sms()) b = 4 * num_sms();
         k_max_abs_w<<<static_cast<unsigned>(b), 256, 0, s>>>(uvw, n_vis, d);
         e = cudaGetLastError();
     }
@@ -1010,46 +1147,61 @@ int dirty_image_w(const double* uvw, const float2* vis, int64_t n_vis, int n, do
     if (2 * pl.h + 2 >= n / 2) return set_error(WT_ERR_RANGE, "%s: a %d-cell kernel does not fit an n = %d grid", fn,
                                                 2 * pl.h + 1, n);
     pl.S = 2 * pl.h + 1;
-    pl.T = pl.S * kWpOversample + 1;
-    const int M = kWpSamples;
+    pl.Tc = pl.S * kWpOversample / 2 + 1;
+    constexpr int H = kWpHalf, O = kWpOversample;
     auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t b_grid = up(nn * sizeof(float2)), b_cnt = 256;
-    const size_t b_f = up(static_cast<size_t>(planes) * M * M * sizeof(float2));
-    const size_t b_tw = up(static_cast<size_t>(pl.T) * M * sizeof(float2));
-    const size_t b_a = up(static_cast<size_t>(planes) * M * pl.T * sizeof(float2));
-    const size_t b_k = up(static_cast<size_t>(planes) * pl.T * pl.T * sizeof(float2));
+    const size_t b_ct = up(static_cast<size_t>(pl.Tc) * H * sizeof(float));
+    const size_t b_ft = up(H * sizeof(double)), b_gc = up(static_cast<size_t>(n) * sizeof(F2));
+    const size_t b_f = up(static_cast<size_t>(planes) * H * H * sizeof(float2));
+    const size_t b_a = up(static_cast<size_t>(planes) * H * pl.Tc * sizeof(float2));
+    const size_t b_q = up(static_cast<size_t>(planes) * pl.Tc * pl.Tc * sizeof(float2));
+    const size_t b_k = up(static_cast<size_t>(planes) * O * O * (pl.S + 1) * (pl.S + 1) * sizeof(float2));
     char* scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), b_grid + b_cnt + b_f + b_tw + b_a + b_k, s);
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch),
+                                    b_grid + b_cnt + b_ct + b_ft + b_gc + b_f + b_a + b_q + b_k, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(WT_ERR_NOMEM, "%s: scratch allocation failed: %s", fn, cudaGetErrorString(e));
     }
-    float2* grid = reinterpret_cast<float2*>(scratch);
-    unsigned long long* count = reinterpret_cast<unsigned long long*>(scratch + b_grid);
-    float2* f = reinterpret_cast<float2*>(scratch + b_grid + b_cnt);
-    float2* tw = reinterpret_cast<float2*>(scratch + b_grid + b_cnt + b_f);
-    float2* a = reinterpret_cast<float2*>(scratch + b_grid + b_cnt + b_f + b_tw);
-    float2* K = reinterpret_cast<float2*>(scratch + b_grid + b_cnt + b_f + b_tw + b_a);
+    char* at = scratch;
+    auto take = [&](size_t b) {
+        char* r = at;
+        at += b;
+        return r;
+    };
+    float2* grid = reinterpret_cast<float2*>(take(b_grid));
+    unsigned long long* count = reinterpret_cast<unsigned long long*>(take(b_cnt));
+    float* ct = reinterpret_cast<float*>(take(b_ct));
+    double* ft = reinterpret_cast<double*>(take(b_ft));
+    F2* gc = reinterpret_cast<F2*>(take(b_gc));
+    float2* f = reinterpret_cast<float2*>(take(b_f));
+    float2* a = reinterpret_cast<float2*>(take(b_a));
+    float2* Kq = reinterpret_cast<float2*>(take(b_q));
+    float2* K = reinterpret_cast<float2*>(take(b_k));
     int rc = WT_OK;
-    const int64_t nf = static_cast<int64_t>(planes) * M * M;
-    k_wp_field<<<static_cast<unsigned>(std::min<int64_t>((nf + 255) / 256, 8192)), 256, 0, s>>>(pl, f);
-    k_wp_twiddles<<<(pl.T * M + 255) / 256, 256, 0, s>>>(pl, tw);
-    k_wp_stage1<<<static_cast<unsigned>(planes * M), 128, 0, s>>>(pl, f, tw, a);
-    k_wp_stage2<<<static_cast<unsigned>(planes * pl.T), 128, 0, s>>>(pl, a, tw, K);
+    k_wp_tables<<<(pl.Tc * H + H + n + 127) / 128, 128, 0, s>>>(pl, n, ct, ft, gc);
+    k_wp_field<<<dim3((H * H + 127) / 128, (planes + kWpFieldPlanes - 1) / kWpFieldPlanes), 128, 0, s>>>(pl, ft, f);
+    k_wp_stage1<<<dim3(planes, H / kWpGroup), 128, 0, s>>>(pl, f, ct, a);
+    k_wp_stage2<<<dim3(planes, (pl.Tc + kWpGroup - 1) / kWpGroup), 128, 0, s>>>(pl, a, ct, Kq);
+    k_wp_layout<<<static_cast<unsigned>(planes * O * O), 256, 0, s>>>(pl, Kq, K);
     if (cudaGetLastError() != cudaSuccess) rc = set_error(WT_ERR_CUDA, "%s: kernel tables", fn);
     if (rc == WT_OK && (cudaMemsetAsync(grid, 0, static_cast<size_t>(nn) * sizeof(float2), s) != cudaSuccess ||
                         cudaMemsetAsync(count, 0, sizeof(unsigned long long), s) != cudaSuccess))
         rc = set_error(WT_ERR_CUDA, "%s: clearing the grid", fn);
     if (rc == WT_OK && n_vis > 0) {
-        int64_t b = (n_vis + 7) / 8;                   // 8 warps per CTA, a warp per visibility
-        const int64_t cap = static_cast<int64_t>(num_sms()) * 32;
-        if (b > cap) b = cap;
-        k_grid_wproj<<<static_cast<unsigned>(b), 256, 0, s>>>(pl, K, uvw, vis, n_vis, n, ndl, grid, count);
+        // 32 visibilities per warp, fewer for a batch that would leave the
+        // chip short of warps (32 per SM)
+        int group = 32;
+        while (group > 4 && n_vis < static_cast<int64_t>(num_sms()) * 32 * group) group /= 2;
+        const int64_t per_cta = 8 * group;
+        k_grid_wproj<<<static_cast<unsigned>((n_vis + per_cta - 1) / per_cta), 256, 0, s>>>(
+            pl, K, uvw, vis, n_vis, n, ndl, group, grid, count);
         if (cudaGetLastError() != cudaSuccess) rc = set_error(WT_ERR_CUDA, "%s: gridding launch", fn);
     }
     if (rc == WT_OK) rc = fft2_forward(grid, n, s);
     if (rc == WT_OK) {
-        k_image_from_fft_wp<<<rows_blocks(n), kImgThreads, 0, s>>>(grid, n, count, image);
+        k_image_from_fft_wp<<<rows_blocks(n), kImgThreads, 0, s>>>(grid, n, count, gc, image);
         if (cudaGetLastError() != cudaSuccess) rc = set_error(WT_ERR_CUDA, "%s: image launch", fn);
     }
     const cudaError_t ef = cudaFreeAsync(scratch, s);
