@@ -59,51 +59,89 @@ __device__ __forceinline__ DF df_from_double(double x)
     return DF{h, __double2float_rn(x - static_cast<double>(h))};
 }
 
-// 2 pi and -1/6 as double-floats (the float32 rounding and its remainder)
-constexpr float kTwoPiH = 6.2831854820251465f, kTwoPiL = -1.7484555314695172e-07f;
-constexpr float kMinusSixthH = -0.1666666716337204f, kMinusSixthL = 4.967053879312289e-09f;
-
-// exp(i 2 pi t) as double-floats for t = th + tl turns, |th| <= 1/2 and tl
-// small (the phase of phase_turns_df). The table method of the float64 form
-// (P. T. P. Tang, ACM TOMS 15(2), 1989) carried out in double-float:
-// k = rint(256 th), f = (th - k/256) + tl (the difference exact, the sum
-// error-free), x = 2 pi f (|x| <= 0.0123 plus the tail), then
-//   sin x = x - x^3/6 + x^5/120 - x^7/5040,  cos x = 1 - x^2/2 + x^4/24 - x^6/720
-// with the terms down to x^3 and x^2 in double-float and the rest, below
-// 2.5e-12 and 1e-9, in float32 (their rounding stays below 1e-16), and
-// finally the rotation by the table entry exp(i 2 pi k/256) = C + i S,
-// tab[k + 128] = (C h, C l, S h, S l).
-__device__ __forceinline__ void sincos_turns_df(float th, float tl, const float4* __restrict__ tab, DF& s, DF& c)
+// Sum of many double-floats: sum + x with the head's rounding error and the
+// low parts gathered in the low part, not renormalised. The head's sum is
+// error-free; the low part holds rounding errors and low parts only, so its
+// own rounding stays 2^-24 below theirs. Eight operations against df_add's 11.
+__device__ __forceinline__ void df_accumulate(DF& sum, float xh, float xl)
 {
-    const float k = rintf(__fmul_rn(th, 256.0f));
-    float fh, fl;
-    two_sum(__fmaf_rn(k, -0.00390625f, th), tl, fh, fl);
-    const DF x = df_mul(DF{fh, fl}, DF{kTwoPiH, kTwoPiL});
-    const DF x2 = df_mul(x, x);
-    const DF x3 = df_mul(x2, x);
-    const float q = x2.h;
-    const float small_s = __fmul_rn(__fmul_rn(x3.h, q), __fmaf_rn(q, -1.9841269841269841e-4f, 8.3333333333333333e-3f));
-    const float small_c = __fmul_rn(__fmul_rn(q, q), __fmaf_rn(q, -1.3888888888888889e-3f, 4.1666666666666667e-2f));
-    const DF sx = df_add_f(df_add(x, df_mul(x3, DF{kMinusSixthH, kMinusSixthL})), small_s);
-    const DF cx = df_add_f(df_add_f(df_neg(df_scale(x2, 0.5f)), 1.0f), small_c);
-    const float4 e = tab[static_cast<int>(k) + 128];
-    const DF C{e.x, e.y}, S{e.z, e.w};
-    c = df_add(df_mul(C, cx), df_neg(df_mul(S, sx)));
-    s = df_add(df_mul(S, cx), df_mul(C, sx));
+    float s, e;
+    two_sum(sum.h, xh, s, e);
+    sum.h = s;
+    sum.l = __fadd_rn(sum.l, __fadd_rn(e, xl));
 }
 
-constexpr int kDfTableEntries = 257;
+// a b as an unevaluated p + e (df_mul without the renormalisation).
+__device__ __forceinline__ void df_product_raw(DF a, DF b, float& p, float& e)
+{
+    p = __fmul_rn(a.h, b.h);
+    e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
+}
 
-// The table of exp(i 2 pi k/256), k = -128 .. 128, as double-floats, from
-// the correctly rounded float64 table of the float64 form: 257 entries,
-// written by the CTA's threads into shared memory.
+__device__ __forceinline__ void df_accumulate_product(DF& sum, DF a, DF b)
+{
+    float p, e;
+    df_product_raw(a, b, p, e);
+    df_accumulate(sum, p, e);
+}
+
+// 2 pi as a double-float (the float32 rounding and its remainder)
+constexpr float kTwoPiH = 6.2831854820251465f, kTwoPiL = -1.7484555314695172e-07f;
+
+// exp(i 2 pi t) as double-floats (unevaluated sums, the low part within a few
+// ulp of the head) for t = th + tl turns, |th| <= 1/2 and tl small (the phase
+// of phase_turns_df). The table method of the float64 form (P. T. P. Tang, ACM
+// TOMS 15(2), 1989) carried out in double-float: k = rint(1024 t), f = (th -
+// k/1024) + tl (the difference exact, the sum error-free), x = 2 pi f, |x| <=
+// 0.0031,
+//   sin x = x - x^3/6 + x^5/120,  cos x - 1 = -x^2/2 + x^4/24
+// (truncated below 6e-22 and 2e-18), x and x^2 in double-float and the rest,
+// below 5e-9 and 4e-12, in float32 (rounded below 3e-16); then the rotation of
+// the table entry C + i S, tab[k mod 1024] = (C h, C l, S h, S l), by the small
+// angle, C + (C (cos x - 1) - S sin x) and S + (S (cos x - 1) + C sin x), whose
+// two products are added to the entry's head error-free one after the other.
+// 74 operations of the float32 pipe; with 256 entries, where x^3 and the
+// cosine itself need double-floats renormalised at every step, 135. With the
+// sums left unnormalised (df_accumulate) the medium regrouped sum went from
+// 9.4 to 6.7 ms at the same error (2e-12).
+__device__ __forceinline__ void sincos_turns_df(float th, float tl, const float4* __restrict__ tab, DF& s, DF& c)
+{
+    const float k = rintf(__fmul_rn(__fadd_rn(th, tl), 1024.0f));
+    float fh, fl;
+    two_sum(__fmaf_rn(k, -0.0009765625f, th), tl, fh, fl);
+    const float4 e = tab[static_cast<int>(k) & 1023];
+    const float xh = __fmul_rn(fh, kTwoPiH);
+    const float xe = __fmaf_rn(fh, kTwoPiL, __fmaf_rn(fl, kTwoPiH, __fmaf_rn(fh, kTwoPiH, -xh)));
+    const float q = __fmul_rn(xh, xh);
+    const float qe = __fmaf_rn(__fadd_rn(xh, xh), xe, __fmaf_rn(xh, xh, -q));
+    const DF sx{xh, __fmaf_rn(__fmul_rn(xh, q), __fmaf_rn(q, 8.3333333333333333e-3f, -1.6666666666666667e-1f), xe)};
+    const DF cm{__fmul_rn(-0.5f, q), __fmaf_rn(__fmul_rn(q, q), 4.1666666666666667e-2f, __fmul_rn(-0.5f, qe))};
+    const DF C{e.x, e.y}, S{e.z, e.w};
+    float p, pe;
+    c = C;
+    df_product_raw(S, sx, p, pe);
+    df_accumulate(c, -p, -pe);
+    df_product_raw(C, cm, p, pe);
+    df_accumulate(c, p, pe);
+    s = S;
+    df_product_raw(C, sx, p, pe);
+    df_accumulate(s, p, pe);
+    df_product_raw(S, cm, p, pe);
+    df_accumulate(s, p, pe);
+}
+
+constexpr int kDfTableEntries = 1024;
+
+static __device__ const float4 kSinCosDF[kDfTableEntries] =
+#include "sincos_table_df.inc"
+    ;
+
+// The table of exp(i 2 pi k/1024), k = 0 .. 1023, as double-floats, copied by
+// the CTA's threads into shared memory.
 __device__ __forceinline__ void load_sincos_table_df(float4* tab)
 {
-    for (int i = threadIdx.x; i < kDfTableEntries; i += blockDim.x) {
-        const double2 e = kSinCos256[i];
-        const DF c = df_from_double(e.x), s = df_from_double(e.y);
-        tab[i] = make_float4(c.h, c.l, s.h, s.l);
-    }
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kDfTableEntries; i += blockDim.x) tab[i] = __ldg(&kSinCosDF[i]);
 }
 
 }  // namespace wt

@@ -145,8 +145,8 @@ struct BodyDF {
         DF s, co;
         sincos_turns_df(th, tl, tab, s, co);
         const DF f{c.flux, c.flux_lo};
-        vr = df_add(vr, df_mul(f, co));
-        vi = df_add(vi, df_mul(f, s));
+        df_accumulate_product(vr, f, co);
+        df_accumulate_product(vi, f, s);
     }
 };
 

@@ -441,26 +441,20 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
             }
             const double q = quarter_sqrt_area(j);
             const double root = (j == 1) ? A1 * d.lambda[n] : 0.0;
-            rd.a = g0;
-            rd.b = g1;
-            rd.c = g2;
-            rd.d = q;
-            rd.e = root;
-            // mixed forms: xi = 4^(J-j) eta, scale factors folded in (RecF)
+            // xi = 4^(J-j) eta, scale factors folded in (RecD, RecF)
             const double sc = ldexp(q, -2 * (J - j - 1));
-            if (single) {
-                rf.a = static_cast<float>(((g0 + g1) + g2) * sc);
-                rf.b = 0.0f;
-                rf.c = 0.0f;
-            } else {
-                rf.a = static_cast<float>(g0 * sc);
-                rf.b = static_cast<float>(g1 * sc);
-                rf.c = static_cast<float>(g2 * sc);
-            }
+            rd.a = single ? ((g0 + g1) + g2) * sc : g0 * sc;
+            rd.b = single ? 0.0 : g1 * sc;
+            rd.c = single ? 0.0 : g2 * sc;
+            rd.d = 0.0;
+            rd.e = ldexp(root, -2 * (J - 1));
+            rf.a = static_cast<float>(rd.a);
+            rf.b = static_cast<float>(rd.b);
+            rf.c = static_cast<float>(rd.c);
             rf.d = 0.0f;
             rf.e = 0.0f;
             rf.f = 0.0f;
-            rf.g = static_cast<float>(ldexp(root, -2 * (J - 1)));
+            rf.g = static_cast<float>(rd.e);
         }
         d.recd[post] = rd;
         d.recf[post] = rf;
@@ -512,7 +506,7 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
         wd.a = rd.a;
         wd.b = rd.b;
         wd.c = rd.c;
-        wd.d = wgt;
+        wd.d = ldexp(wgt, -2 * (J - j));   // weight of xi = 4^(J-j) eta
         wd.e = 0.0;
         wf.meta = wmeta;
         // internal nodes: stack rows of the node's own xi sum and its parent's
@@ -522,7 +516,7 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
         wf.d = leaf ? rf.d : 0.f;
         wf.e = leaf ? rf.e : 0.f;
         wf.f = leaf ? rf.f : 0.f;
-        wf.g = static_cast<float>(ldexp(wgt, -2 * (J - j)));   // weight of xi = 4^(J-j) eta
+        wf.g = static_cast<float>(wd.d);
         if (!leaf) {
             wd.a = wd.b = wd.c = 0.0;
         }

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(NT) k_wavelet_fp64(const Rec* __restrict__ rec
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 b.u[k] = U[k]; b.v[k] = V[k]; b.w[k] = W[k]; b.vr[k] = 0.0; b.vi[k] = 0.0;
-                b.sr[k] = 0.0; b.si[k] = 0.0; b.xr[k] = 0.0; b.xi[k] = 0.0;
+                b.sr[k] = 0.0; b.si[k] = 0.0;
             }
             b.stk = stk;
             b.J = J;
@@ -324,7 +324,7 @@ int stack_rows(int mode, int which, int J)
     if (which == WT_SUM_EQ16) return 0;
     if (mode == WT_FP64_DF) return J > 3 ? J - 2 : 1;   // regrouped (Eq. 16 returned 0 above)
     if (which == WT_SUM_EQ17_REGROUPED) {
-        if (mode == WT_FP64) return J > 3 ? 2 * (J - 2) : 2;
+        if (mode == WT_FP64) return J > 3 ? J - 2 : 1;
         return J > 4 ? J - 3 : 1;
     }
     return J > 1 ? 4 * (J - 1) : 4;

@@ -123,9 +123,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 __device__ __forceinline__ void df_product(F2 x, F2 y, float& p, float& t)
 {
     p = __fmul_rn(x.hi, y.hi);
-    const float e = __fmaf_rn(x.hi, y.hi, -p);
-    const float c = __fmaf_rn(x.hi, y.lo, __fmul_rn(x.lo, y.hi));
-    t = __fadd_rn(e, c);
+    t = __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, __fmaf_rn(x.hi, y.hi, -p)));
 }
 
 // Phase in turns of B.(s - P) = u*su + v*sv + w*sw1 modulo 1, returned as
@@ -182,32 +180,34 @@ __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, f
 
 // ---- float64 sin/cos of 2 pi t (t in turns, |t| < 2^40) ---------------------
 // Table-driven reduction (the table-lookup method of P. T. P. Tang, ACM TOMS
-// 15(2), 1989): k = rint(256 t), f = t - k/256 (exact, |f| <= 1/512), and
-// exp(i 2 pi t) = exp(i 2 pi (k mod 256)/256) exp(i 2 pi f). The table holds
-// the first factor correctly rounded (gen_sincos_table.py, entries for
-// k = -128 .. 128, of which 0 .. 255 modulo 256 are used); the second comes
-// from the Taylor series of sin (to x^7) and cos (to x^6) at x = 2 pi f,
-// |x| <= 0.0123, whose truncation errors (< 2e-20 and < 8e-21) are far below
-// float64 rounding. No separate reduction of t by its nearest integer is
-// needed: k mod 256 absorbs the whole turns.
-static __device__ const double2 kSinCos256[257] =
+// 15(2), 1989): k = rint(1024 t), f = t - k/1024 (exact, |f| <= 1/2048), and
+// exp(i 2 pi t) = exp(i 2 pi (k mod 1024)/1024) exp(i 2 pi f). The table holds
+// the first factor correctly rounded (gen_sincos_table.py); the second comes
+// from the Taylor series of sin (to x^5) and cos (to x^4) at x = 2 pi f, |x| <=
+// 0.0031, as polynomials in f: their truncation errors (< 6e-22 and < 2e-18)
+// are far below float64 rounding. Adding 1.5 2^42 rounds t to a multiple of
+// 2^-10 and leaves k's low bits at the bottom of the sum's word, so there is
+// neither a conversion nor a separate reduction of t by its nearest integer.
+// 13 operations of the float64 pipe, which bounds every kernel that calls it
+// (256 entries, with rint, a conversion to integer and one more term each: 18
+// and two conversions).
+static __device__ const double2 kSinCos1024[1024] =
 #include "sincos_table.inc"
     ;
 
 __device__ __forceinline__ void sincos_turns_f64(double t, double& s, double& c)
 {
-    const double k = rint(t * 256.0);
-    const double f = fma(k, -0.00390625, t);                       // t - k/256, exact
-    const double x = f * 6.283185307179586476925286766559;          // 2 pi f
-    const double x2 = x * x;
-    const double ps = fma(x2, fma(x2, -1.9841269841269841e-4, 8.3333333333333333e-3), -1.6666666666666667e-1);
-    const double sx = fma(x * x2, ps, x);
-    const double pc = fma(x2, fma(x2, fma(x2, -1.3888888888888889e-3, 4.1666666666666667e-2), -0.5), 1.0);
-    // entry j of the table is k = j - 128; k mod 256 in 0 .. 255 -> j = 128 + (k mod 256) - 256 * (k mod 256 >= 128)
-    const int km = static_cast<int>(static_cast<long long>(k) & 255);
-    const double2 tk = __ldg(&kSinCos256[(km < 128) ? km + 128 : km - 128]);
-    c = fma(tk.x, pc, -tk.y * sx);
-    s = fma(tk.y, pc, tk.x * sx);
+    constexpr double kMagic = 6597069766656.0;                      // 1.5 * 2^42
+    const double m = __dadd_rn(t, kMagic);
+    const double f = t - __dsub_rn(m, kMagic);                      // t - k/1024, exact
+    const double2 e = __ldg(&kSinCos1024[__double2loint(m) & 1023]);
+    const double f2 = f * f;
+    // sin 2 pi f = f (2 pi - (2 pi)^3/3! f^2 + (2 pi)^5/5! f^4)
+    const double sx = f * fma(f2, fma(f2, 81.60524927607505, -41.34170224039976), 6.283185307179586);
+    // cos 2 pi f - 1 = f^2 (-(2 pi)^2/2! + (2 pi)^4/4! f^2)
+    const double cm = f2 * fma(f2, 64.93939402266829, -19.739208802178716);
+    c = fma(e.x, cm, fma(-e.y, sx, e.x));
+    s = fma(e.y, cm, fma(e.x, sx, e.y));
 }
 
 // sin and cos of 2 pi (th + tl) from the special-function unit (the fast
@@ -531,10 +531,10 @@ __host__ __device__ __forceinline__ uint32_t rec_level(uint32_t meta) { return (
 
 // float64 record (48 bytes).
 //   leaf:     a, b, c = s_u, s_v, s_w - 1 (pixel centre, uvw frame); d = Phi
-//   internal: a, b, c = gamma^0, gamma^1, gamma^2 -- for a single-child node
-//             each multiplied by that child's sign in the Hadamard row
-//             (exact), so that gamma^m sigma^m = a_m (q eta_c);
-//             d = q = sqrt(A_j) / 4; e = A_1 lambda_1 at level 1, else 0
+//   internal: a, b, c = gamma^m q_j 4^-(J-j-1) (m = 0, 1, 2), for xi = 4^(J-j)
+//             eta as in RecF; for a single-child node a = the sum of the three,
+//             each with that child's Hadamard sign, and b = c = 0; d = 0;
+//             e = A_1 lambda_1 4^-(J-1) at level 1, else 0
 struct RecD {
     uint32_t meta;
     uint32_t pad;
@@ -542,8 +542,7 @@ struct RecD {
 };
 static_assert(sizeof(RecD) == 48, "RecD layout");
 
-// float32 record of the mixed form (32 bytes). The mixed predictors carry,
-// per node, xi_j = 4^(J-j) eta_j: the plain sum of the children's xi (a
+// float32 record of the mixed form (32 bytes). The predictors carry, per node, xi_j = 4^(J-j) eta_j: the plain sum of the children's xi (a
 // leaf's xi is its eta), so the 1/4 of Eq. 9 disappears, and the factors
 // q_j = sqrt(A_j)/4 and 4^-(J-j-1) that turn the children's xi into
 // sigma^m are folded into gamma^m here, in float64, rounded once.
@@ -586,7 +585,8 @@ constexpr uint32_t kRwGroup = 1u << 12;
 constexpr int kRwGroupShift = 13;
 constexpr int kRecChunkW = 128;   // records per staging buffer of the regrouped float32 form
 
-// float64 (48 bytes): a, b, c = leaf pixel centre (s_u, s_v, s_w - 1); d = w.
+// float64 (48 bytes): a, b, c = leaf pixel centre (s_u, s_v, s_w - 1);
+// d = w_n 4^-(J-j), the weight of xi = 4^(J-j) eta.
 struct RecWD {
     uint32_t meta;
     uint32_t pad;
