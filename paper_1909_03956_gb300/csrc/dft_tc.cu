@@ -61,8 +61,8 @@ namespace wt {
 
 // dft.cu: the exact pass of the mixed direct sum over 128-visibility tiles
 // marked by mark_deferred.
-int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, const double* uvw, int64_t n_vis,
-                       float2* vis, int sign, int* status, cudaStream_t s);
+int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, const TermParts& tp, const double* uvw,
+                       int64_t n_vis, float2* vis, int sign, int* status, cudaStream_t s);
 
 namespace {
 
@@ -274,10 +274,13 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 // memory and leaves.
 constexpr int kTcThreads = 160;
 
-template <int kTcTiles>
+// CUT: the terms are cut into parts on grid.y (the uncut kernel is kept free
+// of the parts' bookkeeping, which cost it 4 %).
+template <int kTcTiles, bool CUT>
 __global__ void __launch_bounds__(kTcThreads) k_dft_tc(const unsigned char* __restrict__ bsl,
                                                       const float* __restrict__ bfl, int64_t n_chunks,
-                                                      int64_t n_stages, const int64_t* __restrict__ n_dev,
+                                                      int64_t n_stages, int64_t part_stages,
+                                                      const int64_t* __restrict__ n_dev,
                                                       const uint32_t* __restrict__ bound,
                                                       const double* __restrict__ uvw, int64_t n_vis,
                                                       float2* __restrict__ vis, float sgn, int* status)
@@ -290,6 +293,18 @@ __global__ void __launch_bounds__(kTcThreads) k_dft_tc(const unsigned char* __re
         const int64_t nc = nd > 0 ? (nd + kTcNC - 1) / kTcNC : 0;
         if (nc < n_chunks) n_chunks = nc;
         n_stages = (n_chunks + kTcG - 1) / kTcG;
+    }
+    if constexpr (CUT) {   // this part's stages: from .. from + part_stages
+        const int64_t from = static_cast<int64_t>(blockIdx.y) * part_stages;
+        bsl += from * kTcStageBytes;
+        bfl += from * kTcStageComps;
+        vis += blockIdx.y * n_vis;
+        n_stages = max(n_stages - from, int64_t(0));
+        n_chunks = max(n_chunks - from * kTcG, int64_t(0));
+        if (blockIdx.y + 1 < gridDim.y) {   // the last part takes the rest
+            n_stages = min(n_stages, part_stages);
+            n_chunks = min(n_chunks, part_stages * kTcG);
+        }
     }
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[2], bar_empty[2], bar_ld[2], bar_sdone[2];
@@ -533,10 +548,10 @@ namespace {
 
 template <int TILES>
 int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks, int64_t stages,
-                    const int64_t* n_dev, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
+                    const TermParts& tp, const int64_t* n_dev, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
                     int sign, int* status, cudaStream_t s, const char* fn)
 {
-    auto kernel = k_dft_tc<TILES>;
+    auto kernel = tp.parts > 1 ? k_dft_tc<TILES, true> : k_dft_tc<TILES, false>;
     // no more CTAs per SM than their tensor memory allows (a CTA beyond
     // that would wait in tcgen05.alloc)
     const size_t need = 1024 + TILES * kTcRows * 128 + 2 * kTcStageBytes + 2 * kTcStageComps * 4;
@@ -552,8 +567,9 @@ int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks
     const int64_t cta_vis = static_cast<int64_t>(kTcRows) * TILES;
     const int64_t tiles = (n_vis + cta_vis - 1) / cta_vis;
     if (tiles > 0x7fffffff) return set_error(WT_ERR_RANGE, "%s: too many visibilities for one launch", fn);
-    kernel<<<static_cast<unsigned>(tiles), kTcThreads, smem, s>>>(bsl, bfl, n_chunks, stages, n_dev, bound, uvw, n_vis,
-                                                                  vis, static_cast<float>(sign), status);
+    kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(tp.parts)), kTcThreads, smem, s>>>(
+        bsl, bfl, n_chunks, stages, tp.per_part / kTcStageComps, n_dev, bound, uvw, n_vis, vis,
+        static_cast<float>(sign), status);
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;
 }
@@ -562,24 +578,32 @@ int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks
 // of `stages` stages, n_chunks chunks of it used (or those *n_dev items
 // need, when n_dev is given); chunks_hint, the chunks the host expects,
 // picks two tiles per CTA for a few hundred terms.
-int tc_main_launch(const unsigned char* bsl, const float* bfl, int64_t n_chunks, int64_t stages, const int64_t* n_dev,
-                   int64_t chunks_hint, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
+int tc_main_launch(const unsigned char* bsl, const float* bfl, int64_t n_chunks, int64_t stages, const TermParts& tp,
+                   const int64_t* n_dev, int64_t chunks_hint, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
                    int sign, int* status, cudaStream_t s, const char* fn)
 {
     if (chunks_hint <= kTcTwoTileMaxChunks)
-        return tc_launch_tiles<2>(bsl, bfl, n_chunks, stages, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
-    return tc_launch_tiles<1>(bsl, bfl, n_chunks, stages, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
+        return tc_launch_tiles<2>(bsl, bfl, n_chunks, stages, tp, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
+    return tc_launch_tiles<1>(bsl, bfl, n_chunks, stages, tp, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
 }
 
 }  // namespace
+
+// Tiles (CTAs per part) of the launch tc_main_launch makes.
+int64_t dft_tc_tiles(int64_t n_vis, int64_t n_comp)
+{
+    const int64_t cta_vis = (n_comp + kTcNC - 1) / kTcNC <= kTcTwoTileMaxChunks ? 2 * kTcRows : kTcRows;
+    return (n_vis + cta_vis - 1) / cta_vis;
+}
+static_assert(kTcStageComps == kPartTerms, "a part is whole stages");
 
 // The tensor-core direct sum on components already packed (recs, bound:
 // k_pack_components in the mixed layout) with `tc` (dft_tc_scratch_bytes,
 // 256-byte aligned) for the slices; then the exact pass over the tiles left
 // to it.
 int dft_tc_launch(const double* l, const double* m, const double* flux, int64_t n_comp, const void* recs,
-                  const uint32_t* bound, void* tc, const double* uvw, int64_t n_vis, float2* vis, int sign,
-                  int* status, cudaStream_t s)
+                  const uint32_t* bound, void* tc, const TermParts& tp, const double* uvw, int64_t n_vis, float2* vis,
+                  int sign, int* status, cudaStream_t s)
 {
     if (n_vis == 0) return WT_OK;
     const int64_t stages = (n_comp + kTcStageComps - 1) / kTcStageComps;
@@ -593,10 +617,10 @@ int dft_tc_launch(const double* l, const double* m, const double* flux, int64_t 
         WT_CUDA_TRY(cudaGetLastError());
     }
     const int64_t chunks = (n_comp + kTcNC - 1) / kTcNC;
-    int rc = tc_main_launch(bsl, bfl, chunks, stages, nullptr, chunks, bound, uvw, n_vis, vis, sign, status, s,
+    int rc = tc_main_launch(bsl, bfl, chunks, stages, tp, nullptr, chunks, bound, uvw, n_vis, vis, sign, status, s,
                             "dft_predict_vis");
     if (rc) return rc;
-    return dft_exact_pass_128(recs, bound, n_comp, uvw, n_vis, vis, sign, status, s);
+    return dft_exact_pass_128(recs, bound, n_comp, tp, uvw, n_vis, vis, sign, status, s);
 }
 
 // Eq. 16 in the tensor-core form over leaf records (RecF, at most cap of
@@ -613,7 +637,11 @@ int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t
     const int64_t stages = (cap + kTcStageComps - 1) / kTcStageComps;
     const int64_t cap_pad = stages * kTcStageComps;
     const size_t exact_bytes = static_cast<size_t>(cap_pad > 0 ? cap_pad : 1) * sizeof(CompF);
-    const size_t bytes = ((exact_bytes + 255) / 256) * 256 + dft_tc_scratch_bytes(cap_pad);
+    const size_t base = ((exact_bytes + 255) / 256) * 256 + (dft_tc_scratch_bytes(cap_pad) + 255) / 256 * 256;
+    // few visibilities: the terms cut by the count the host expects (the last
+    // part takes whatever more there is)
+    const TermParts tp = term_parts(dft_tc_tiles(n_vis, n_hint), n_hint, 4);
+    const size_t bytes = base + (tp.parts > 1 ? sizeof(float2) * static_cast<size_t>(tp.parts * n_vis) : 0);
     unsigned char* scratch = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, s);
     if (e != cudaSuccess) {
@@ -622,6 +650,7 @@ int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t
                          cudaGetErrorString(e));
     }
     CompF* exact = reinterpret_cast<CompF*>(scratch);
+    float2* out = tp.parts > 1 ? reinterpret_cast<float2*>(scratch + base) : vis;
     unsigned char* bsl = scratch + ((exact_bytes + 255) / 256) * 256;
     float* bfl = reinterpret_cast<float*>(bsl + stages * kTcStageBytes);
     int rc = WT_OK;
@@ -633,10 +662,11 @@ int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t
     }
     const uint32_t* bound = reinterpret_cast<const uint32_t*>(hdr->smax);   // device address of the bounds
     if (rc == WT_OK)
-        rc = tc_main_launch(bsl, bfl, stages * kTcG, stages, &hdr->n_leaves, (n_hint + kTcNC - 1) / kTcNC, bound, uvw,
-                            n_vis, vis, sign, status, s, fn);
+        rc = tc_main_launch(bsl, bfl, stages * kTcG, stages, tp, &hdr->n_leaves, (n_hint + kTcNC - 1) / kTcNC, bound,
+                            uvw, n_vis, out, sign, status, s, fn);
     // the exact pass over every capacity record (those beyond the count are zero)
-    if (rc == WT_OK) rc = dft_exact_pass_128(exact, bound, cap_pad, uvw, n_vis, vis, sign, status, s);
+    if (rc == WT_OK) rc = dft_exact_pass_128(exact, bound, cap_pad, tp, uvw, n_vis, out, sign, status, s);
+    if (rc == WT_OK && tp.parts > 1) rc = sum_parts(out, tp, n_vis, vis, false, s);
     cudaError_t ef = cudaFreeAsync(scratch, s);
     if (rc != WT_OK) return rc;
     if (ef != cudaSuccess) return cuda_error(ef, "cudaFreeAsync");

@@ -482,6 +482,10 @@ __device__ __forceinline__ void sincos_mixed2(float2 h, float2 tl, float2& e0, f
 // and each partial enters the Kahan sum once.
 constexpr int kSumBlock = 8;
 
+// A part of a direct sum cut over its terms is a multiple of this many (a
+// stage of the tensor-core form's operand).
+constexpr int kPartTerms = 128;
+
 // Kahan-compensated sum of pairs (each element as kahan_add).
 __device__ __forceinline__ void kahan_add2(float2& sum, float2& comp, float2 x)
 {
@@ -731,7 +735,13 @@ inline size_t vis_align(int mode) { return (mode == WT_FP64 || mode == WT_FP64_D
 // dft_tc.cu: Eq. 16 over leaf records with the phase on the tensor cores
 int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t n_hint, const double* uvw,
                    int64_t n_vis, float2* vis, int sign, int* status, cudaStream_t s, const char* fn);
-// dft.cu
+// dft.cu: a direct sum over few visibilities, its terms cut into parts
+struct TermParts {
+    int64_t parts;        // grid.y of the sum's kernels (1: not cut)
+    int64_t per_part;     // terms per part, a multiple of kPartTerms
+};
+TermParts term_parts(int64_t tiles, int64_t n_terms, int fill);
+int sum_parts(const void* partial, const TermParts& tp, int64_t n_vis, void* vis, bool c128, cudaStream_t s);
 int predict_dft(const double* l, const double* m, const double* flux, int64_t n_comp, const double* uvw,
                 int64_t n_vis, void* vis, int mode, int sign, cudaStream_t s);
 // subtract.cu
