@@ -212,6 +212,52 @@ static int check_tree(wt_tree t, const char* fn)
 
 namespace {
 
+// Pinned header copies of freed trees, kept for the next ones (allocating and
+// freeing pinned memory, with a second wait for the stream, took 340 of the 500
+// us of a small major cycle): at most kKeptHeaders, each of the context it was
+// allocated in; one of a context that is gone is dropped with it. A header is
+// given back only after its tree's stream has been waited for, so no copy into
+// it is pending.
+constexpr size_t kKeptHeaders = 32;
+struct KeptHeader {
+    TreeHeader* p;
+    uint64_t ctx;
+};
+std::mutex g_hdr_mu;
+std::vector<KeptHeader> g_hdrs;
+
+TreeHeader* take_header(cudaError_t* e)
+{
+    const uint64_t ctx = wt::current_context_id();
+    {
+        std::lock_guard<std::mutex> lk(g_hdr_mu);
+        for (size_t i = g_hdrs.size(); i-- > 0;)
+            if (g_hdrs[i].ctx == ctx) {
+                TreeHeader* p = g_hdrs[i].p;
+                g_hdrs.erase(g_hdrs.begin() + static_cast<std::ptrdiff_t>(i));
+                return p;
+            }
+    }
+    TreeHeader* p = nullptr;
+    *e = cudaMallocHost(reinterpret_cast<void**>(&p), sizeof(TreeHeader));
+    return *e == cudaSuccess ? p : nullptr;
+}
+
+void give_back_header(TreeHeader* p)
+{
+    if (!p) return;
+    const uint64_t ctx = wt::current_context_id();
+    if (ctx != 0) {
+        std::lock_guard<std::mutex> lk(g_hdr_mu);
+        if (g_hdrs.size() == kKeptHeaders && g_hdrs.front().ctx != ctx) g_hdrs.erase(g_hdrs.begin());
+        if (g_hdrs.size() < kKeptHeaders) {
+            g_hdrs.push_back(KeptHeader{p, ctx});
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
 // A new tree handle built from `src` (checked by the caller).
 int new_tree(const char* fn, const wt::KeySource& src, const double* flux, int64_t n_comp, double ra0, double dec0,
              int J, wt_tree* out, void* stream)
@@ -229,8 +275,9 @@ int new_tree(const char* fn, const wt::KeySource& src, const double* flux, int64
     t->dec0 = dec0;
     t->n_comp = n_comp;
     t->stream = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&t->host_hdr), sizeof(TreeHeader));
-    if (e != cudaSuccess) {
+    cudaError_t e = cudaSuccess;
+    t->host_hdr = take_header(&e);
+    if (!t->host_hdr) {
         t->magic = 0;
         delete t;
         return cuda_error(e, "cudaMallocHost");
@@ -238,8 +285,8 @@ int new_tree(const char* fn, const wt::KeySource& src, const double* flux, int64
     rc = wt::build_tree(src, flux, n_comp, ra0, dec0, J, t, t->stream);
     if (rc != WT_OK) {
         if (t->block) cudaFreeAsync(t->block, t->stream);
-        cudaStreamSynchronize(t->stream);
-        cudaFreeHost(t->host_hdr);
+        if (cudaStreamSynchronize(t->stream) == cudaSuccess) give_back_header(t->host_hdr);
+        else cudaFreeHost(t->host_hdr);
         t->magic = 0;
         delete t;
         return rc;
@@ -420,10 +467,10 @@ void wt_free_tree(wt_tree t)
     cudaGetDevice(&prev);
     if (prev != t->device) cudaSetDevice(t->device);
     wt::batch_forget_tree(t);
-    cudaStreamSynchronize(t->stream);
+    const bool quiet = cudaStreamSynchronize(t->stream) == cudaSuccess;
     if (t->block) cudaFreeAsync(t->block, t->stream);
-    cudaStreamSynchronize(t->stream);
-    if (t->host_hdr) cudaFreeHost(t->host_hdr);
+    if (quiet) give_back_header(t->host_hdr);
+    else if (t->host_hdr) cudaFreeHost(t->host_hdr);
     cudaGetLastError();
     if (prev >= 0 && prev != t->device) cudaSetDevice(prev);
     t->magic = 0;
