@@ -302,21 +302,22 @@ __device__ __forceinline__ void phase_turns_df2(const DF2& u, const DF2& v, cons
 
 // ---- phase with the heads on a common grid ----------------------------------
 // The error-free sums of phase_turns_df2 exist to add the three head
-// products without losing their low bits. When every head is first rounded
-// onto one common grid G = 2^(k-23), with k chosen per visibility so that
-// every product stays below 2^(k-1), the heads and their partial sums are
-// multiples of G below 2^(k+1): 24 significant bits at most, so plain
-// float32 additions are exact. A head is rounded onto the grid by one FMA
-// against the constant C = 1.5 * 2^k (the sum x y + C stays in C's binade,
-// where the spacing of floats is G) and recovered by one exact subtraction
-// (Sterbenz); its remainder x y - (x y)_G, below G/2, goes to the tail with
-// the cross terms. Per visibility and term this is 20 float32 operations
-// against 29 for the error-free sums, with the same phase accuracy: the
-// tail's roundings are of order 2^-24 G, the dropped x.lo y.lo below 2^-48
-// of the product. Valid while k <= kGridMaxK, which keeps |tail| <= 2 G
-// small enough for both sin/cos forms (sincos_turns_f32 then sees
-// |x| <= 0.84); larger phases take phase_turns_df2 (the caller decides).
-constexpr int kGridMinK = -8;    // finest grid used: 2^-31 turns
+// products without losing their low bits. Here they are added by FMAs onto
+// C = 1.5 * 2^k instead: with k chosen per visibility so that the heads'
+// magnitudes sum to less than 2^(k-1), every partial sum h_1 = C + x_1 y_1,
+// h_2 = h_1 + x_2 y_2, h_3 = h_2 + x_3 y_3 stays in C's binade, where floats
+// are spaced by G = 2^(k-23), so each FMA rounds its product onto that grid
+// and nothing else. Differences of partial sums are exact, and what a product
+// leaves behind, x_c y_c - (h_c - h_(c-1)), below G/2, comes from one more FMA
+// and joins the tail with the cross terms. C is a whole number, so h_3 is
+// reduced by its own nearest integer. Per visibility and term 18 float32
+// operations, against 29 for the error-free sums and 20 with each head rounded
+// and recovered by itself, with the same phase accuracy: the tail's roundings
+// are of order 2^-24 G, the dropped x.lo y.lo below 2^-48 of the product.
+// Valid while k <= kGridMaxK, which keeps |tail| <= 2 G small enough for both
+// sin/cos forms (sincos_turns_f32 then sees |x| <= 0.84); larger phases take
+// phase_turns_df2 (the caller decides).
+constexpr int kGridMinK = 1;     // C a whole number; finest grid 2^-22 turns
 constexpr int kGridMaxK = 15;    // heads below 2^14 turns
 
 // C = 1.5 * 2^k for the smallest k >= kGridMinK with bound < 2^(k-1); also
@@ -332,14 +333,13 @@ __device__ __forceinline__ float grid_magic(float bound, int& kk)
     return __int_as_float(((kc + 127) << 23) | 0x400000);
 }
 
-// Head of x y on the grid of C, negated, and the tail, for both elements
-// (element-wise C): nq = -(x.hi y.hi rounded to the grid), exactly;
-// t = (x.hi y.hi + nq) + x.lo y.hi + x.hi y.lo, the first term exact.
-__device__ __forceinline__ void grid_product2n(const DF2& x, F2 y, float2 C, float2& nq, float2& t)
+// One coordinate, both elements: h1 = h0 + x.hi y.hi rounded onto the grid,
+// t = (x.hi y.hi - (h1 - h0)) + x.lo y.hi + x.hi y.lo, the first term exact.
+__device__ __forceinline__ void grid_step2(const DF2& x, F2 y, float2 h0, float2& h1, float2& t)
 {
     const float2 yh = bcast2(y.hi);
-    nq = sub2(C, fma2(x.hi, yh, C));
-    t = fma2(x.hi, bcast2(y.lo), fma2(x.lo, yh, fma2(x.hi, yh, nq)));
+    h1 = fma2(x.hi, yh, h0);
+    t = fma2(x.hi, bcast2(y.lo), fma2(x.lo, yh, fma2(x.hi, yh, sub2(h0, h1))));
 }
 
 // phase_turns_df2 on the grid of C (per element): returns h and tl with the
@@ -347,12 +347,11 @@ __device__ __forceinline__ void grid_product2n(const DF2& x, F2 y, float2 C, flo
 __device__ __forceinline__ void phase_turns_grid2(const DF2& u, const DF2& v, const DF2& w, F2 su, F2 sv, F2 sw1,
                                                   float2 C, float2& h, float2& tl)
 {
-    float2 q1, t1, q2, t2, q3, t3;
-    grid_product2n(u, su, C, q1, t1);
-    grid_product2n(v, sv, C, q2, t2);
-    grid_product2n(w, sw1, C, q3, t3);
-    const float2 b = add2(add2(q1, q2), q3);          // exact: multiples of the grid below 2^(k+1)
-    h = sub2(b, make_float2(rintf(b.x), rintf(b.y)));
+    float2 h1, h2, h3, t1, t2, t3;
+    grid_step2(u, su, C, h1, t1);
+    grid_step2(v, sv, h1, h2, t2);
+    grid_step2(w, sw1, h2, h3, t3);
+    h = sub2(make_float2(rintf(h3.x), rintf(h3.y)), h3);   // exact
     tl = add2(add2(t1, t2), t3);
 }
 
@@ -361,14 +360,13 @@ __device__ __forceinline__ void phase_turns_grid2(const DF2& u, const DF2& v, co
 __device__ __forceinline__ void phase_turns_grid(F2 u, F2 v, F2 w, F2 su, F2 sv, F2 sw1, float C, float& th,
                                                  float& tl)
 {
-    const float p1 = __fsub_rn(__fmaf_rn(u.hi, su.hi, C), C);
-    const float p2 = __fsub_rn(__fmaf_rn(v.hi, sv.hi, C), C);
-    const float p3 = __fsub_rn(__fmaf_rn(w.hi, sw1.hi, C), C);
-    const float t1 = __fmaf_rn(u.hi, su.lo, __fmaf_rn(u.lo, su.hi, __fmaf_rn(u.hi, su.hi, -p1)));
-    const float t2 = __fmaf_rn(v.hi, sv.lo, __fmaf_rn(v.lo, sv.hi, __fmaf_rn(v.hi, sv.hi, -p2)));
-    const float t3 = __fmaf_rn(w.hi, sw1.lo, __fmaf_rn(w.lo, sw1.hi, __fmaf_rn(w.hi, sw1.hi, -p3)));
-    const float b = __fadd_rn(__fadd_rn(p1, p2), p3);
-    th = __fsub_rn(b, rintf(b));
+    const float h1 = __fmaf_rn(u.hi, su.hi, C);
+    const float h2 = __fmaf_rn(v.hi, sv.hi, h1);
+    const float h3 = __fmaf_rn(w.hi, sw1.hi, h2);
+    const float t1 = __fmaf_rn(u.hi, su.lo, __fmaf_rn(u.lo, su.hi, __fmaf_rn(u.hi, su.hi, __fsub_rn(C, h1))));
+    const float t2 = __fmaf_rn(v.hi, sv.lo, __fmaf_rn(v.lo, sv.hi, __fmaf_rn(v.hi, sv.hi, __fsub_rn(h1, h2))));
+    const float t3 = __fmaf_rn(w.hi, sw1.lo, __fmaf_rn(w.lo, sw1.hi, __fmaf_rn(w.hi, sw1.hi, __fsub_rn(h2, h3))));
+    th = __fsub_rn(h3, rintf(h3));
     tl = __fadd_rn(__fadd_rn(t1, t2), t3);
 }
 
