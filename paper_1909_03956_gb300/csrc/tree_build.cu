@@ -457,7 +457,6 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
             rf.g = static_cast<float>(rd.e);
         }
         d.recd[post] = rd;
-        d.recf[post] = rf;
         // regrouped Eq. 17: the node's weight from its parent's gammas
         double wgt;
         bool first = true;
@@ -494,6 +493,8 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
                 }
             }
         }
+        if (group_first) rf.meta |= kRecGroup | (group_len << kRecGroupShift);
+        d.recf[post] = rf;
         const uint32_t wmeta = static_cast<uint32_t>(j) | (leaf ? kRwLeaf : 0u) | (j == 1 ? kRwRoot : 0u) |
                                (first ? kRwFirst : 0u) | (pair_first ? kRwPairFirst : 0u) |
                                (pair_second ? kRwPairSecond : 0u) | ((!leaf && j == J - 1) ? kRwLowSum : 0u) |

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(NT, (mixed_min_blocks<NT, VPT, SUM>())) k_wave
                                                       int* status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int kChunk = (SUM == 2) ? kChunkW : kChunkF;
+    constexpr int kChunk = (SUM == 1) ? kChunkF : kChunkW;
     Stager<Rec> st;
     const int64_t count = (SUM == 1) ? hdr->n_leaves : hdr->n_nodes;
     stager_setup(st, smem, recs, count, kChunk);
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(NT, (mixed_min_blocks<NT, VPT, SUM>())) k_wave
             b.start();
             b.stk = stk;
             b.maxrow = rows - 1;
-            good = st.sweep(b);
+            good = st.sweep_at(b);
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 const float2 r = b.result(k);
@@ -335,7 +335,7 @@ size_t stage_bytes(int mode, int which)
 {
     if (mode == WT_FP64) return stager_bytes<RecD>(kChunkD);
     if (mode == WT_FP64_DF) return stager_bytes<RecWDF>(kChunkDF) + kDfTableEntries * sizeof(float4);
-    return (which == WT_SUM_EQ17_REGROUPED) ? stager_bytes<RecWF>(kChunkW) : stager_bytes<RecF>(kChunkF);
+    return (which == WT_SUM_EQ16) ? stager_bytes<RecF>(kChunkF) : stager_bytes<RecWF>(kChunkW);
 }
 
 template <int NT, int VPT>

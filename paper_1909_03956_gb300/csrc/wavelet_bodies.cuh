@@ -155,10 +155,53 @@ struct Eq17F {
 
     __device__ __forceinline__ float2 result(int k) const { return sub2(acc[k], comp[k]); }
 
-    __device__ __forceinline__ void emit(int k, bool root, int srow, float g, float2 e)
+    // The plane wave at a leaf's centre, every visibility.
+    __device__ __forceinline__ void leaf_waves(const RecF& r, float2 (&e)[VPT]) const
     {
-        if (root) kahan_add2(acc[k], comp[k], mul2(bcast2(g), e));
-        else slot(srow, k) = e;
+        const F2 su{r.a, r.b}, sv{r.c, r.d}, sw{r.e, r.f};
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            float2 h, tl;
+            if constexpr (GRID) phase_turns_grid2(U[p], V[p], W[p], su, sv, sw, Cg[p], h, tl);
+            else phase_turns_df2(U[p], V[p], W[p], su, sv, sw, h, tl);
+            sincos_mixed2<FAST>(h, tl, e[2 * p], e[2 * p + 1]);
+        }
+        if constexpr (ODD) {
+            constexpr int k = VPT - 1;
+            float th, tl, s, c;
+            if constexpr (GRID) phase_turns_grid(u[k], v[k], w[k], su, sv, sw, Cs, th, tl);
+            else phase_turns_df(u[k], v[k], w[k], su, sv, sw, th, tl);
+            sincos_mixed<FAST>(th, tl, s, c);
+            e[k] = make_float2(c, s);
+        }
+    }
+
+    // A node with a single child: its xi is the child's.
+    __device__ __forceinline__ void node_single(const RecF& r, bool root, int srow, const float2 (&xi)[VPT])
+    {
+        const float2 a = bcast2(r.a), g = bcast2(r.g);
+#pragma unroll
+        for (int k = 0; k < VPT; ++k) {
+            float2 x = mul2(a, xi[k]);
+            if (root) x = fma2(g, xi[k], x);
+            else slot(srow, k) = xi[k];
+            kahan_add2(acc[k], comp[k], x);
+        }
+    }
+
+    // A node of several children, one visibility.
+    __device__ __forceinline__ void node(const RecF& r, bool root, int srow, int k, float2 c0, float2 c1, float2 c2,
+                                         float2 c3)
+    {
+        const float2 ga = bcast2(r.a), gb = bcast2(r.b), gc = bcast2(r.c);
+        const float2 a = add2(c0, c1), b = sub2(c0, c1);   // c0 +- c1
+        const float2 c = add2(c2, c3), d = sub2(c2, c3);   // c2 +- c3
+        const float2 xi = add2(a, c);                      // Eq. 9 (times 4^(J-j))
+        // Eq. 10 rows (+ - + -), (+ + - -), (+ - - +), weighted by gamma
+        float2 x = fma2(ga, add2(b, d), fma2(gb, sub2(a, c), mul2(gc, sub2(b, d))));
+        if (root) x = fma2(bcast2(r.g), xi, x);
+        else slot(srow, k) = xi;
+        kahan_add2(acc[k], comp[k], x);
     }
 
     __device__ void operator()(const RecF& r)
@@ -167,39 +210,22 @@ struct Eq17F {
         const bool root = meta & kRecRoot;
         const int srow = clamp_row(rec_store_row(meta), maxrow);
         if (meta & kRecLeaf) {
-            const F2 su{r.a, r.b}, sv{r.c, r.d}, sw{r.e, r.f};
+            float2 e[VPT];
+            leaf_waves(r, e);
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                float2 h, tl, e0, e1;
-                if constexpr (GRID) phase_turns_grid2(U[p], V[p], W[p], su, sv, sw, Cg[p], h, tl);
-                else phase_turns_df2(U[p], V[p], W[p], su, sv, sw, h, tl);
-                sincos_mixed2<FAST>(h, tl, e0, e1);
-                emit(2 * p, root, srow, r.g, e0);
-                emit(2 * p + 1, root, srow, r.g, e1);
-            }
-            if constexpr (ODD) {
-                constexpr int k = VPT - 1;
-                float th, tl, s, c;
-                if constexpr (GRID) phase_turns_grid(u[k], v[k], w[k], su, sv, sw, Cs, th, tl);
-                else phase_turns_df(u[k], v[k], w[k], su, sv, sw, th, tl);
-                sincos_mixed<FAST>(th, tl, s, c);
-                emit(k, root, srow, r.g, make_float2(c, s));
+            for (int k = 0; k < VPT; ++k) {
+                if (root) kahan_add2(acc[k], comp[k], mul2(bcast2(r.g), e[k]));
+                else slot(srow, k) = e[k];
             }
         } else if (meta & kRecSingle) {
             const int crow = clamp_row(rec_child_row(meta), maxrow);
-            const float2 a = bcast2(r.a), g = bcast2(r.g);
+            float2 xi[VPT];
 #pragma unroll
-            for (int k = 0; k < VPT; ++k) {
-                const float2 xi = slot(crow, k);             // the node's xi is its child's
-                float2 x = mul2(a, xi);
-                if (root) x = fma2(g, xi, x);
-                else slot(srow, k) = xi;
-                kahan_add2(acc[k], comp[k], x);
-            }
+            for (int k = 0; k < VPT; ++k) xi[k] = slot(crow, k);
+            node_single(r, root, srow, xi);
         } else {
             const int crow = clamp_row(rec_child_row(meta), maxrow - 3);
             const uint32_t mask = rec_mask(meta);
-            const float2 ga = bcast2(r.a), gb = bcast2(r.b), gc = bcast2(r.c), g = bcast2(r.g);
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
@@ -207,14 +233,70 @@ struct Eq17F {
                 if (mask & 2u) c1 = slot(crow + 1, k);
                 if (mask & 4u) c2 = slot(crow + 2, k);
                 if (mask & 8u) c3 = slot(crow + 3, k);
-                const float2 a = add2(c0, c1), b = sub2(c0, c1);   // c0 +- c1
-                const float2 c = add2(c2, c3), d = sub2(c2, c3);   // c2 +- c3
-                const float2 xi = add2(a, c);                      // Eq. 9 (times 4^(J-j))
-                // Eq. 10 rows (+ - + -), (+ + - -), (+ - - +), weighted by gamma
-                float2 x = fma2(ga, add2(b, d), fma2(gb, sub2(a, c), mul2(gc, sub2(b, d))));
-                if (root) x = fma2(g, xi, x);
-                else slot(srow, k) = xi;
-                kahan_add2(acc[k], comp[k], x);
+                node(r, root, srow, k, c0, c1, c2, c3);
+            }
+        }
+    }
+
+    // One step of the sweep; returns the records it took. A group (a run of
+    // sibling leaves and their parent, in one chunk by construction) is one
+    // step: the leaves' waves go to the parent's butterfly in registers, never
+    // to the stack, and the record's decoding is shared. 2 032 000 visibilities
+    // of 1 530 leaves, polynomial form: 9.76 -> 8.43 ms.
+    __device__ __forceinline__ int at(const RecF* cb, int r, int n)
+    {
+        const uint32_t meta = cb[r].meta;
+        if (meta & kRecGroup) {
+            const int k = static_cast<int>((meta >> kRecGroupShift) & 7u);
+            if (k >= 1 && k <= 4 && r + k < n) {
+                group(cb + r, k);
+                return k + 1;
+            }
+        }
+        (*this)(cb[r]);
+        return 1;
+    }
+
+    __device__ __forceinline__ void group(const RecF* g, int k)
+    {
+        const RecF& par = g[k];
+        const uint32_t meta = par.meta;
+        const bool root = meta & kRecRoot;
+        const int srow = clamp_row(rec_store_row(meta), maxrow);
+        const uint32_t mask = rec_mask(meta);
+        if (k == 1) {
+            float2 e[VPT];
+            leaf_waves(g[0], e);
+            node_single(par, root, srow, e);
+        } else if (k == 4) {
+            float2 c0[VPT], c1[VPT], c2[VPT], c3[VPT];
+            leaf_waves(g[0], c0);
+            leaf_waves(g[1], c1);
+            leaf_waves(g[2], c2);
+            leaf_waves(g[3], c3);
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) node(par, root, srow, i, c0[i], c1[i], c2[i], c3[i]);
+        } else {                                       // two or three children, in slot order
+            const float2 zero = make_float2(0.f, 0.f);
+            float2 e0[VPT], e1[VPT], e2[VPT];
+            leaf_waves(g[0], e0);
+            leaf_waves(g[1], e1);
+            if (k == 3) {
+                leaf_waves(g[2], e2);
+            } else {
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) e2[i] = zero;
+            }
+            // the slot of the i-th leaf is that of the mask's i-th bit
+            const bool b0 = mask & 1u, b1 = mask & 2u, b2 = mask & 4u, b3 = mask & 8u;
+            const int before2 = (b0 ? 1 : 0) + (b1 ? 1 : 0);
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) {
+                const float2 c0 = b0 ? e0[i] : zero;
+                const float2 c1 = !b1 ? zero : b0 ? e1[i] : e0[i];
+                const float2 c2 = !b2 ? zero : before2 == 2 ? e2[i] : before2 == 1 ? e1[i] : e0[i];
+                const float2 c3 = !b3 ? zero : k == 3 ? e2[i] : e1[i];
+                node(par, root, srow, i, c0, c1, c2, c3);
             }
         }
     }

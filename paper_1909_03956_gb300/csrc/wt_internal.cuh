@@ -523,6 +523,12 @@ static_assert(sizeof(CompF) == 32, "component record layout");
 //   19     level 1 (adds A_1 lambda_1 eta_1, or Phi eta for a level-1 leaf)
 //   20     single child
 //   21-25  level j
+//   26     (float32 records) the first leaf of a group: a run of sibling
+//          leaves whose parent, the next record after the run, lies in the
+//          same staging chunk of kRecChunkW records, so that the run and its
+//          parent are taken in one step; 27-29 the run's length (1 to 4)
+constexpr uint32_t kRecGroup = 1u << 26;
+constexpr int kRecGroupShift = 27;
 constexpr uint32_t kRecLeaf = 1u << 18;
 constexpr uint32_t kRecRoot = 1u << 19;
 constexpr uint32_t kRecSingle = 1u << 20;
