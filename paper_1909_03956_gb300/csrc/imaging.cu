@@ -26,10 +26,10 @@
 // fl(I - fl(f B)). Two schedules, identical results:
 //   persistent  the whole minor cycle in one cooperative launch: each CTA
 //               keeps its rows of the image in shared memory for every
-//               iteration, subtracts the pending component there (the beam
-//               is read from global memory and stays in L2), and joins a
-//               grid-wide maximum of the CTAs' (value, pixel) keys once per
-//               iteration, which also serves as the iteration's barrier;
+//               iteration; the CTAs meet once for a batch of components,
+//               each found among the largest pixels they posted there, and
+//               subtract the batch from their rows (the beam is read from
+//               global memory and stays in L2);
 //   per launch  one launch per iteration when the rows do not fit in shared
 //               memory: every CTA subtracts the previous component over its
 //               pixels and finds its largest updated value; a 64-bit
@@ -651,40 +651,48 @@ __global__ void k_hogbom_reset(HogbomState* st, int* n_comp)
 }
 
 // ---------------------------------------------------------------- persistent Hogbom
-constexpr int kHogThreads = 512;
-constexpr int kMaxHogCtas = 1024;   // grid cap of the persistent clean
-constexpr int kRowsAhead = 4;   // rows whose beam values a thread loads before using them
-// Polls of the grid barrier before a CTA gives up: each poll is an L2 load
-// and a 40 ns sleep, so the limit is of the order of a second (a healthy
+// Several components per synchronisation. Finding one component over the whole
+// grid costs a grid-wide exchange (3 us, half an iteration at 2048 x 2048 and
+// nearly all of it below 1024 x 1024), but the next components are almost always among
+// a few hundred pixels that are already known to be the largest. So after a
+// scan of its rows each CTA posts its kTop largest pixels and a bound on all
+// its others, the CTAs meet once, and then every CTA plays the following
+// iterations through on the posted pixels alone: their values are updated with
+// the same operations in the same order as in the image, and the bound grows
+// by what a subtraction can at most add to a pixel (|f| times the beam's most
+// negative value, rounded up). While the largest posted value stays above the
+// bound it is the image's largest, and the next component; once it does not,
+// or after kBatch components, the CTAs subtract the batch from their rows, in
+// order, and scan again. Components, fluxes and image are those of the one-by-
+// one clean bit for bit; the image's rows are read and written once per batch.
+constexpr int kHogThreads = 1024;
+constexpr int kHogWarps = kHogThreads / 32;
+constexpr int kMaxHogCtas = 256;   // grid cap of the persistent clean
+constexpr int kTop = 8;            // pixels a CTA posts
+constexpr int kWarpTop = 4;        // of them at most from one warp
+constexpr int kBatch = 64;         // components per synchronisation at most
+constexpr int kPerThread = kMaxHogCtas * kTop / kHogThreads;   // posted pixels a thread plays
+// Polls of the grid barrier before a CTA gives up: each poll is a round trip
+// to L2 and a 40 ns sleep, so the limit is of the order of a second (a healthy
 // barrier completes within microseconds).
 constexpr uint32_t kGridSpinLimit = 1u << 20;
 
-// Grid-wide maximum of one 64-bit key per CTA, once per iteration, in three
-// rotating slots: iteration i uses slot i % 3.
+// The CTAs' meeting place. Posts alternate between two sets: a CTA writes set
+// e + 2 over e only after the meeting e + 1, which everyone joins after
+// reading all of e.
 struct HogSync {
-    unsigned int count[3];        // CTAs arrived
-    int abort;                    // 1 once a CTA gave up waiting
-    unsigned long long key[3];    // running maximum of the arrived CTAs' keys
-    unsigned long long result[3]; // the maximum, published by the last CTA to arrive (0: not yet)
+    unsigned int count;                              // arrivals, over all meetings
+    int abort;                                       // 1 once a CTA gave up waiting
+    float beam[kMaxHogCtas][2];                      // largest -psf and psf of a CTA's share
+    float bound[2][kMaxHogCtas];
+    unsigned long long key[2][kMaxHogCtas][kTop];
 };
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p)
+__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p)
 {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-
-__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned int atom_add_acq_rel(unsigned int* p, unsigned int v)
-{
-    unsigned int old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
 }
 
 __device__ __forceinline__ float unordered(unsigned int o)
@@ -692,191 +700,294 @@ __device__ __forceinline__ float unordered(unsigned int o)
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);   // inverse of ordered()
 }
 
-// Called by one thread of every CTA of a cooperative launch (all resident)
-// with the CTA's key (nonzero); returns the grid's maximum in *out, or false
-// when this CTA gave up waiting (WT_ERR_TIMEOUT recorded) or another CTA had.
-// Each CTA folds its key into the slot's maximum and then counts itself in;
-// the last to arrive reads the maximum and publishes it with a release
-// store; the others poll for it with acquire loads, at most `limit` times.
-// CTA 0 clears the slot of the previous iteration once this one's result is
-// out: every CTA has read that slot's result before arriving here, and no
-// CTA uses it again before CTA 0 arrives at the next iteration.
-__device__ bool grid_max(HogSync* sy, int it, unsigned long long key, unsigned long long* out,
-                         uint32_t limit = kGridSpinLimit)
+// Key of a value at a pixel: larger values first, then lower pixels. 0: none.
+__device__ __forceinline__ unsigned long long pixel_key(float v, unsigned int pixel)
 {
-    const int slot = it % 3;
-    atomicMax(&sy->key[slot], key);
-    unsigned long long r = 0;
-    // release: the key, and this CTA's clearing of a slot, before its
-    // arrival; acquire: for the last to arrive, every other CTA's key
-    if (atom_add_acq_rel(&sy->count[slot], 1u) == gridDim.x - 1) {
-        r = atomicAdd(&sy->key[slot], 0ull);   // every key is in
-        st_release_u64(&sy->result[slot], r);
-    } else {
-        uint32_t polls = 0;
-        while ((r = ld_acquire_u64(&sy->result[slot])) == 0) {
-            if (*reinterpret_cast<volatile int*>(&sy->abort) || ++polls > limit) {
-                atomicExch(&sy->abort, 1);
-                return false;
-            }
-            __nanosleep(40);
+    return (static_cast<unsigned long long>(ordered(v)) << 32) | (0xffffffffu - pixel);
+}
+__device__ __forceinline__ unsigned int key_pixel(unsigned long long key)
+{
+    return 0xffffffffu - static_cast<unsigned int>(key);
+}
+__device__ __forceinline__ float key_value(unsigned long long key)
+{
+    return unordered(static_cast<unsigned int>(key >> 32));   // no key: NaN
+}
+
+// The largest key of a warp, in every lane.
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key)
+{
+    const unsigned int hi = static_cast<unsigned int>(key >> 32);
+    const unsigned int mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned int ml = __reduce_max_sync(0xffffffffu, hi == mh ? static_cast<unsigned int>(key) : 0u);
+    return (static_cast<unsigned long long>(mh) << 32) | ml;
+}
+
+// One thread of every CTA of a cooperative launch (all resident), its CTA's
+// writes made visible to it by a CTA barrier: counts itself in (release) and
+// waits (acquire) until `target` arrivals are in, over all meetings so far;
+// false when this CTA gave up waiting or another CTA had.
+__device__ bool grid_meet(HogSync* sy, unsigned int target, uint32_t limit = kGridSpinLimit)
+{
+    __threadfence();
+    atomicAdd(&sy->count, 1u);
+    for (uint32_t polls = 0; static_cast<int>(ld_acquire_u32(&sy->count) - target) < 0; ++polls) {
+        if (*reinterpret_cast<volatile int*>(&sy->abort) || polls >= limit) {
+            atomicExch(&sy->abort, 1);
+            return false;
         }
+        __nanosleep(40);
     }
-    if (blockIdx.x == 0) {
-        const int prev = (it + 2) % 3;
-        sy->count[prev] = 0;
-        sy->key[prev] = 0;
-        sy->result[prev] = 0;
-    }
-    *out = r;
+    __threadfence();
     return true;
 }
 
-// A grid maximum that never completes: the arrival count starts past the
-// grid size.
+// A meeting that never completes: one arrival more than the grid makes.
 __global__ void k_selftest_grid_barrier(HogSync* sy, uint32_t limit, int* status)
 {
-    unsigned long long r;
-    if (threadIdx.x == 0 && !grid_max(sy, 0, 1ull, &r, limit)) record_status(status, WT_ERR_TIMEOUT);
+    if (threadIdx.x == 0 && !grid_meet(sy, gridDim.x + 1, limit)) record_status(status, WT_ERR_TIMEOUT);
 }
 
 // CTA b owns image rows b, b + G, b + 2G, ... (G = gridDim.x <= n), held in
-// shared memory as local rows 0, 1, 2, ... for the whole clean. V4: n is a
-// multiple of 4 and the image 16-byte aligned (four pixels per thread step).
-template <bool V4>
-__global__ void __launch_bounds__(kHogThreads) k_hogbom_persistent(float* __restrict__ img,
-                                                                  const float* __restrict__ psf, int n, float gain,
-                                                                  float threshold, int max_iter,
-                                                                  HogSync* __restrict__ sy, int* __restrict__ comp_pix,
-                                                                  float* __restrict__ comp_flux,
-                                                                  int* __restrict__ n_comp, int* status)
+// shared memory as local rows 0, 1, 2, ... for the whole clean; one CTA per SM.
+// A warp takes segments of 128 pixels of a row (every 32nd of the CTA's
+// row-major list of them), a lane the pixels lane, lane + 32, ...: the beam,
+// shifted by any number of pixels, is read in whole lines. The beam comes from
+// L2, four bytes per pixel and component, which bounds large images; playing a
+// component (a CTA-wide maximum and a gather of the beam) bounds small ones.
+// Microseconds a component, one component per meeting before -> now: 64 x 64
+// 3.2 -> 1.2, 512 x 512 3.9 -> 1.7, 1024 x 1024 4.1 -> 2.0, 2048 x 2048 6.5 ->
+// 3.5 (noise, little to batch); a 2048 x 2048 field of 300 sources 6.7 -> 3.3.
+__global__ void __launch_bounds__(kHogThreads, 1) k_hogbom_persistent(float* __restrict__ img,
+                                                                     const float* __restrict__ psf, int n, float gain,
+                                                                     float threshold, int max_iter,
+                                                                     HogSync* __restrict__ sy,
+                                                                     int* __restrict__ comp_pix,
+                                                                     float* __restrict__ comp_flux,
+                                                                     int* __restrict__ n_comp, int* status)
 {
     extern __shared__ __align__(16) float rows[];
-    __shared__ unsigned long long wbest[kHogThreads / 32];
-    __shared__ unsigned long long gbest;
+    __shared__ unsigned long long wkey[2][kHogWarps * kWarpTop];
+    __shared__ unsigned int wbound[kHogWarps];
+    __shared__ int b_oy[kBatch], b_ox[kBatch];   // the beam's row and column over image pixel (0, 0)
+    __shared__ float b_f[kBatch];
+    __shared__ bool gave_up;
     const int G = gridDim.x, b = blockIdx.x, c = n / 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nloc = (n - 1 - b) / G + 1;
-    constexpr int kStep = V4 ? 4 : 1;
-    for (int r = 0; r < nloc; ++r) {
-        const float* src = img + static_cast<int64_t>(b + r * G) * n;
-        float* dst = rows + static_cast<int64_t>(r) * n;
-        if constexpr (V4) {
-            for (int x = 4 * threadIdx.x; x < n; x += 4 * kHogThreads)
-                *reinterpret_cast<float4*>(dst + x) = __ldcg(reinterpret_cast<const float4*>(src + x));
-        } else {
-            for (int x = threadIdx.x; x < n; x += kHogThreads) dst[x] = __ldcg(src + x);
+    const int segs = (n + 127) / 128, items = segs * nloc;
+    float neg = 0.0f, pos = 0.0f;                // the beam's largest -psf and psf, at least 0 (NaN aside)
+    for (int r = 0; r < nloc; ++r)
+        for (int x = tid; x < n; x += kHogThreads) {
+            const int64_t q = static_cast<int64_t>(b + r * G) * n + x;
+            rows[r * n + x] = __ldcg(img + q);
+            const float p = __ldg(psf + q);
+            neg = fmaxf(neg, -p);
+            pos = fmaxf(pos, p);
         }
+    // non-negative floats order as their bits
+    wkey[0][warp] = (static_cast<unsigned long long>(__reduce_max_sync(0xffffffffu, __float_as_uint(neg))) << 32) |
+                    __reduce_max_sync(0xffffffffu, __float_as_uint(pos));
+    __syncthreads();
+    if (tid == 0) {
+        unsigned int hn = 0, hp = 0;
+        for (int w = 0; w < kHogWarps; ++w) {
+            hn = max(hn, static_cast<unsigned int>(wkey[0][w] >> 32));
+            hp = max(hp, static_cast<unsigned int>(wkey[0][w]));
+        }
+        sy->beam[b][0] = __uint_as_float(hn);
+        sy->beam[b][1] = __uint_as_float(hp);
     }
     __syncthreads();
-    int pend = -1, it = 0;
-    float pf = 0.0f;
-    for (;;) {
-        const int py = pend >= 0 ? pend / n : 0, px = pend >= 0 ? pend % n : 0;
-        // this thread's largest value and its pixel (ties: the lower pixel)
-        float bv = -INFINITY;
+
+    int m = 0, it = 0;                           // components of the batch, and in all
+    bool finished = false;
+    for (unsigned int epoch = 0;; ++epoch) {
+        // ---- the batch off the rows; the thread's largest pixel and the
+        // largest of its others (pixels in increasing order: a strict
+        // comparison keeps the first of equals)
+        float b1 = -INFINITY, b2 = -INFINITY;
         unsigned int bq = 0xffffffffu;
-        for (int qx = kStep * threadIdx.x; qx < n; qx += kStep * kHogThreads) {
-            for (int r0 = 0; r0 < nloc; r0 += kRowsAhead) {
-                // the beam values of kRowsAhead rows first: their loads overlap
-                float bm[kRowsAhead][kStep];
-                bool in[kRowsAhead][kStep];
+        for (int item = warp; item < items; item += kHogWarps) {
+            const int r = item / segs, xs = (item - r * segs) * 128;
+            const int row = b + r * G;
+            float* px = rows + r * n + xs + lane;
+            float v[4];
 #pragma unroll
-                for (int i = 0; i < kRowsAhead; ++i) {
-                    const int by = b + (r0 + i) * G - py + c;   // beam row under image row b + (r0 + i) G
-                    const bool hit = pend >= 0 && r0 + i < nloc && by >= 0 && by < n;
-                    const float* brow = psf + static_cast<int64_t>(hit ? by : 0) * n;
+            for (int j = 0; j < 4; ++j) v[j] = xs + lane + 32 * j < n ? px[32 * j] : 0.0f;
+            for (int i0 = 0; i0 < m; i0 += 4) {
+                float bm[4][4];
+                bool in[4];
+                bool whole = xs + 128 <= n;      // every pixel of the segment under every beam of the four
 #pragma unroll
-                    for (int j = 0; j < kStep; ++j) {
-                        const int bx = qx + j - px + c;         // beam column under qx + j
-                        in[i][j] = hit && bx >= 0 && bx < n;
-                        bm[i][j] = in[i][j] ? __ldg(brow + bx) : 0.0f;
-                    }
+                for (int i = 0; i < 4; ++i) {
+                    const int by = row + b_oy[i0 + i], bx = xs + b_ox[i0 + i];   // past m: rows off the beam
+                    in[i] = by >= 0 && by < n;
+                    whole = whole && (!in[i] || (bx >= 0 && bx + 128 <= n));
                 }
+                if (whole) {
 #pragma unroll
-                for (int i = 0; i < kRowsAhead; ++i) {
-                    const int r = r0 + i;
-                    if (r >= nloc) break;
-                    float* row = rows + static_cast<int64_t>(r) * n;
-                    float v[kStep];
-                    if constexpr (V4) {
-                        const float4 v4 = *reinterpret_cast<const float4*>(row + qx);
-                        v[0] = v4.x; v[1] = v4.y; v[2] = v4.z; v[3] = v4.w;
-                    } else {
-                        v[0] = row[qx];
+                    for (int i = 0; i < 4; ++i) {
+                        const float* p = psf + static_cast<int64_t>(in[i] ? row + b_oy[i0 + i] : 0) * n +
+                                         (in[i] ? xs + b_ox[i0 + i] : 0) + lane;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) bm[i][j] = __ldg(p + 32 * j);
                     }
-                    bool any = false;
 #pragma unroll
-                    for (int j = 0; j < kStep; ++j)
-                        if (in[i][j]) {
-                            v[j] = __fsub_rn(v[j], __fmul_rn(pf, bm[i][j]));
-                            any = true;
-                        }
-                    if (any) {
-                        if constexpr (V4) {
-                            *reinterpret_cast<float4*>(row + qx) = make_float4(v[0], v[1], v[2], v[3]);
-                        } else {
-                            row[qx] = v[0];
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        if (!in[i]) continue;
+                        const float f = b_f[i0 + i];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[j] = __fsub_rn(v[j], __fmul_rn(f, bm[i][j]));
                     }
-                    const unsigned int q0 = static_cast<unsigned int>(b + r * G) * static_cast<unsigned int>(n);
+                } else {
 #pragma unroll
-                    for (int j = 0; j < kStep; ++j) {
-                        const unsigned int q = q0 + static_cast<unsigned int>(qx + j);
-                        if (v[j] > bv || (v[j] == bv && q < bq)) {
-                            bv = v[j];
-                            bq = q;
+                    for (int i = 0; i < 4; ++i) {
+                        if (!in[i]) continue;
+                        const float* p = psf + static_cast<int64_t>(row + b_oy[i0 + i]) * n;
+                        const float f = b_f[i0 + i];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int x = xs + lane + 32 * j, bx = x + b_ox[i0 + i];
+                            if (x < n && bx >= 0 && bx < n) v[j] = __fsub_rn(v[j], __fmul_rn(f, __ldg(p + bx)));
                         }
                     }
                 }
             }
-        }
-        unsigned long long key =
-            bq == 0xffffffffu ? 0ull : (static_cast<unsigned long long>(ordered(bv)) << 32) | (0xffffffffu - bq);
+            const unsigned int q0 = static_cast<unsigned int>(row) * static_cast<unsigned int>(n) + xs + lane;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
-            if (other > key) key = other;
-        }
-        if ((threadIdx.x & 31) == 0) wbest[threadIdx.x >> 5] = key;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long m = wbest[0];
-            for (int w = 1; w < kHogThreads / 32; ++w)
-                if (wbest[w] > m) m = wbest[w];
-            // a CTA without a comparable value (all NaN) still takes part with
-            // the smallest key, which decodes to NaN and stops the clean
-            if (m == 0) m = 1;
-            unsigned long long g = 0;
-            if (!grid_max(sy, it, m, &g)) {
-                record_status(status, WT_ERR_TIMEOUT);
-                g = 0;
+            for (int j = 0; j < 4; ++j) {
+                if (xs + lane + 32 * j >= n) continue;
+                if (m > 0) px[32 * j] = v[j];
+                if (v[j] > b1) {
+                    b2 = b1;
+                    b1 = v[j];
+                    bq = q0 + 32 * j;
+                } else {
+                    b2 = fmaxf(b2, v[j]);
+                }
             }
-            gbest = g;
+        }
+        if (finished) break;
+
+        // ---- the CTA's kTop largest of the threads' pixels, at most kWarpTop
+        // from a warp, and the bound on all the others
+        {
+            unsigned long long key = bq == 0xffffffffu ? 0ull : pixel_key(b1, bq);
+            float rest = b2;
+#pragma unroll
+            for (int k = 0; k < kWarpTop; ++k) {
+                const unsigned long long top = warp_max_key(key);
+                if (lane == 0) wkey[0][warp * kWarpTop + k] = top;
+                if (key == top) key = 0ull;      // keys are distinct, but for none
+            }
+            if (key != 0ull) rest = fmaxf(rest, key_value(key));
+            const unsigned int o = __reduce_max_sync(0xffffffffu, ordered(rest));
+            if (lane == 0) wbound[warp] = o;
         }
         __syncthreads();
-        if (gbest == 0) return;   // gave up waiting: every CTA leaves
-        const unsigned long long k = gbest;
-        const float peak = unordered(static_cast<unsigned int>(k >> 32));
-        if (it >= max_iter || !(peak >= threshold)) break;
-        pend = static_cast<int>(0xffffffffu - static_cast<unsigned int>(k & 0xffffffffu));
-        pf = __fmul_rn(gain, peak);
-        if (b == 0 && threadIdx.x == 0) {
-            comp_pix[it] = pend;
-            comp_flux[it] = pf;
+        if (warp == 0) {
+            // a lane's keys are a warp's, in decreasing order
+            const unsigned long long* mine = wkey[0] + lane * kWarpTop;
+            int taken = 0;
+            unsigned long long out = 0ull;
+#pragma unroll
+            for (int k = 0; k < kTop; ++k) {
+                const unsigned long long head = taken < kWarpTop ? mine[taken] : 0ull;
+                const unsigned long long top = warp_max_key(head);
+                if (head == top && head != 0ull) ++taken;
+                if (lane == k) out = top;
+            }
+            unsigned int o = wbound[lane];
+            if (taken < kWarpTop && mine[taken] != 0ull)
+                o = max(o, static_cast<unsigned int>(mine[taken] >> 32));
+            o = __reduce_max_sync(0xffffffffu, o);
+            if (lane < kTop) __stcg(&sy->key[epoch & 1][b][lane], out);
+            if (lane == 0) __stcg(&sy->bound[epoch & 1][b], unordered(o));
+            __syncwarp();
+            if (lane == 0) {
+                const bool ok = grid_meet(sy, (epoch + 1) * static_cast<unsigned int>(G));
+                if (!ok) record_status(status, WT_ERR_TIMEOUT);
+                gave_up = !ok;
+            }
         }
-        ++it;
-    }
-    for (int r = 0; r < nloc; ++r) {
-        float* dst = img + static_cast<int64_t>(b + r * G) * n;
-        const float* src = rows + static_cast<int64_t>(r) * n;
-        if constexpr (V4) {
-            for (int x = 4 * threadIdx.x; x < n; x += 4 * kHogThreads)
-                *reinterpret_cast<float4*>(dst + x) = *reinterpret_cast<const float4*>(src + x);
-        } else {
-            for (int x = threadIdx.x; x < n; x += kHogThreads) dst[x] = src[x];
+        __syncthreads();
+        if (gave_up) return;   // every CTA leaves
+
+        // ---- the posted pixels of this thread, and the bound on all others
+        float pv[kPerThread];
+        int py[kPerThread], px[kPerThread];
+        float lim = -INFINITY;
+        for (int g = lane; g < G; g += 32) lim = fmaxf(lim, __ldcg(&sy->bound[epoch & 1][g]));
+        lim = unordered(__reduce_max_sync(0xffffffffu, ordered(lim)));
+        if (epoch == 0) {
+            for (int g = lane; g < G; g += 32) {
+                neg = fmaxf(neg, __ldcg(&sy->beam[g][0]));
+                pos = fmaxf(pos, __ldcg(&sy->beam[g][1]));
+            }
+            neg = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(neg)));
+            pos = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(pos)));
         }
+#pragma unroll
+        for (int i = 0; i < kPerThread; ++i) {
+            const int k = tid + i * kHogThreads;
+            const unsigned long long key = k < G * kTop ? __ldcg(&sy->key[epoch & 1][0][0] + k) : 0ull;
+            pv[i] = key_value(key);              // NaN: none
+            const int q = key ? static_cast<int>(key_pixel(key)) : 0;
+            py[i] = q / n;
+            px[i] = q - py[i] * n;
+        }
+
+        // ---- the iterations that are certain
+        for (m = 0; m < kBatch;) {
+            unsigned long long key = 0ull;
+#pragma unroll
+            for (int i = 0; i < kPerThread; ++i)
+                if (pv[i] > -INFINITY) {
+                    const unsigned long long k = pixel_key(pv[i], static_cast<unsigned int>(py[i] * n + px[i]));
+                    key = k > key ? k : key;
+                }
+            key = warp_max_key(key);
+            if (lane == 0) wkey[m & 1][warp] = key;
+            __syncthreads();
+            key = warp_max_key(wkey[m & 1][lane]);
+            const float peak = key_value(key);
+            if (m > 0 && !(peak > lim)) break;   // another pixel may be larger
+            if (it >= max_iter || !(peak >= threshold)) {
+                finished = true;
+                break;
+            }
+            const int q = static_cast<int>(key_pixel(key));
+            const int oy = c - q / n, ox = c - (q - q / n * n);
+            const float f = __fmul_rn(gain, peak);
+            if (tid == 0) {
+                b_oy[m] = oy;
+                b_ox[m] = ox;
+                b_f[m] = f;
+                if (b == 0) {
+                    comp_pix[it] = q;
+                    comp_flux[it] = f;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kPerThread; ++i) {
+                const int by = py[i] + oy, bx = px[i] + ox;
+                if (pv[i] > -INFINITY && by >= 0 && by < n && bx >= 0 && bx < n)
+                    pv[i] = __fsub_rn(pv[i], __fmul_rn(f, __ldg(psf + static_cast<int64_t>(by) * n + bx)));
+            }
+            lim = f >= 0.0f ? __fadd_ru(lim, __fmul_ru(f, neg)) : __fadd_ru(lim, __fmul_ru(-f, pos));
+            ++m;
+            ++it;
+        }
+        __syncthreads();                         // the batch's list, and the keys' last readers
+        if (finished && m == 0) break;
+        if (tid < ((m + 3) & ~3) - m) b_oy[m + tid] = 2 * n;   // a last group of four filled up with beams off every row
+        __syncthreads();
     }
-    if (b == 0 && threadIdx.x == 0) *n_comp = it;
+    __syncthreads();
+    for (int r = 0; r < nloc; ++r)
+        for (int x = tid; x < n; x += kHogThreads) img[static_cast<int64_t>(b + r * G) * n + x] = rows[r * n + x];
+    if (b == 0 && tid == 0) *n_comp = it;
 }
 
 // ---------------------------------------------------------------- components
@@ -932,7 +1043,6 @@ size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 // CTAs and shared-memory bytes of a persistent clean of an n x n image, or 0
 // CTAs when the schedule does not apply (rows too large for shared memory,
 // no cooperative launch, or WT_HOGBOM=launches in the environment).
-template <bool V4>
 int persistent_grid(int n, size_t* smem)
 {
     const char* e = getenv("WT_HOGBOM");
@@ -945,38 +1055,31 @@ int persistent_grid(int n, size_t* smem)
         return 0;
     }
     const int sms = num_sms();
-    for (int per_sm = 2; per_sm >= 1; --per_sm) {
-        const int G = std::min(std::min(n, per_sm * sms), kMaxHogCtas);
-        const size_t bytes = static_cast<size_t>((n + G - 1) / G) * n * sizeof(float);
-        if (bytes > static_cast<size_t>(optin) - 1024) continue;
-        if (cudaFuncSetAttribute(k_hogbom_persistent<V4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(bytes)) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hogbom_persistent<V4>, kHogThreads, bytes) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        if (static_cast<int64_t>(occ) * sms >= G) {
-            *smem = bytes;
-            return G;
-        }
+    const int G = std::min(std::min(n, sms), kMaxHogCtas);
+    const size_t bytes = static_cast<size_t>((n + G - 1) / G) * n * sizeof(float);
+    cudaFuncAttributes fa;
+    int occ = 0;
+    if (cudaFuncGetAttributes(&fa, k_hogbom_persistent) != cudaSuccess ||
+        bytes + fa.sharedSizeBytes > static_cast<size_t>(optin) ||
+        cudaFuncSetAttribute(k_hogbom_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(bytes)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hogbom_persistent, kHogThreads, bytes) != cudaSuccess ||
+        static_cast<int64_t>(occ) * sms < G) {
+        cudaGetLastError();
+        return 0;
     }
-    return 0;
+    *smem = bytes;
+    return G;
 }
 
-template <bool V4>
 int launch_persistent(int G, size_t smem, float* image, const float* psf, int n, float gain, float threshold,
                       int max_iter, HogSync* sy, int* comp_pix, float* comp_flux, int* n_comp, cudaStream_t s)
 {
     int* status = device_status_word();
     if (!status) return set_error(WT_ERR_CUDA, "wt_hogbom: no device status word");
-    WT_CUDA_TRY(cudaMemsetAsync(sy, 0, sizeof(HogSync), s));
+    WT_CUDA_TRY(cudaMemsetAsync(sy, 0, offsetof(HogSync, beam), s));
     void* args[] = {&image, &psf, &n, &gain, &threshold, &max_iter, &sy, &comp_pix, &comp_flux, &n_comp, &status};
-    WT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_hogbom_persistent<V4>), dim3(G),
+    WT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_hogbom_persistent), dim3(G),
                                             dim3(kHogThreads), args, smem, s));
     return WT_OK;
 }
@@ -987,14 +1090,10 @@ int hogbom(float* image, const float* psf, int n, float gain, float threshold, i
            float* comp_flux, int* n_comp, void* state, cudaStream_t s)
 {
     HogSync* sy = reinterpret_cast<HogSync*>(static_cast<char*>(state) + round256(sizeof(HogbomState)));
-    const bool v4 = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(image) & 15) == 0;
     size_t smem = 0;
-    const int G = v4 ? persistent_grid<true>(n, &smem) : persistent_grid<false>(n, &smem);
+    const int G = persistent_grid(n, &smem);
     if (G > 0)
-        return v4 ? launch_persistent<true>(G, smem, image, psf, n, gain, threshold, max_iter, sy, comp_pix,
-                                            comp_flux, n_comp, s)
-                  : launch_persistent<false>(G, smem, image, psf, n, gain, threshold, max_iter, sy, comp_pix,
-                                             comp_flux, n_comp, s);
+        return launch_persistent(G, smem, image, psf, n, gain, threshold, max_iter, sy, comp_pix, comp_flux, n_comp, s);
     k_hogbom_reset<<<1, 1, 0, s>>>(static_cast<HogbomState*>(state), n_comp);
     const int blocks = rows_blocks(n);
     // max_iter + 1 launches: the last subtracts the last component and stops
@@ -1248,7 +1347,6 @@ extern "C" int wt_selftest_grid_barrier(uint32_t spin_limit, void* stream)
     WT_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&sy), sizeof(HogSync), s));
     int rc = WT_OK;
     cudaError_t e = cudaMemsetAsync(sy, 0, sizeof(HogSync), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&sy->count[0], 0x02, sizeof(unsigned int), s);   // 0x02020202 arrivals
     if (e == cudaSuccess) {
         void* args[] = {&sy, &spin_limit, &status};
         e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_selftest_grid_barrier), dim3(2), dim3(32),
