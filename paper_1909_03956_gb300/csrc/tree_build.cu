@@ -17,9 +17,13 @@
 //                      topology and Eqs. 9/10 in the paper's order.
 //   k_tree_records     one thread per node: post-order position and the
 //                      packed records the predictors stream.
+//   k_build_small      for up to kSmallComps components, everything up to the
+//                      records in one CTA, its levels in shared memory.
 // Rounding: every float64 step that must match the CPU definition bit for bit
 // uses the _rn intrinsics, which the compiler never contracts into FMAs.
 #include <math.h>
+
+#include <algorithm>
 
 #include "sphere.cuh"
 #include "wt_internal.cuh"
@@ -221,6 +225,55 @@ __device__ __forceinline__ double quarter_sqrt_area(int j)
     return __dmul_rn(ldexp(__dsqrt_rn(kPi / 3.0), 1 - j), 0.25);
 }
 
+// What a leaf holds: its merged flux, lambda_J = Phi / A_J, pixel centre and
+// range; smax, the bounds of the coordinates' float32 heads (float bits).
+__device__ __forceinline__ double leaf_values(const TreeDev& d, int64_t leaf, int64_t key, double phi_k, int J,
+                                              const Rot& R, unsigned* smax)
+{
+    const double lambda = __ddiv_rn(phi_k, area_level(J));
+    d.leaf_flux[leaf] = phi_k;
+    d.lambda[leaf] = lambda;
+    d.gamma[3 * leaf + 0] = 0.0;
+    d.gamma[3 * leaf + 1] = 0.0;
+    d.gamma[3 * leaf + 2] = 0.0;
+    d.first_child[leaf] = -1;
+    d.mask[leaf] = 0;
+    d.leaf_lo[leaf] = static_cast<int32_t>(leaf);
+    d.leaf_hi[leaf] = static_cast<int32_t>(leaf + 1);
+    d.size[leaf] = 1;
+    // pixel centre -> xyz (y to the NCP, x to RA 6h, z to RA 0h) -> uvw = R^T xyz
+    double z, st, ph;
+    pixel_centre(J - 1, key, z, st, ph);
+    double sph, cph;
+    sincos(ph, &sph, &cph);
+    const double x = st * sph, y = z, zc = st * cph;
+    const double su = R.r[0] * x + R.r[3] * y + R.r[6] * zc;
+    const double sv = R.r[1] * x + R.r[4] * y + R.r[7] * zc;
+    const double sw = R.r[2] * x + R.r[5] * y + R.r[8] * zc;
+    const double sw1 = (sw > 0.0) ? -(su * su + sv * sv) / (1.0 + sw) : sw - 1.0;
+    d.leaf_dir[3 * leaf + 0] = su;
+    d.leaf_dir[3 * leaf + 1] = sv;
+    d.leaf_dir[3 * leaf + 2] = sw1;
+    // the float32 heads the records carry (split_f64), whose products the
+    // grid pass bounds
+    atomicMax(&smax[0], __float_as_uint(fabsf(split_f64(su).hi)));
+    atomicMax(&smax[1], __float_as_uint(fabsf(split_f64(sv).hi)));
+    atomicMax(&smax[2], __float_as_uint(fabsf(split_f64(sw1).hi)));
+    return lambda;
+}
+
+// Eq. 9 and Eq. 10 of node P at level j from its children's lambda by slot,
+// children added left to right in slot order; returns lambda.
+__device__ __forceinline__ double node_values(const TreeDev& d, int64_t P, double q, const double (&ch)[4])
+{
+    const double lambda = __dmul_rn(0.25, __dadd_rn(__dadd_rn(__dadd_rn(ch[0], ch[1]), ch[2]), ch[3]));
+    d.lambda[P] = lambda;
+    d.gamma[3 * P + 0] = __dmul_rn(q, __dsub_rn(__dadd_rn(__dsub_rn(ch[0], ch[1]), ch[2]), ch[3]));
+    d.gamma[3 * P + 1] = __dmul_rn(q, __dsub_rn(__dsub_rn(__dadd_rn(ch[0], ch[1]), ch[2]), ch[3]));
+    d.gamma[3 * P + 2] = __dmul_rn(q, __dadd_rn(__dsub_rn(__dsub_rn(ch[0], ch[1]), ch[2]), ch[3]));
+    return lambda;
+}
+
 __global__ void __launch_bounds__(kLevelThreads) k_tree_levels(const uint64_t* __restrict__ skeys,
                                                                const double* __restrict__ sflux, int64_t n_comp,
                                                                int J, Rot R, TreeDev d)
@@ -260,40 +313,12 @@ __global__ void __launch_bounds__(kLevelThreads) k_tree_levels(const uint64_t* _
     __syncthreads();
 
     // ---- leaf values: Phi_k summed in input order, lambda_J, pixel centre
-    const double AJ = area_level(J);
     for (int64_t leaf = tid; leaf < n_leaves; leaf += nt) {
         const int64_t e0 = d.parent[leaf];
         const int64_t e1 = (leaf + 1 < n_leaves) ? d.parent[leaf + 1] : n_comp;
         double phi_k = 0.0;
         for (int64_t e = e0; e < e1; ++e) phi_k = __dadd_rn(phi_k, sflux[e]);
-        d.leaf_flux[leaf] = phi_k;
-        d.lambda[leaf] = __ddiv_rn(phi_k, AJ);
-        d.gamma[3 * leaf + 0] = 0.0;
-        d.gamma[3 * leaf + 1] = 0.0;
-        d.gamma[3 * leaf + 2] = 0.0;
-        d.first_child[leaf] = -1;
-        d.mask[leaf] = 0;
-        d.leaf_lo[leaf] = static_cast<int32_t>(leaf);
-        d.leaf_hi[leaf] = static_cast<int32_t>(leaf + 1);
-        d.size[leaf] = 1;
-        // pixel centre -> xyz (y to the NCP, x to RA 6h, z to RA 0h) -> uvw = R^T xyz
-        double z, st, ph;
-        pixel_centre(J - 1, d.key[leaf], z, st, ph);
-        double sph, cph;
-        sincos(ph, &sph, &cph);
-        const double x = st * sph, y = z, zc = st * cph;
-        const double su = R.r[0] * x + R.r[3] * y + R.r[6] * zc;
-        const double sv = R.r[1] * x + R.r[4] * y + R.r[7] * zc;
-        const double sw = R.r[2] * x + R.r[5] * y + R.r[8] * zc;
-        const double sw1 = (sw > 0.0) ? -(su * su + sv * sv) / (1.0 + sw) : sw - 1.0;
-        d.leaf_dir[3 * leaf + 0] = su;
-        d.leaf_dir[3 * leaf + 1] = sv;
-        d.leaf_dir[3 * leaf + 2] = sw1;
-        // the float32 heads the records carry (split_f64), whose products
-        // the grid pass bounds
-        atomicMax(&s_smax[0], __float_as_uint(fabsf(split_f64(su).hi)));
-        atomicMax(&s_smax[1], __float_as_uint(fabsf(split_f64(sv).hi)));
-        atomicMax(&s_smax[2], __float_as_uint(fabsf(split_f64(sw1).hi)));
+        leaf_values(d, leaf, d.key[leaf], phi_k, J, R, s_smax);
     }
     __syncthreads();
 
@@ -340,11 +365,7 @@ __global__ void __launch_bounds__(kLevelThreads) k_tree_levels(const uint64_t* _
             d.size[P] = size;
             d.leaf_lo[P] = d.leaf_lo[base_c + fc];
             d.leaf_hi[P] = d.leaf_hi[base_c + lc - 1];
-            // Eq. 9 and Eq. 10, children added left to right in slot order
-            d.lambda[P] = __dmul_rn(0.25, __dadd_rn(__dadd_rn(__dadd_rn(ch[0], ch[1]), ch[2]), ch[3]));
-            d.gamma[3 * P + 0] = __dmul_rn(q, __dsub_rn(__dadd_rn(__dsub_rn(ch[0], ch[1]), ch[2]), ch[3]));
-            d.gamma[3 * P + 1] = __dmul_rn(q, __dsub_rn(__dsub_rn(__dadd_rn(ch[0], ch[1]), ch[2]), ch[3]));
-            d.gamma[3 * P + 2] = __dmul_rn(q, __dadd_rn(__dsub_rn(__dsub_rn(ch[0], ch[1]), ch[2]), ch[3]));
+            node_values(d, P, q, ch);
         }
         __syncthreads();
     }
@@ -365,11 +386,259 @@ __global__ void __launch_bounds__(kLevelThreads) k_tree_levels(const uint64_t* _
     }
 }
 
+// ---------------------------------------------------------------- small trees
+// Up to kSmallComps components, a thread each, in one CTA: keys, stable radix
+// sort, leaves, levels J-1 .. 1 and the post-order positions, the level being
+// read kept in shared memory (global memory is only written). The general path
+// takes 3 ceil((2J + 2) / 8) + 4 launches, latency bound; 100 components at
+// J = 8: SMALL_HERE.
+constexpr int kSmallComps = 1024;
+
+struct SmallSmem {
+    uint64_t key[2][kSmallComps];          // sort; then the levels' keys
+    double lambda[2][kSmallComps];
+    double flux[kSmallComps];
+    uint32_t idx[2][kSmallComps];
+    int32_t size[2][kSmallComps], lo[2][kSmallComps], hi[2][kSmallComps];
+    int32_t first[kSmallComps];
+    uint32_t wcnt[32][257];
+    uint32_t total[256];
+    uint32_t wsum[2][32];
+};
+
+// Exclusive prefix count of a flag per thread over the CTA's 32 warps, one
+// barrier (`buf`: one of two alternating sets of warp counts).
+__device__ __forceinline__ int flag_scan(bool flag, uint32_t* buf, int& total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned bits = __ballot_sync(0xffffffffu, flag);
+    if (lane == 0) buf[warp] = __popc(bits);
+    __syncthreads();
+    const unsigned cnt = buf[lane];
+    total = static_cast<int>(__reduce_add_sync(0xffffffffu, cnt));
+    const int before = static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? cnt : 0u));
+    return before + __popc(bits & ((1u << lane) - 1u));
+}
+
+// SRC: 0 components at (l, m), 1 image pixels through a cross-reference table,
+// 2 leaves already in key order.
+template <int SRC>
+__global__ void __launch_bounds__(kSmallComps) k_build_small(KeySource src, const double* __restrict__ flux, int n,
+                                                             int J, int passes, Rot R, TreeDev d, int* status)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
+    __shared__ int64_t s_count[kMaxJ + 2];
+    __shared__ int64_t s_roff[kMaxJ + 2];
+    __shared__ unsigned s_smax[3];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool valid = tid < n;
+    if (tid < 3) s_smax[tid] = 0u;
+    if (tid < kMaxJ + 2) {
+        s_count[tid] = 0;
+        s_roff[tid] = 0;
+    }
+
+    // ---- keys
+    uint64_t key = 0;
+    uint32_t idx = static_cast<uint32_t>(tid);
+    if (valid) {
+        const double f = flux[tid];
+        sm.flux[tid] = f;
+        if constexpr (SRC == 0) {
+            if (!isfinite(f) || !map_lm(src.l[tid], src.m[tid], R, J, &key)) {
+                key = 0;
+                record_status(status, WT_ERR_RANGE);
+            }
+        } else if constexpr (SRC == 1) {
+            const int32_t p = src.pix[tid];
+            const int64_t k = (p >= 0 && p < src.n_pix) ? src.table[p] : -1;
+            if (k < 0 || !isfinite(f)) record_status(status, WT_ERR_RANGE);
+            else key = static_cast<uint64_t>(k);
+        } else {
+            key = static_cast<uint64_t>(src.leaf_keys[tid]);
+        }
+    }
+
+    // ---- stable sort, 8 bits a pass
+    if constexpr (SRC != 2) {
+        const int nw = (n + 31) / 32;
+        for (int ps = 0; ps < passes; ++ps) {
+            const uint32_t dig = valid ? static_cast<uint32_t>((key >> (8 * ps)) & 255u) : 256u;
+            for (int k = tid; k < nw * 257; k += kSmallComps) sm.wcnt[k / 257][k % 257] = 0;
+            __syncthreads();
+            const unsigned peers = __match_any_sync(0xffffffffu, dig);
+            const int lrank = __popc(peers & ((1u << lane) - 1u));
+            if (valid && lrank == 0) sm.wcnt[warp][dig] = static_cast<uint32_t>(__popc(peers));
+            __syncthreads();
+            if (tid < 256) {
+                uint32_t run = 0;
+                for (int w = 0; w < nw; ++w) {
+                    const uint32_t c = sm.wcnt[w][tid];
+                    sm.wcnt[w][tid] = run;
+                    run += c;
+                }
+                sm.total[tid] = run;
+            }
+            __syncthreads();
+            if (warp == 0) {                       // exclusive prefix of the 256 totals, 8 per lane
+                uint32_t t[8], sum = 0;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    t[k] = sum;
+                    sum += sm.total[8 * lane + k];
+                }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) sm.total[8 * lane + k] = incl - sum + t[k];
+            }
+            __syncthreads();
+            if (valid) {
+                const uint32_t pos = sm.total[dig] + sm.wcnt[warp][dig] + static_cast<uint32_t>(lrank);
+                sm.key[0][pos] = key;
+                sm.idx[0][pos] = idx;
+            }
+            __syncthreads();
+            if (valid) {
+                key = sm.key[0][tid];
+                idx = sm.idx[0][tid];
+            }
+        }
+    }
+    if (valid) sm.key[1][tid] = key;
+    sm.idx[1][tid] = idx;
+    __syncthreads();
+
+    // ---- leaves
+    const bool lead = valid && (tid == 0 || sm.key[1][tid - 1] != key);
+    int n_leaves = 0;
+    const int leaf_at = flag_scan(lead, sm.wsum[0], n_leaves);
+    if (lead) sm.first[leaf_at] = tid;
+    __syncthreads();
+    if (tid < n_leaves) {
+        const int e0 = sm.first[tid], e1 = tid + 1 < n_leaves ? sm.first[tid + 1] : n;
+        const uint64_t k = sm.key[1][e0];
+        double phi_k = 0.0;
+        for (int e = e0; e < e1; ++e) phi_k = __dadd_rn(phi_k, sm.flux[sm.idx[1][e]]);
+        d.key[tid] = static_cast<int64_t>(k);
+        sm.key[0][tid] = k;
+        sm.lambda[0][tid] = leaf_values(d, tid, static_cast<int64_t>(k), phi_k, J, R, s_smax);
+        sm.size[0][tid] = 1;
+        sm.lo[0][tid] = tid;
+        sm.hi[0][tid] = tid + 1;
+    }
+    if (tid == 0) s_count[J] = n_leaves;
+    __syncthreads();
+
+    // ---- levels J-1 .. 1: the children's level in set b, the parents' in set 1 - b
+    int b = 0, n_c = n_leaves, base_c = 0;
+    for (int j = J - 1; j >= 1; --j, b ^= 1) {
+        const int base_p = base_c + n_c;
+        const bool child = tid < n_c;
+        const uint64_t kc = child ? sm.key[b][tid] : 0ull;
+        const bool head = child && (tid == 0 || (sm.key[b][tid - 1] >> 2) != (kc >> 2));
+        int n_p = 0;
+        const int ex = flag_scan(head, sm.wsum[j & 1], n_p);
+        if (head) {
+            sm.key[1 - b][ex] = kc >> 2;
+            sm.first[ex] = tid;
+        }
+        if (child) d.parent[base_c + tid] = ex + (head ? 1 : 0) - 1;
+        __syncthreads();
+        if (tid < n_p) {
+            const int fc = sm.first[tid], lc = tid + 1 < n_p ? sm.first[tid + 1] : n_c;
+            double ch[4] = {0.0, 0.0, 0.0, 0.0};
+            uint32_t mask = 0;
+            int32_t size = 1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = fc + k;
+                if (c < lc) {
+                    const int slot = static_cast<int>(sm.key[b][c] & 3ull);
+                    const double x = sm.lambda[b][c];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (slot == q) ch[q] = x;
+                    mask |= 1u << slot;
+                    d.post[base_c + c] = size - 1;     // the earlier siblings' subtrees, for now
+                    size += sm.size[b][c];
+                }
+            }
+            const int64_t P = base_p + tid;
+            d.key[P] = static_cast<int64_t>(sm.key[1 - b][tid]);
+            d.first_child[P] = fc;
+            d.mask[P] = static_cast<uint8_t>(mask);
+            d.size[P] = size;
+            d.leaf_lo[P] = sm.lo[b][fc];
+            d.leaf_hi[P] = sm.hi[b][lc - 1];
+            sm.lambda[1 - b][tid] = node_values(d, P, quarter_sqrt_area(j), ch);
+            sm.size[1 - b][tid] = size;
+            sm.lo[1 - b][tid] = sm.lo[b][fc];
+            sm.hi[1 - b][tid] = sm.hi[b][lc - 1];
+        }
+        if (tid == 0) {
+            s_count[j] = n_p;
+            s_roff[j] = base_p;
+        }
+        base_c = base_p;
+        n_c = n_p;
+        __syncthreads();
+    }
+
+    // ---- post-order positions, level 1 down: a subtree starts where its
+    // parent's does plus its earlier siblings' subtrees (level 1: at most 12
+    // pixels in key order), and its root comes last
+    int32_t* start = sm.lo[0];
+    int32_t* next = sm.lo[1];
+    if (tid == 0) {
+        int run = 0;
+        for (int k = 0; k < n_c; ++k) {
+            start[k] = run;
+            const int size = d.size[base_c + k];
+            d.post[base_c + k] = run + size - 1;
+            run += size;
+        }
+    }
+    __syncthreads();
+    for (int j = 2; j <= J; ++j) {
+        const int n_j = static_cast<int>(s_count[j]), base = static_cast<int>(s_roff[j]);
+        if (tid < n_j) {
+            const int at = start[d.parent[base + tid]] + d.post[base + tid];
+            next[tid] = at;
+            d.post[base + tid] = at + d.size[base + tid] - 1;
+        }
+        __syncthreads();
+        int32_t* t = start;
+        start = next;
+        next = t;
+    }
+
+    if (tid >= 1 && tid <= J) {
+        d.hdr->per_level[tid] = s_count[tid];
+        d.hdr->rev_offset[tid] = s_roff[tid];
+    }
+    if (tid == 0) {
+        const int64_t total = s_roff[1] + s_count[1];
+        d.hdr->per_level[0] = 0;
+        d.hdr->rev_offset[0] = total;
+        d.hdr->n_leaves = n_leaves;
+        d.hdr->n_nodes = total;
+        for (int c = 0; c < 3; ++c) d.hdr->smax[c] = __uint_as_float(s_smax[c]);
+        d.hdr->smax[3] = 0.0f;
+    }
+}
+
 // ---------------------------------------------------------------- records
 // Post-order position of a node n with leaf range [lo, hi) and subtree size
 // S: the nodes entirely left of its range (at every level, those whose leaf
 // range ends at or before lo) come first, then its S - 1 descendants.
-__global__ void k_tree_records(TreeDev d, int J, int* status)
+// placed: the positions are in d.post (k_build_small).
+__global__ void k_tree_records(TreeDev d, int J, bool placed, int* status)
 {
     const TreeHeader* h = d.hdr;
     const int64_t T = h->n_nodes;
@@ -380,8 +649,8 @@ __global__ void k_tree_records(TreeDev d, int J, int* status)
         int j = J;
         while (j > 1 && n >= h->rev_offset[j] + h->per_level[j]) --j;
         const int32_t lo = d.leaf_lo[n];
-        int64_t before = 0;
-        for (int jj = 1; jj <= J; ++jj) {
+        int64_t before = placed ? d.post[n] + 1 - d.size[n] : 0;
+        for (int jj = 1; jj <= J && !placed; ++jj) {
             // count level-jj nodes whose leaf range ends at or before lo
             const int32_t* hi = d.leaf_hi + h->rev_offset[jj];
             int64_t a = 0, b = h->per_level[jj];
@@ -552,8 +821,7 @@ int64_t carve_bytes(int64_t cap_nodes, int64_t cap_leaves)
 {
     auto b = [](int64_t x) { return (x + 255) & ~int64_t(255); };
     return b(cap_nodes * 8) + b(cap_nodes * 8) + b(cap_nodes * 24) + b(cap_nodes * 4) + b(cap_nodes) +
-           4 * b(cap_nodes * 4) + b(cap_leaves * 24) + b(cap_leaves * 8) + b(cap_leaves * 8) +
-           b(cap_leaves * 4) + b(cap_nodes * int64_t(sizeof(RecD))) + b(cap_nodes * int64_t(sizeof(RecF))) +
+           5 * b(cap_nodes * 4) + b(cap_leaves * 24) + b(cap_leaves * 8) + b(cap_nodes * int64_t(sizeof(RecD))) + b(cap_nodes * int64_t(sizeof(RecF))) +
            b(cap_leaves * int64_t(sizeof(RecD))) + b(cap_leaves * int64_t(sizeof(RecF))) +
            b(cap_nodes * int64_t(sizeof(RecWD))) + b(cap_nodes * int64_t(sizeof(RecWF))) +
            b(cap_nodes * int64_t(sizeof(RecWDF))) + b(sizeof(TreeHeader));
@@ -594,6 +862,7 @@ int build_tree(const KeySource& src, const double* flux, int64_t n_comp, double 
     // scratch for the sort: keys x2, idx x2, histogram, sorted fluxes
     const int nblk = static_cast<int>((n_comp + kSortTile - 1) / kSortTile);
     auto b256 = [](int64_t x) { return (x + 255) & ~int64_t(255); };
+    const bool small = n_comp <= kSmallComps;   // no scratch
     const int64_t scratch_bytes = 2 * b256(capl * 8) + 2 * b256(capl * 4) + b256(int64_t(256) * (nblk > 0 ? nblk : 1) * 4) +
                                   b256(capl * 8);
     const int64_t tree_bytes = carve_bytes(cap1, capl);
@@ -606,7 +875,7 @@ int build_tree(const KeySource& src, const double* flux, int64_t n_comp, double 
                          (long long)tree_bytes, cudaGetErrorString(e));
     }
     char* scratch = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), scratch_bytes, s);
+    e = small ? cudaSuccess : cudaMallocAsync(reinterpret_cast<void**>(&scratch), scratch_bytes, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFreeAsync(block, s);
@@ -627,10 +896,9 @@ int build_tree(const KeySource& src, const double* flux, int64_t n_comp, double 
     d.leaf_hi = carve<int32_t>(p, cap1);
     d.size = carve<int32_t>(p, cap1);
     d.parent = carve<int32_t>(p, cap1);
+    d.post = carve<int32_t>(p, cap1);
     d.leaf_dir = carve<double>(p, 3 * capl);
     d.leaf_flux = carve<double>(p, capl);
-    d.anc_sum = carve<int64_t>(p, capl);
-    d.anc = carve<int32_t>(p, capl);
     d.recd = carve<RecD>(p, cap1);
     d.recf = carve<RecF>(p, cap1);
     d.leafd = carve<RecD>(p, capl);
@@ -653,13 +921,25 @@ int build_tree(const KeySource& src, const double* flux, int64_t n_comp, double 
     int* status = device_status_word();
     if (!status) return set_error(WT_ERR_CUDA, "wt_build_tree: no device status word");
 
-    if (n_comp > 0 && src.leaf_keys) {
+    // (a thread per node: enough CTAs for the capacity, four per SM at most)
+    const unsigned rec_blocks =
+        static_cast<unsigned>(std::min<int64_t>((cap1 + 255) / 256, static_cast<int64_t>(num_sms()) * 4));
+    if (n_comp > 0 && small) {
+        const int passes = (2 * J + 2 + 7) / 8;
+        auto k = src.leaf_keys ? k_build_small<2> : src.table ? k_build_small<1> : k_build_small<0>;
+        WT_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(sizeof(SmallSmem))));
+        k<<<1, kSmallComps, sizeof(SmallSmem), s>>>(src, flux, static_cast<int>(n_comp), J, passes, R, d, status);
+        WT_CUDA_TRY(cudaGetLastError());
+        k_tree_records<<<rec_blocks, 256, 0, s>>>(d, J, true, status);
+        WT_CUDA_TRY(cudaGetLastError());
+    } else if (n_comp > 0 && src.leaf_keys) {
         // the leaves themselves (a tree re-imported from its export): one
         // component per distinct pixel, already in key order
         k_tree_levels<<<1, kLevelThreads, 0, s>>>(reinterpret_cast<const uint64_t*>(src.leaf_keys), flux, n_comp, J, R,
                                                   d);
         WT_CUDA_TRY(cudaGetLastError());
-        k_tree_records<<<num_sms() * 4, 256, 0, s>>>(d, J, status);
+        k_tree_records<<<rec_blocks, 256, 0, s>>>(d, J, false, status);
         WT_CUDA_TRY(cudaGetLastError());
     } else if (n_comp > 0) {
         const int tb = 256;
@@ -691,14 +971,13 @@ int build_tree(const KeySource& src, const double* flux, int64_t n_comp, double 
         WT_CUDA_TRY(cudaGetLastError());
         k_tree_levels<<<1, kLevelThreads, 0, s>>>(kin, sflux, n_comp, J, R, d);
         WT_CUDA_TRY(cudaGetLastError());
-        const int nsm = num_sms();
-        k_tree_records<<<nsm * 4, 256, 0, s>>>(d, J, status);
+        k_tree_records<<<rec_blocks, 256, 0, s>>>(d, J, false, status);
         WT_CUDA_TRY(cudaGetLastError());
     } else {
         WT_CUDA_TRY(cudaMemsetAsync(d.hdr, 0, sizeof(TreeHeader), s));
     }
     WT_CUDA_TRY(cudaMemcpyAsync(t->host_hdr, d.hdr, sizeof(TreeHeader), cudaMemcpyDeviceToHost, s));
-    WT_CUDA_TRY(cudaFreeAsync(scratch, s));
+    if (scratch) WT_CUDA_TRY(cudaFreeAsync(scratch, s));
     t->host_valid = false;
     return WT_OK;
 }

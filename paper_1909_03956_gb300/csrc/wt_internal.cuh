@@ -648,8 +648,7 @@ struct TreeDev {
     int32_t* parent;      // index of the parent within its level
     double* leaf_dir;     // [n_leaves cap][3]
     double* leaf_flux;    // [n_leaves cap]
-    int64_t* anc_sum;     // per leaf: sum over levels of the ancestor's index
-    int32_t* anc;         // per leaf: current ancestor index
+    int32_t* post;        // post-order position (filled by the small build only)
     RecD* recd;           // post-order records [cap]
     RecF* recf;
     RecD* leafd;          // leaf records in key order [n_leaves cap] (Eq. 16)
