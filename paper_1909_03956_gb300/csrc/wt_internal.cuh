@@ -150,24 +150,24 @@ __device__ __forceinline__ void phase_turns_df(F2 u, F2 v, F2 w, F2 su, F2 sv, F
 // float32. Quadrant reduction q = rint(4 th), f = (4 th - q) + 4 tl, the
 // first difference exact, so |f| <= 1/2 + 4|tl|; angle x = f * pi/2 (pi/2
 // rounded to float32: relative error 3e-8, below the float32 result's own
-// rounding); then the Taylor series of sin (to x^9) and cos (to x^10),
-// whose truncation errors on |x| <= 0.8 (< 4e-9 and < 5e-10) are below
-// float32 rounding.
+// rounding); then sin to x^7 and cos to x^8 with the coefficients that
+// minimise the largest error on |x| <= 0.84 (Remez exchange; 7e-9 and 7e-10
+// with the coefficients rounded to float32, below float32 rounding; the
+// Taylor series need a term more each for as much).
+constexpr float kSinC3 = -0.1666664332151413f, kSinC5 = 0.00833156332373619f, kSinC7 = -0.0001944637333508581f;
+constexpr float kCosC4 = 0.04166663810610771f, kCosC6 = -0.0013886900851503015f, kCosC8 = 2.43866270466242e-05f;
+
 __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, float& c)
 {
     const float q = rintf(4.0f * th);
     const float f = __fmaf_rn(4.0f, tl, __fsub_rn(4.0f * th, q));
     const float x = __fmul_rn(f, 1.57079637050628662109375f);
     const float x2 = __fmul_rn(x, x);
-    // sin x = x (1 - x^2/3! + x^4/5! - x^6/7! + x^8/9!)
-    float ps = __fmaf_rn(x2, 2.7557319223985893e-6f, -1.9841269841269841e-4f);
-    ps = __fmaf_rn(x2, ps, 8.3333333333333333e-3f);
-    ps = __fmaf_rn(x2, ps, -1.6666666666666667e-1f);
+    float ps = __fmaf_rn(x2, kSinC7, kSinC5);
+    ps = __fmaf_rn(x2, ps, kSinC3);
     const float sx = __fmaf_rn(__fmul_rn(x, x2), ps, x);
-    // cos x = 1 - x^2/2! + x^4/4! - x^6/6! + x^8/8! - x^10/10!
-    float pc = __fmaf_rn(x2, -2.7557319223985891e-7f, 2.4801587301587302e-5f);
-    pc = __fmaf_rn(x2, pc, -1.3888888888888889e-3f);
-    pc = __fmaf_rn(x2, pc, 4.1666666666666667e-2f);
+    float pc = __fmaf_rn(x2, kCosC8, kCosC6);
+    pc = __fmaf_rn(x2, pc, kCosC4);
     pc = __fmaf_rn(x2, pc, -0.5f);
     const float cx = __fmaf_rn(x2, pc, 1.0f);
     const int qi = static_cast<int>(q) & 3;
@@ -440,13 +440,11 @@ __device__ __forceinline__ void sincos_turns_f32x2(float2 h, float2 tl, float2& 
     const float2 f = fma2(bcast2(4.0f), tl, sub2(t4, q));
     const float2 x = mul2(f, bcast2(1.57079637050628662109375f));
     const float2 x2 = mul2(x, x);
-    float2 ps = fma2(x2, bcast2(2.7557319223985893e-6f), bcast2(-1.9841269841269841e-4f));
-    ps = fma2(x2, ps, bcast2(8.3333333333333333e-3f));
-    ps = fma2(x2, ps, bcast2(-1.6666666666666667e-1f));
+    float2 ps = fma2(x2, bcast2(kSinC7), bcast2(kSinC5));
+    ps = fma2(x2, ps, bcast2(kSinC3));
     const float2 sx = fma2(mul2(x, x2), ps, x);
-    float2 pc = fma2(x2, bcast2(-2.7557319223985891e-7f), bcast2(2.4801587301587302e-5f));
-    pc = fma2(x2, pc, bcast2(-1.3888888888888889e-3f));
-    pc = fma2(x2, pc, bcast2(4.1666666666666667e-2f));
+    float2 pc = fma2(x2, bcast2(kCosC8), bcast2(kCosC6));
+    pc = fma2(x2, pc, bcast2(kCosC4));
     pc = fma2(x2, pc, bcast2(-0.5f));
     const float2 cx = fma2(x2, pc, bcast2(1.0f));
     const int q0 = static_cast<int>(q.x) & 3, q1 = static_cast<int>(q.y) & 3;
