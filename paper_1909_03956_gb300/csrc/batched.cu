@@ -121,16 +121,17 @@ __global__ void __launch_bounds__(NT) k_batched(const BatchChan* __restrict__ ch
         bool good;
         if constexpr (KIND == kKindDF) {
             Eq17DF<NT, VPT> b;
+            F2 u[VPT], v[VPT], w[VPT];
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 const int64_t n = n0 + static_cast<int64_t>(k) * NT;
                 const bool ok = n < n_vis;
                 const double s = sgn * ch.scale;   // sign folded into B (exact negation)
-                b.u[k] = split_f64(ok ? uvw_m[3 * n] * s : 0.0);
-                b.v[k] = split_f64(ok ? uvw_m[3 * n + 1] * s : 0.0);
-                b.w[k] = split_f64(ok ? uvw_m[3 * n + 2] * s : 0.0);
-                b.vr[k] = b.vi[k] = b.lr[k] = b.li[k] = DF{0.f, 0.f};
+                u[k] = split_f64(ok ? uvw_m[3 * n] * s : 0.0);
+                v[k] = split_f64(ok ? uvw_m[3 * n + 1] * s : 0.0);
+                w[k] = split_f64(ok ? uvw_m[3 * n + 2] * s : 0.0);
             }
+            b.start(u, v, w);
             b.stk = reinterpret_cast<float4*>(stk_base) + threadIdx.x;
             b.tab = tab;
             b.J = ch.J;
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(NT) k_batched(const BatchChan* __restrict__ ch
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 const int64_t n = n0 + static_cast<int64_t>(k) * NT;
-                if (good && n < n_vis) out[n] = make_double2(df_to_double(b.vr[k]), df_to_double(b.vi[k]));
+                if (good && n < n_vis) out[n] = b.result(k);
             }
         } else if constexpr (KIND == kKindMixed) {
             float2* out = static_cast<float2*>(vis) + ch.out_offset;

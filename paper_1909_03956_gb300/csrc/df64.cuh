@@ -6,9 +6,9 @@
 // float64 pipe runs at a small fraction of its float32 rate). The building
 // blocks are the two error-free transforms: Knuth's two-sum (a + b = s + e
 // exactly) and the FMA product error (a b = p + e exactly, e = fma(a, b, -p)).
-// Sums and products are renormalised with Dekker's fast two-sum; the sum
-// drops the rounding error of the low parts' addition (absolute error below
-// 2^-47 of the operands), the product drops l_a l_b (below 2^-48 of it).
+// Sums gather the heads' rounding errors and the low parts in the low part and
+// are renormalised (Dekker's fast two-sum) after a few terms; a product drops
+// l_a l_b (below 2^-48 of it).
 #pragma once
 
 #include "wt_internal.cuh"
@@ -19,50 +19,18 @@ struct DF {
     float h, l;
 };
 
-__device__ __forceinline__ DF df_renorm(float s, float e)
-{
-    const float h = __fadd_rn(s, e);
-    return DF{h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-
-__device__ __forceinline__ DF df_add(DF a, DF b)
-{
-    float s, e;
-    two_sum(a.h, b.h, s, e);
-    return df_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
-}
-
-__device__ __forceinline__ DF df_add_f(DF a, float b)
-{
-    float s, e;
-    two_sum(a.h, b, s, e);
-    return df_renorm(s, __fadd_rn(e, a.l));
-}
-
-__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.h, -a.l}; }
-
-__device__ __forceinline__ DF df_mul(DF a, DF b)
-{
-    const float p = __fmul_rn(a.h, b.h);
-    const float e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
-    return df_renorm(p, e);
-}
-
 // times a power of two: exact
 __device__ __forceinline__ DF df_scale(DF a, float pow2) { return DF{__fmul_rn(a.h, pow2), __fmul_rn(a.l, pow2)}; }
 
 __device__ __forceinline__ double df_to_double(DF a) { return static_cast<double>(a.h) + static_cast<double>(a.l); }
 
-__device__ __forceinline__ DF df_from_double(double x)
-{
-    const float h = __double2float_rn(x);
-    return DF{h, __double2float_rn(x - static_cast<double>(h))};
-}
-
 // Sum of many double-floats: sum + x with the head's rounding error and the
 // low parts gathered in the low part, not renormalised. The head's sum is
 // error-free; the low part holds rounding errors and low parts only, so its
-// own rounding stays 2^-24 below theirs. Eight operations against df_add's 11.
+// own rounding stays 2^-24 below theirs as long as few terms gather there: a
+// long sum is renormalised (df_renorm) every few terms. Left alone over 10 000
+// terms, the low part's roundings doubled the error; renormalised at every term
+// a sum takes 11 operations, not eight.
 __device__ __forceinline__ void df_accumulate(DF& sum, float xh, float xl)
 {
     float s, e;
@@ -71,7 +39,14 @@ __device__ __forceinline__ void df_accumulate(DF& sum, float xh, float xl)
     sum.l = __fadd_rn(sum.l, __fadd_rn(e, xl));
 }
 
-// a b as an unevaluated p + e (df_mul without the renormalisation).
+__device__ __forceinline__ void df_renorm(DF& x)
+{
+    const float h = __fadd_rn(x.h, x.l);
+    x.l = __fsub_rn(x.l, __fsub_rn(h, x.h));
+    x.h = h;
+}
+
+// a b as an unevaluated p + e.
 __device__ __forceinline__ void df_product_raw(DF a, DF b, float& p, float& e)
 {
     p = __fmul_rn(a.h, b.h);
@@ -130,6 +105,124 @@ __device__ __forceinline__ void sincos_turns_df(float th, float tl, const float4
     df_accumulate(s, p, pe);
 }
 
+// ---- two visibilities at once -------------------------------------------------
+// The same operations on packed pairs, element 0 one visibility and element 1
+// another: the float32 pipe takes a pair every two cycles in one issue slot, so
+// half of them are left for the records, the table and the sweep (one
+// visibility at a time the double-float sums issued an instruction in 9 of 10
+// cycles). A pair cannot be negated for free, so products are formed with their
+// heads negated (from a factor that is kept negated) and subtracted.
+struct DFP {
+    float2 h, l;
+};
+
+__device__ __forceinline__ DFP dfp_zero() { return DFP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+
+// sum + (-nh + l), as df_accumulate.
+__device__ __forceinline__ void dfp_accumulate_neg(DFP& sum, float2 nh, float2 l)
+{
+    const float2 s = sub2(sum.h, nh);
+    const float2 bp = sub2(s, sum.h);                         // what of -nh arrived
+    const float2 e = sub2(sub2(sum.h, sub2(s, bp)), add2(nh, bp));
+    sum.h = s;
+    sum.l = add2(sum.l, add2(e, l));
+}
+
+// sum + x.
+__device__ __forceinline__ void dfp_accumulate(DFP& sum, const DFP& x)
+{
+    float2 s, e;
+    two_sum2(sum.h, x.h, s, e);
+    sum.h = s;
+    sum.l = add2(sum.l, add2(e, x.l));
+}
+
+// a b = -np + e, na = -a.h.
+__device__ __forceinline__ void dfp_product(const DFP& a, float2 na, const DFP& b, float2& np, float2& e)
+{
+    np = mul2(na, b.h);
+    e = fma2(a.h, b.l, fma2(a.l, b.h, fma2(a.h, b.h, np)));
+}
+
+__device__ __forceinline__ void dfp_renorm(DFP& x)
+{
+    const float2 h = add2(x.h, x.l);
+    x.l = sub2(x.l, sub2(h, x.h));
+    x.h = h;
+}
+
+// A factor common to both elements, with its negated head.
+struct DFS {
+    DFP v;
+    float2 nh;
+};
+__device__ __forceinline__ DFS dfs(float h, float l) { return DFS{DFP{bcast2(h), bcast2(l)}, bcast2(-h)}; }
+
+__device__ __forceinline__ void dfp_accumulate_product(DFP& sum, const DFS& a, const DFP& b)
+{
+    float2 np, e;
+    dfp_product(a.v, a.nh, b, np, e);
+    dfp_accumulate_neg(sum, np, e);
+}
+
+// phase_turns_df2 with the phase as th + tl.
+__device__ __forceinline__ void phase_turns_dfp(const DF2& u, const DF2& v, const DF2& w, F2 su, F2 sv, F2 sw1,
+                                                float2& th, float2& tl)
+{
+    float2 q1, t1, q2, t2, q3, t3, a, ea, b, eb;
+    df_product2n(u, su, q1, t1);
+    df_product2n(v, sv, q2, t2);
+    df_product2n(w, sw1, q3, t3);
+    two_sum2(q1, q2, a, ea);
+    two_sum2(a, q3, b, eb);
+    th = sub2(make_float2(rintf(b.x), rintf(b.y)), b);
+    tl = sub2(add2(add2(t1, t2), sub2(t3, ea)), eb);
+}
+
+// sincos_turns_df of two phases.
+__device__ __forceinline__ void sincos_turns_dfp(float2 th, float2 tl, const float4* __restrict__ tab, DFP& s, DFP& c)
+{
+    const float2 t = mul2(add2(th, tl), bcast2(1024.0f));
+    const float2 k = make_float2(rintf(t.x), rintf(t.y));
+    float2 fh, fl;
+    two_sum2(fma2(k, bcast2(-0.0009765625f), th), tl, fh, fl);
+    const float4 e0 = tab[static_cast<int>(k.x) & 1023], e1 = tab[static_cast<int>(k.y) & 1023];
+    const float2 xh = mul2(fh, bcast2(kTwoPiH)), nx = mul2(fh, bcast2(-kTwoPiH));
+    const float2 xe = fma2(fh, bcast2(kTwoPiL), fma2(fl, bcast2(kTwoPiH), fma2(fh, bcast2(kTwoPiH), nx)));
+    const float2 nq = mul2(nx, xh);                            // -x^2
+    const float2 qe = fma2(add2(xh, xh), xe, fma2(xh, xh, nq));
+    // sin x = x - x^3/6 + x^5/120, cos x - 1 = -x^2/2 + x^4/24
+    const DFP sx{xh, fma2(mul2(xh, nq), fma2(nq, bcast2(8.3333333333333333e-3f), bcast2(1.6666666666666667e-1f)), xe)};
+    const DFP cm{mul2(nq, bcast2(0.5f)),
+                 fma2(mul2(nq, nq), bcast2(4.1666666666666667e-2f), mul2(qe, bcast2(-0.5f)))};
+    const float2 ncm = mul2(nq, bcast2(-0.5f));
+    const DFP C{make_float2(e0.x, e1.x), make_float2(e0.y, e1.y)}, S{make_float2(e0.z, e1.z), make_float2(e0.w, e1.w)};
+    float2 np, e;
+    c = C;
+    dfp_product(sx, nx, S, np, e);                             // -S sin x: head np, low -e
+    {
+        float2 sum, err;
+        two_sum2(c.h, np, sum, err);
+        c.h = sum;
+        c.l = add2(c.l, sub2(err, e));
+    }
+    dfp_product(cm, ncm, C, np, e);
+    dfp_accumulate_neg(c, np, e);
+    s = S;
+    dfp_product(sx, nx, C, np, e);
+    dfp_accumulate_neg(s, np, e);
+    dfp_product(cm, ncm, S, np, e);
+    dfp_accumulate_neg(s, np, e);
+}
+
+__device__ __forceinline__ double2 dfp_vis(const DFP& re, const DFP& im, int k)
+{
+    return k == 0 ? make_double2(static_cast<double>(re.h.x) + static_cast<double>(re.l.x),
+                                 static_cast<double>(im.h.x) + static_cast<double>(im.l.x))
+                  : make_double2(static_cast<double>(re.h.y) + static_cast<double>(re.l.y),
+                                 static_cast<double>(im.h.y) + static_cast<double>(im.l.y));
+}
+
 constexpr int kDfTableEntries = 1024;
 
 static __device__ const float4 kSinCosDF[kDfTableEntries] =
@@ -140,7 +233,7 @@ static __device__ const float4 kSinCosDF[kDfTableEntries] =
 // the CTA's threads into shared memory.
 __device__ __forceinline__ void load_sincos_table_df(float4* tab)
 {
-#pragma unroll 4
+#pragma unroll 16
     for (int i = threadIdx.x; i < kDfTableEntries; i += blockDim.x) tab[i] = __ldg(&kSinCosDF[i]);
 }
 

@@ -133,23 +133,40 @@ struct BodyF2 {
     }
 };
 
-// The float64-class double-float form: one visibility per thread, every
-// step in double-float (df64.cuh).
+// The float64-class double-float form: two visibilities per thread (n and n +
+// NT of its tile) as a pair, every step in double-float (df64.cuh).
 struct BodyDF {
-    F2 u, v, w;
-    DF vr, vi;
+    DF2 U, V, W;
+    DFP vr, vi;
     const float4* tab;
-    __device__ void operator()(const CompF& c)
+    __device__ __forceinline__ void term(const CompF& c)
     {
-        float th, tl;
-        phase_turns_df(u, v, w, F2{c.lh, c.ll}, F2{c.mh, c.ml}, F2{c.nh, c.nl}, th, tl);
-        DF s, co;
-        sincos_turns_df(th, tl, tab, s, co);
-        const DF f{c.flux, c.flux_lo};
-        df_accumulate_product(vr, f, co);
-        df_accumulate_product(vi, f, s);
+        float2 th, tl;
+        phase_turns_dfp(U, V, W, F2{c.lh, c.ll}, F2{c.mh, c.ml}, F2{c.nh, c.nl}, th, tl);
+        DFP s, co;
+        sincos_turns_dfp(th, tl, tab, s, co);
+        const DFS f = dfs(c.flux, c.flux_lo);
+        dfp_accumulate_product(vr, f, co);
+        dfp_accumulate_product(vi, f, s);
+    }
+    // a block of components (kSumBlock, or what is left of a chunk), then the
+    // sums renormalised; returns how many
+    __device__ __forceinline__ int at(const CompF* cb, int r, int n)
+    {
+        int taken = kSumBlock;
+        if (r + kSumBlock <= n) {
+#pragma unroll 4
+            for (int j = 0; j < kSumBlock; ++j) term(cb[r + j]);
+        } else {
+            taken = n - r;
+            for (int j = r; j < n; ++j) term(cb[j]);
+        }
+        dfp_renorm(vr);
+        dfp_renorm(vi);
+        return taken;
     }
 };
+constexpr int kChunkDirDF = 128;   // records per staging buffer beside the 16 KB table
 
 // Few visibilities. A CTA per tile of visibilities leaves most SMs idle when
 // there are fewer tiles than SMs (one integration of 128 antennas, 8 128
@@ -197,26 +214,29 @@ __global__ void __launch_bounds__(NT) k_dft_df(const CompF* __restrict__ comps, 
     extern __shared__ __align__(16) unsigned char smem[];
     vis += blockIdx.y * n_vis;
     Stager<CompF> st;
-    stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunk);
-    float4* tab = reinterpret_cast<float4*>(smem + stager_bytes<CompF>(kChunk));
+    stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunkDirDF);
+    float4* tab = reinterpret_cast<float4*>(smem + stager_bytes<CompF>(kChunkDirDF));
     load_sincos_table_df(tab);
     __syncthreads();
-    const int64_t ntiles = (n_vis + NT - 1) / NT;
+    const int64_t ntiles = (n_vis + 2 * NT - 1) / (2 * NT);
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t n = tile * NT + threadIdx.x;
-        const bool valid = n < n_vis;
+        const int64_t n0 = tile * 2 * NT + threadIdx.x, n1 = n0 + NT;
+        const bool ok0 = n0 < n_vis, ok1 = n1 < n_vis;
+        auto pair = [&](int c) {   // sign folded into the baseline (exact)
+            return df2_pack(split_f64(ok0 ? sgn * uvw[3 * n0 + c] : 0.0), split_f64(ok1 ? sgn * uvw[3 * n1 + c] : 0.0));
+        };
         BodyDF b;
-        b.u = split_f64(valid ? sgn * uvw[3 * n] : 0.0);   // sign folded into the baseline (exact)
-        b.v = split_f64(valid ? sgn * uvw[3 * n + 1] : 0.0);
-        b.w = split_f64(valid ? sgn * uvw[3 * n + 2] : 0.0);
-        b.vr = DF{0.f, 0.f};
-        b.vi = DF{0.f, 0.f};
+        b.U = pair(0);
+        b.V = pair(1);
+        b.W = pair(2);
+        b.vr = b.vi = dfp_zero();
         b.tab = tab;
-        if (!st.sweep(b)) {
+        if (!st.sweep_at(b)) {
             if (threadIdx.x == 0) record_status(status, WT_ERR_TIMEOUT);
             return;
         }
-        if (valid) vis[n] = make_double2(df_to_double(b.vr), df_to_double(b.vi));
+        if (ok0) vis[n0] = dfp_vis(b.vr, b.vi, 0);
+        if (ok1) vis[n1] = dfp_vis(b.vr, b.vi, 1);
     }
 }
 
@@ -343,11 +363,13 @@ TermParts term_parts(int64_t tiles, int64_t n_terms, int fill)
 
 namespace {
 // The cut of a form's sum by the tiles of its main kernel: CTAs of 128 threads
-// (160 on the tensor cores), four to fill an SM, or of 256 (mixed), two.
+// (160 on the tensor cores), four to fill an SM; of 256 (mixed), two; of 64
+// (double-float), eight.
 TermParts dft_parts(int mode, int64_t n_vis, int64_t n_comp)
 {
     if (mode == WT_MIXED || mode == WT_MIXED_FAST) return term_parts((n_vis + 511) / 512, n_comp, 2);
-    return term_parts(mode == WT_MIXED_TC ? dft_tc_tiles(n_vis, n_comp) : (n_vis + 127) / 128, n_comp, 4);
+    return term_parts(mode == WT_MIXED_TC ? dft_tc_tiles(n_vis, n_comp) : (n_vis + 127) / 128, n_comp,
+                      mode == WT_FP64_DF ? 8 : 4);
 }
 }  // namespace
 
@@ -382,10 +404,10 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
         k<<<grid, NT, smem, s>>>(static_cast<const CompD*>(scratch), n_comp, tp.per_part, uvw, n_vis,
                                  static_cast<double2*>(vis), static_cast<double>(sign), status);
     } else if (mode == WT_FP64_DF) {
-        constexpr int NT = 128;
-        const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunk)) + kDfTableEntries * sizeof(float4);
+        constexpr int NT = 64;
+        const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunkDirDF)) + kDfTableEntries * sizeof(float4);
         auto k = k_dft_df<NT>;
-        int rc = grid_for(k, NT, NT, smem, n_vis, grid);
+        int rc = grid_for(k, NT, 2 * NT, smem, n_vis, grid);
         if (rc) return rc;
         grid.y = static_cast<unsigned>(tp.parts);
         k<<<grid, NT, smem, s>>>(static_cast<const CompF*>(scratch), n_comp, tp.per_part, uvw, n_vis,

@@ -141,20 +141,18 @@ __global__ void __launch_bounds__(NT) k_wavelet_df(const RecWDF* __restrict__ re
         const int64_t n0 = tile * per_tile + threadIdx.x;
         using Body = typename std::conditional<SUM == 1, Eq16DF<VPT>, Eq17DF<NT, VPT>>::type;
         Body b;
+        F2 u[VPT], v[VPT], w[VPT];
 #pragma unroll
         for (int k = 0; k < VPT; ++k) {
             const int64_t n = n0 + static_cast<int64_t>(k) * NT;
             const bool ok = n < n_vis;
-            b.u[k] = split_f64(ok ? sgn * uvw[3 * n] : 0.0);   // sign folded in (exact)
-            b.v[k] = split_f64(ok ? sgn * uvw[3 * n + 1] : 0.0);
-            b.w[k] = split_f64(ok ? sgn * uvw[3 * n + 2] : 0.0);
-            b.vr[k] = DF{0.f, 0.f};
-            b.vi[k] = DF{0.f, 0.f};
+            u[k] = split_f64(ok ? sgn * uvw[3 * n] : 0.0);   // sign folded in (exact)
+            v[k] = split_f64(ok ? sgn * uvw[3 * n + 1] : 0.0);
+            w[k] = split_f64(ok ? sgn * uvw[3 * n + 2] : 0.0);
         }
+        b.start(u, v, w);
         b.tab = tab;
         if constexpr (SUM != 1) {
-#pragma unroll
-            for (int k = 0; k < VPT; ++k) b.lr[k] = b.li[k] = DF{0.f, 0.f};
             b.stk = stk;
             b.J = J;
             b.maxrow = rows - 1;
@@ -166,7 +164,7 @@ __global__ void __launch_bounds__(NT) k_wavelet_df(const RecWDF* __restrict__ re
 #pragma unroll
         for (int k = 0; k < VPT; ++k) {
             const int64_t n = n0 + static_cast<int64_t>(k) * NT;
-            if (n < n_vis) vis[n] = make_double2(df_to_double(b.vr[k]), df_to_double(b.vi[k]));
+            if (n < n_vis) vis[n] = b.result(k);
         }
     }
 }
