@@ -347,11 +347,11 @@ __global__ void k_w2_to_bf16(const float* __restrict__ params, uint32_t* __restr
 
 // ---------------------------------------------------------------- training
 constexpr int kTrainThreads = 256;
-constexpr int kS = 64;          // samples per CTA tile
 constexpr int kLdB = kH + 8;    // row stride of the bfloat16 operands: the 8 rows of an ldmatrix in distinct banks
 constexpr int kLdF = kH + 4;    // row stride of the float32 ones
 
-// Shared memory of a tile, 84 KB: two CTAs per SM.
+// Shared memory of a tile of S samples, 84 KB for 64: two CTAs per SM.
+template <int kS>
 struct TrainSmem {
     __nv_bfloat16 w2[kH][kLdB];        // W2[o][k], rounded
     __nv_bfloat16 h1[kS][kLdB];        // h1[s][k], rounded
@@ -361,7 +361,7 @@ struct TrainSmem {
     float W1[kH * 3], b1[kH], b2[kH], W3[2 * kH], b3[2];
     float x[kS][3];
     float t[kS][2];
-    float ypart[2][kS][2];             // the output's sums over each half of the hidden units
+    float ypart[128 / kS][kS][2];      // the output's sums over each block of the hidden units
     float dy[kS][2];
     float valid[kS];
     float e2[kS][2];                   // squared errors of the current samples
@@ -406,19 +406,21 @@ __device__ __forceinline__ void silu_both(float z, float& h, float& d)
     d = s * (1.0f + z * (1.0f - s));
 }
 
-// Forward and backward over a batch, 64 samples per CTA tile. The three
-// 64 x 64 x 64 products of a tile (z2 = h1 W2^T, dh1 = dz2 W2, gW2 = dz2^T h1)
+// Forward and backward over a batch, kS samples per CTA tile (64, or 32 where
+// that gives every SM two CTAs at most: see run_grad). The three kS x 64 x 64
+// products of a tile (z2 = h1 W2^T, dh1 = dz2 W2, gW2 = dz2^T h1)
 // run on the tensor cores: h1 and W2 are bfloat16 by definition, and dz2
 // enters as three bfloat16 that sum to it exactly, so every product is exact
 // and the sums are float32, as on the FMA pipe. A tile's products are too
 // small (2 MFLOP) for a tensor-memory accumulator's round trips to pay;
-// m16n8k16 fragments keep a warp's 16 x 32 block of every activation in its
+// m16n8k16 fragments keep a warp's 16-row block of every activation in its
 // registers from the forward to the backward pass. Bound by the chain of small
 // dependent steps (two warps per scheduler, issue 23 % active): at 8 192 samples
 // (128 tiles on 152 SMs) 11.6 us, against 62 us with the products on the FMA
 // pipe an element per thread from shared memory, 16.9 us with 4 x 4 register
 // blocks there (bound by their 16-byte shared-memory loads); a training step
 // with k_mlp_adam 73 -> 14.9 us.
+template <int kS>
 __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float* __restrict__ params,
                                                                      const double* __restrict__ uvw,
                                                                      const float* __restrict__ target, int64_t first,
@@ -426,12 +428,15 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
                                                                      float scale, float* __restrict__ part)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smem_raw);
+    TrainSmem<kS>& sm = *reinterpret_cast<TrainSmem<kS>*>(smem_raw);
+    constexpr int kCB = 128 / kS;      // column blocks of the activations: 8 warps over kS / 16 row blocks
+    constexpr int kNB = kH / kCB / 8;  // of kNB times 8 units each
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t2 = 2 * (lane & 3);
-    // this warp's block of every 64 x 64 product: rows r0 .. r0 + 15 (samples,
-    // or units o of gW2), columns c0 .. c0 + 31 in four blocks of 8
-    const int r0 = 16 * (warp >> 1), c0 = 32 * (warp & 1);
+    // this warp's block of the activations: samples r0 .. r0 + 15, units c0 ..
+    // in kNB blocks of 8; of gW2: units o0 .. o0 + 15 by k0 .. k0 + 31
+    const int cb = warp % kCB, r0 = 16 * (warp / kCB), c0 = 8 * kNB * cb;
+    const int o0 = 16 * (warp >> 1), k0 = 32 * (warp & 1);
     // the first tile's sample of this thread (tid < 64), in flight while the
     // weights are staged; later tiles' likewise, one tile ahead
     float nx[3] = {0.f, 0.f, 0.f}, nt[2] = {0.f, 0.f}, nvalid = 0.f;
@@ -485,14 +490,14 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
         __syncthreads();
         // layer 1: element (i, j) of a fragment is row r0 + g + 8 (j / 2),
         // column c0 + 8 i + t2 + j % 2
-        float ds1[4][4];
+        float ds1[kNB][4];
         {
             float x[2][3];
 #pragma unroll
             for (int e = 0; e < 2; ++e)
                 for (int d = 0; d < 3; ++d) x[e][d] = sm.x[r0 + g + 8 * e][d];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kNB; ++i) {
                 float h[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -508,11 +513,11 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
         }
         __syncthreads();
         // layer 2, and this warp's half of layer 3
-        float ds2[4][4];
+        float ds2[kNB][4];
         {
-            float z[4][4];
+            float z[kNB][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kNB; ++i) {
                 const float2 b = *reinterpret_cast<const float2*>(&sm.b2[c0 + 8 * i + t2]);
                 z[i][0] = z[i][2] = b.x;
                 z[i][1] = z[i][3] = b.y;
@@ -522,7 +527,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
                 uint32_t a[4];
                 ldsm_x4(&sm.h1[r0 + (lane & 15)][kk + 8 * (lane >> 4)], a);
 #pragma unroll
-                for (int i = 0; i < 4; i += 2) {
+                for (int i = 0; i < kNB; i += 2) {
                     uint32_t b[4];
                     ldsm_x4(&sm.w2[c0 + 8 * i + (lane & 7) + 8 * (lane >> 4)][kk + 8 * ((lane >> 3) & 1)], b);
                     mma_bf16(z[i], a, b[0], b[1]);
@@ -531,7 +536,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
             }
             float y[2][2] = {{0.f, 0.f}, {0.f, 0.f}};   // [row][output]
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kNB; ++i) {
                 const int c = c0 + 8 * i + t2;
                 const float2 wa = *reinterpret_cast<const float2*>(&sm.W3[c]);
                 const float2 wb = *reinterpret_cast<const float2*>(&sm.W3[kH + c]);
@@ -551,7 +556,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
                 for (int o = 0; o < 2; ++o) {
                     y[e][o] += __shfl_xor_sync(0xffffffffu, y[e][o], 1);
                     y[e][o] += __shfl_xor_sync(0xffffffffu, y[e][o], 2);
-                    if ((lane & 3) == 0) sm.ypart[warp & 1][r0 + g + 8 * e][o] = y[e][o];
+                    if ((lane & 3) == 0) sm.ypart[cb][r0 + g + 8 * e][o] = y[e][o];
                 }
         }
         __syncthreads();
@@ -563,16 +568,18 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
 #pragma unroll
                 for (int o = 0; o < 2; ++o) {
                     const int s = r0 + g + 8 * e;
-                    const float y = sm.b3[o] + sm.ypart[0][s][o] + sm.ypart[1][s][o];
+                    float y = sm.b3[o];
+#pragma unroll
+                    for (int q = 0; q < kCB; ++q) y += sm.ypart[q][s][o];
                     const float err = (sm.valid[s] != 0.f) ? y - sm.t[s][o] : 0.f;
                     dy[e][o] = 2.f * err * inv_n;
-                    if ((warp & 1) == 0 && (lane & 3) == 0) {
+                    if (cb == 0 && (lane & 3) == 0) {
                         sm.e2[s][o] = err * err;
                         sm.dy[s][o] = dy[e][o];
                     }
                 }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kNB; ++i) {
                 const int c = c0 + 8 * i + t2;
                 const float2 wa = *reinterpret_cast<const float2*>(&sm.W3[c]);
                 const float2 wb = *reinterpret_cast<const float2*>(&sm.W3[kH + c]);
@@ -593,30 +600,42 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
             }
         }
         __syncthreads();
-        // gW2 (rows o, columns k, summed over the samples) and dh1
-        float dh[4][4];
+        // gW2 (rows o, columns k, summed over the samples), then dh1; of each
+        // product's three parts the small ones first
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int kk = 0; kk < kS; kk += 16) {
+            uint32_t bh[2][4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) dh[i][j] = 0.f;
+            for (int i = 0; i < 2; ++i)
+                ldsm_x4_t(&sm.h1[kk + (lane & 7) + 8 * ((lane >> 3) & 1)][k0 + 16 * i + 8 * (lane >> 4)], bh[i]);
 #pragma unroll
-        for (int kk = 0; kk < kH; kk += 16) {
-            uint32_t bh[2][4], bw[2][4];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int rr = kk + (lane & 7) + 8 * ((lane >> 3) & 1), cc = c0 + 16 * i + 8 * (lane >> 4);
-                ldsm_x4_t(&sm.h1[rr][cc], bh[i]);
-                ldsm_x4_t(&sm.w2[rr][cc], bw[i]);
-            }
-#pragma unroll
-            for (int q = 2; q >= 0; --q) {   // the small parts first
-                uint32_t at[4], ad[4];
-                ldsm_x4_t(&sm.dz2b[q][kk + (lane & 7) + 8 * (lane >> 4)][r0 + 8 * ((lane >> 3) & 1)], at);
-                ldsm_x4(&sm.dz2b[q][r0 + (lane & 15)][kk + 8 * (lane >> 4)], ad);
+            for (int q = 2; q >= 0; --q) {
+                uint32_t at[4];
+                ldsm_x4_t(&sm.dz2b[q][kk + (lane & 7) + 8 * (lane >> 4)][o0 + 8 * ((lane >> 3) & 1)], at);
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     mma_bf16(gW2[2 * i], at, bh[i][0], bh[i][1]);
                     mma_bf16(gW2[2 * i + 1], at, bh[i][2], bh[i][3]);
+                }
+            }
+        }
+        float dh[kNB][4];
+#pragma unroll
+        for (int i = 0; i < kNB; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dh[i][j] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < kH; kk += 16) {
+            uint32_t bw[kNB / 2][4];
+#pragma unroll
+            for (int i = 0; i < kNB / 2; ++i)
+                ldsm_x4_t(&sm.w2[kk + (lane & 7) + 8 * ((lane >> 3) & 1)][c0 + 16 * i + 8 * (lane >> 4)], bw[i]);
+#pragma unroll
+            for (int q = 2; q >= 0; --q) {
+                uint32_t ad[4];
+                ldsm_x4(&sm.dz2b[q][r0 + (lane & 15)][kk + 8 * (lane >> 4)], ad);
+#pragma unroll
+                for (int i = 0; i < kNB / 2; ++i) {
                     mma_bf16(dh[2 * i], ad, bw[i][0], bw[i][1]);
                     mma_bf16(dh[2 * i + 1], ad, bw[i][2], bw[i][3]);
                 }
@@ -646,7 +665,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < kNB; ++i)
 #pragma unroll
             for (int e = 0; e < 2; ++e)
                 *reinterpret_cast<float2*>(&sm.dz2[r0 + g + 8 * e][c0 + 8 * i + t2]) =
@@ -674,7 +693,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int e = 0; e < 2; ++e)
-            *reinterpret_cast<float2*>(row + oW2 + (r0 + g + 8 * e) * kH + c0 + 8 * i + t2) =
+            *reinterpret_cast<float2*>(row + oW2 + (o0 + g + 8 * e) * kH + k0 + 8 * i + t2) =
                 make_float2(gW2[i][2 * e], gW2[i][2 * e + 1]);
     row[tid < kH * 3 ? oW1 + tid : ob1 + tid - kH * 3] = g1;
     if (tid < 2 * kH) row[oW3 + tid] = g23;
@@ -685,40 +704,31 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
 static_assert(oW2 % 4 == 0 && kPartStride % 4 == 0, "16-byte rows of the partial gradients");
 
 // Column sums of the partial rows: a CTA takes 32 columns (one 128-byte line
-// of every row), its 8 warps the rows of a block of 128 into shared memory at
-// once, and the first warp adds each column in row order; returns the sum of
-// column 32 blockIdx.x + threadIdx.x in the first warp. Latency bound: every
-// load of a block is in flight together (a thread per column walking the rows
-// 16 at a time: 9.0 us against 4.9 for 128 rows).
-constexpr int kRedThreads = 256, kRedRows = 128;
+// of every row), each of its 8 warps a contiguous eighth of the rows, its loads
+// 16 at a time, and the first warp adds the eighths in order: the sum of column
+// 32 blockIdx.x + threadIdx.x in the first warp. Latency bound (a thread per
+// column walking all rows: 9.0 us against 4.9 for 128 rows).
+constexpr int kRedThreads = 256;
 
 __device__ __forceinline__ float sum_rows(const float* __restrict__ part, int rows)
 {
-    __shared__ float buf[kRedRows][32];
+    __shared__ float buf[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int col = blockIdx.x * 32 + lane;
+    const int col = min(blockIdx.x * 32 + lane, kNumParams);
+    const int per = (rows + 7) / 8, end = min(rows, (warp + 1) * per);
     float a = 0.f;
-    for (int r0 = 0; r0 < rows; r0 += kRedRows) {
-        float v[kRedRows / 8];
+    for (int r = warp * per; r < end; r += 16) {
+        float v[16];
 #pragma unroll
-        for (int k = 0; k < kRedRows / 8; ++k) {
-            const int r = r0 + 8 * k + warp;
-            v[k] = r < rows && col <= kNumParams ? part[static_cast<int64_t>(r) * kPartStride + col] : 0.f;
-        }
+        for (int k = 0; k < 16; ++k) v[k] = r + k < end ? part[static_cast<int64_t>(r + k) * kPartStride + col] : 0.f;
 #pragma unroll
-        for (int k = 0; k < kRedRows / 8; ++k) buf[8 * k + warp][lane] = v[k];
-        __syncthreads();
-        if (warp == 0) {
-            const int n = min(kRedRows, rows - r0);
-            if (n == kRedRows) {
-#pragma unroll 32
-                for (int r = 0; r < kRedRows; ++r) a += buf[r][lane];
-            } else {
-                for (int r = 0; r < n; ++r) a += buf[r][lane];
-            }
-        }
-        __syncthreads();
+        for (int k = 0; k < 16; ++k) a += v[k];
     }
+    buf[warp][lane] = a;
+    __syncthreads();
+    a = buf[0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) a += buf[w][lane];
     return a;
 }
 constexpr int kRedBlocks = (kNumParams + 1 + 31) / 32;
@@ -855,17 +865,22 @@ int run_grad(wt_mlp m, const double* uvw, const float* target, int64_t first, in
              bool pdl, int* rows, cudaStream_t s)
 {
     using namespace wt;
-    const size_t smem = sizeof(TrainSmem);
-    WT_CUDA_TRY(cudaFuncSetAttribute(k_mlp_train_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem)));
+    // tiles of 32 samples where they give an SM two CTAs at most, all resident
+    // (8 192 samples: 256 tiles, a step 11.9 us against 14.9 with 128 tiles
+    // of 64, whose warps have twice the elementwise work); else of 64, whose
+    // barriers and weights serve twice the samples
+    const int64_t two_per_sm = static_cast<int64_t>(num_sms()) * 2;
+    const bool fine = (count + 31) / 32 <= two_per_sm;
+    auto kernel = fine ? k_mlp_train_grad<32> : k_mlp_train_grad<64>;
+    const size_t smem = fine ? sizeof(TrainSmem<32>) : sizeof(TrainSmem<64>);
+    WT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     const float scale = static_cast<float>(ldexp(sqrt(kPi / 3.0), 1 - m->level));
-    int64_t blocks = (count + kS - 1) / kS;
-    const int64_t cap = static_cast<int64_t>(num_sms()) * 2;
-    if (blocks > cap) blocks = cap;
+    int64_t blocks = fine ? (count + 31) / 32 : (count + 63) / 64;
+    if (blocks > two_per_sm) blocks = two_per_sm;
     if (blocks < 1) blocks = 1;
     if (blocks > m->part_rows) blocks = m->part_rows;
-    WT_CUDA_TRY(launch_step(k_mlp_train_grad, static_cast<unsigned>(blocks), kTrainThreads, smem, pdl, s, m->params,
-                            uvw, target, first, count, count, n_data, scale, m->part));
+    WT_CUDA_TRY(launch_step(kernel, static_cast<unsigned>(blocks), kTrainThreads, smem, pdl, s, m->params, uvw, target,
+                            first, count, count, n_data, scale, m->part));
     *rows = static_cast<int>(blocks);
     return WT_OK;
 }
