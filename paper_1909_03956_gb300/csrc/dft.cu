@@ -36,8 +36,8 @@ struct CompD {
 static_assert(sizeof(CompD) == 32, "component record layout");
 
 // n - 1 = -(l^2 + m^2) / (1 + sqrt(1 - l^2 - m^2)), free of cancellation.
-// bound (float records only; zeroed before the launch): the largest |l|,
-// |m|, |n - 1| of the float32 heads as float bit patterns (non-negative
+// bound (float records only; zeroed before the launch, its fourth word the
+// flag of deferred tiles): the largest |l|, |m|, |n - 1| of the float32 heads as float bit patterns (non-negative
 // floats order as their bits), reduced per warp, then by atomicMax; a
 // component that fails the range check adds nothing.
 __global__ void k_pack_components(const double* __restrict__ l, const double* __restrict__ m,
@@ -275,6 +275,9 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
                                                   float2* __restrict__ vis, float sgn, int* status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    if constexpr (!GRIDPASS) {
+        if (!any_deferred(reinterpret_cast<const float*>(bound))) return;
+    }
     vis += blockIdx.y * n_vis;
     Stager<CompF> st;
     stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunk);
@@ -312,7 +315,7 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
             return;
         }
         if (defer) {
-            mark_deferred(first_vis);
+            mark_deferred(first_vis, reinterpret_cast<const float*>(bound));
             continue;
         }
         if (ok0) vis[n0] = sub2(b.acc[0], b.comp[0]);
@@ -428,7 +431,7 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
         float2* out = static_cast<float2*>(vis);
         kg<<<grid, NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign), status);
         WT_CUDA_TRY(cudaGetLastError());
-        ke<<<grid_e, NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign),
+        ke<<<exact_grid(grid_e), NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign),
                                     status);
     }
     WT_CUDA_TRY(cudaGetLastError());
@@ -449,7 +452,7 @@ int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, 
     int rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid);
     if (rc) return rc;
     grid.y = static_cast<unsigned>(tp.parts);
-    ke<<<grid, NT, smem, s>>>(static_cast<const CompF*>(recs), n_comp, tp.per_part, bound, uvw, n_vis, vis,
+    ke<<<exact_grid(grid), NT, smem, s>>>(static_cast<const CompF*>(recs), n_comp, tp.per_part, bound, uvw, n_vis, vis,
                               static_cast<float>(sign), status);
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;

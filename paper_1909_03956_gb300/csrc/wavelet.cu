@@ -191,6 +191,9 @@ __global__ void __launch_bounds__(NT, (mixed_min_blocks<NT, VPT, SUM>())) k_wave
                                                       float2* __restrict__ vis, float sgn, int rows, int J,
                                                       int* status)
 {
+    if constexpr (!GRIDPASS) {
+        if (!any_deferred(hdr->smax)) return;
+    }
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int kChunk = (SUM == 1) ? kChunkF : kChunkW;
     Stager<Rec> st;
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(NT, (mixed_min_blocks<NT, VPT, SUM>())) k_wave
             return;
         }
         if (defer) {
-            mark_deferred(vis + tile * per_tile);
+            mark_deferred(vis + tile * per_tile, hdr->smax);
             continue;
         }
 #pragma unroll
@@ -397,7 +400,7 @@ int run_mixed_form(const WaveletJob& jb, cudaStream_t s)
         if ((rc = prepare(ke, NT, smem, int64_t(NT) * VPT, jb.n_vis, grid_e))) return rc;
         kg<<<grid, NT, smem, s>>>(jb.recf_leaf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
         WT_CUDA_TRY(cudaGetLastError());
-        ke<<<grid_e, NT, smem, s>>>(jb.recf_leaf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
+        ke<<<exact_grid(grid_e), NT, smem, s>>>(jb.recf_leaf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
     } else if (jb.which == WT_SUM_EQ17) {
         // the grid pass, then the exact pass over the tiles it left marked
         auto kg = k_wavelet_mixed<NT, VPT, 0, RecF, FAST, true>;
@@ -407,7 +410,7 @@ int run_mixed_form(const WaveletJob& jb, cudaStream_t s)
         if ((rc = prepare(ke, NT, smem, int64_t(NT) * VPT, jb.n_vis, grid_e))) return rc;
         kg<<<grid, NT, smem, s>>>(jb.recf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
         WT_CUDA_TRY(cudaGetLastError());
-        ke<<<grid_e, NT, smem, s>>>(jb.recf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
+        ke<<<exact_grid(grid_e), NT, smem, s>>>(jb.recf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
     } else {
         // the grid pass, then the exact pass over the tiles it left marked
         auto kg = k_wavelet_mixed<NT, VPT, 2, RecWF, FAST, true>;
@@ -417,7 +420,7 @@ int run_mixed_form(const WaveletJob& jb, cudaStream_t s)
         if ((rc = prepare(ke, NT, smem, int64_t(NT) * VPT, jb.n_vis, grid_e))) return rc;
         kg<<<grid, NT, smem, s>>>(jb.recwf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
         WT_CUDA_TRY(cudaGetLastError());
-        ke<<<grid_e, NT, smem, s>>>(jb.recwf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
+        ke<<<exact_grid(grid_e), NT, smem, s>>>(jb.recwf, jb.hdr, jb.uvw, jb.n_vis, out, sg, rows, jb.J, jb.status);
     }
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;

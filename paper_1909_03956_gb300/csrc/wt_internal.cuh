@@ -388,7 +388,11 @@ __device__ __forceinline__ float phase_bound(F2 u, F2 v, F2 w, const float* smax
 // both parts of its first visibility and is left to the exact pass, which
 // evaluates only tiles so marked, with error-free sums (phase_turns_df2).
 // The two kernels are launched back to back on one stream; kept apart, each
-// stays within its register budget.
+// stays within its register budget. Marking a tile also sets a flag (a word
+// beside the bounds smax, cleared where they are made and never after), and
+// while it is clear the exact pass returns at once: without it, reading every
+// tile's mark took 115 us for 125 000 tiles. A flag left by an earlier call on
+// the same tree only means that the marks are read.
 constexpr uint32_t kDeferredMark = 0x7fc4b1d3u;   // a quiet NaN
 
 // Grid constants of a thread's visibilities and the CTA's vote on whether
@@ -423,10 +427,20 @@ __device__ __forceinline__ bool tile_deferred(const float2* first_vis)
     return s_deferred != 0;
 }
 
-__device__ __forceinline__ void mark_deferred(float2* first_vis)
+__device__ __forceinline__ void mark_deferred(float2* first_vis, const float* smax)
 {
-    if (threadIdx.x == 0) *first_vis = make_float2(__uint_as_float(kDeferredMark), __uint_as_float(kDeferredMark));
+    if (threadIdx.x == 0) {
+        *first_vis = make_float2(__uint_as_float(kDeferredMark), __uint_as_float(kDeferredMark));
+        *reinterpret_cast<volatile float*>(const_cast<float*>(smax) + 3) = 1.0f;
+    }
 }
+__device__ __forceinline__ bool any_deferred(const float* smax)
+{
+    return *reinterpret_cast<const volatile float*>(smax + 3) != 0.0f;
+}
+// CTAs of an exact pass over `tiles` tiles: they stride beyond this many per
+// SM, so that a pass with nothing to do stays short.
+constexpr int kExactCtasPerSm = 128;
 
 // sincos_turns_f32 of the phase tl - h (turns) of two visibilities, each
 // result written as the pair (cos, sin) of its own visibility: e0 for
@@ -630,7 +644,8 @@ struct TreeHeader {
     int64_t per_level[kMaxJ + 1];   // [j] = nodes at level j (index 0 unused)
     int64_t rev_offset[kMaxJ + 2];  // start of level j in the level-J-first layout
     float smax[4];                  // max over the leaves of |s_u|, |s_v|, |s_w - 1| as the float32
-                                    // heads of their records (0 for an empty tree); [3] unused
+                                    // heads of their records (0 for an empty tree); [3] the flag of
+                                    // deferred tiles (any_deferred)
 };
 
 struct TreeDev {
@@ -749,5 +764,11 @@ int predict_dft(const double* l, const double* m, const double* flux, int64_t n_
 int subtract(const void* obs, const void* model, void* resid, int64_t n_vis, int mode, cudaStream_t s);
 // utilities
 int num_sms();
+inline dim3 exact_grid(dim3 grid)
+{
+    const unsigned most = static_cast<unsigned>(num_sms()) * kExactCtasPerSm;
+    if (grid.x > most) grid.x = most;
+    return grid;
+}
 void rotation_matrix(double ra0, double dec0, double* R);
 }  // namespace wt
