@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(NT) k_batched(const BatchChan* __restrict__ ch
             float2* out = static_cast<float2*>(vis) + ch.out_offset;
             float2* first_vis = out + (item - ch.tile_base) * per_tile;
             if constexpr (!GRIDPASS) {
-                if (!any_deferred(ch.hdr->smax) || !tile_deferred(first_vis)) continue;   // done by the grid pass
+                if (!tile_deferred(first_vis)) continue;   // done by the grid pass
             }
             F2 U[VPT], V[VPT], W[VPT];
 #pragma unroll
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(NT) k_batched(const BatchChan* __restrict__ ch
             } else {
                 good = sweep_regrouped_mixed<NT, VPT, FAST, false, false>(st, U, V, W, C, rstk, ch.J, maxrow, res);
             }
-            if (good && defer) mark_deferred(first_vis, ch.hdr->smax);
+            if (good && defer) mark_deferred(first_vis);
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
                 const int64_t n = n0 + static_cast<int64_t>(k) * NT;

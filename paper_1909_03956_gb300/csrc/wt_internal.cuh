@@ -392,7 +392,9 @@ __device__ __forceinline__ float phase_bound(F2 u, F2 v, F2 w, const float* smax
 // beside the bounds smax, cleared where they are made and never after), and
 // while it is clear the exact pass returns at once: without it, reading every
 // tile's mark took 115 us for 125 000 tiles. A flag left by an earlier call on
-// the same tree only means that the marks are read.
+// the same tree only means that the marks are read. (The batched kernel sets no
+// flag: its bounds are a channel's, and keeping their address over the sweep
+// cost it 19 %.)
 constexpr uint32_t kDeferredMark = 0x7fc4b1d3u;   // a quiet NaN
 
 // Grid constants of a thread's visibilities and the CTA's vote on whether
@@ -427,12 +429,14 @@ __device__ __forceinline__ bool tile_deferred(const float2* first_vis)
     return s_deferred != 0;
 }
 
+__device__ __forceinline__ void mark_deferred(float2* first_vis)
+{
+    if (threadIdx.x == 0) *first_vis = make_float2(__uint_as_float(kDeferredMark), __uint_as_float(kDeferredMark));
+}
 __device__ __forceinline__ void mark_deferred(float2* first_vis, const float* smax)
 {
-    if (threadIdx.x == 0) {
-        *first_vis = make_float2(__uint_as_float(kDeferredMark), __uint_as_float(kDeferredMark));
-        *reinterpret_cast<volatile float*>(const_cast<float*>(smax) + 3) = 1.0f;
-    }
+    mark_deferred(first_vis);
+    if (threadIdx.x == 0) *reinterpret_cast<volatile float*>(const_cast<float*>(smax) + 3) = 1.0f;
 }
 __device__ __forceinline__ bool any_deferred(const float* smax)
 {
