@@ -111,7 +111,7 @@ int choose_wavelet_variant(wt_tree t, const WaveletJob& jb, cudaStream_t s)
         const int v = atoi(pin);
         if (wavelet_variant_fits(v, jb.mode, jb.which, jb.J)) return v;
     }
-    if (!tuning_enabled()) return fallback;
+    if (!tuning_enabled() || wavelet_untuned(jb.mode, jb.which, jb.J)) return fallback;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
         cudaGetLastError();

@@ -319,6 +319,30 @@ int prepare(K kernel, int nt, size_t smem, int64_t per_tile, int64_t n_vis, dim3
     return WT_OK;
 }
 
+// Resident CTAs per SM for tiles of 64 threads whose every warp keeps the
+// float64 pipe busy for the whole sweep. All the tiles take alike, so they run
+// in waves of SMs x resident CTAs and a wave's time goes with its CTAs per SM:
+// the last one, however few tiles are left to it, costs as much as the others.
+// More CTAs hide latency (a wave's time per CTA, measured: 1.09, 1.035 and 1 at
+// two, three and four), fewer make finer waves; the count with the smallest
+// product. 201 563 visibilities (3 150 tiles; J = 12): four CTAs 13.6 ms in six
+// waves, three 12.3 in seven.
+int fp64_resident(int64_t tiles, int most)
+{
+    static const double per_cta[] = {0.0, 2.04, 1.088, 1.035, 1.0};
+    int best = most;
+    double least = 1e300;
+    for (int r = most < 4 ? most : 4; r >= 1; --r) {
+        const int64_t wave = static_cast<int64_t>(num_sms()) * r;
+        const double time = static_cast<double>((tiles + wave - 1) / wave * r) * per_cta[r];
+        if (time < least) {
+            least = time;
+            best = r;
+        }
+    }
+    return best;
+}
+
 // Shared-memory stack rows a form needs for a tree of depth J.
 int stack_rows(int mode, int which, int J)
 {
@@ -344,7 +368,15 @@ int run_fp64(const WaveletJob& jb, cudaStream_t s)
 {
     const int rows = stack_rows(WT_FP64, jb.which, jb.J);
     const size_t stack = static_cast<size_t>(rows) * VPT * NT * sizeof(double2);
-    const size_t smem = stage_bytes(WT_FP64, jb.which) + stack;
+    size_t smem = stage_bytes(WT_FP64, jb.which) + stack;
+    if (jb.which == WT_SUM_EQ17 && NT == 64 && VPT == 1) {
+        // as many CTAs per SM as fp64_resident says, by the shared memory each takes
+        constexpr size_t kSmem = 227 * 1024, kReserve = 1024;
+        const int most = static_cast<int>(kSmem / (smem + kReserve));
+        const int r = fp64_resident((jb.n_vis + NT - 1) / NT, most < 1 ? 1 : most);
+        const size_t share = (kSmem / static_cast<size_t>(r) - kReserve) & ~size_t(15);
+        if (share > smem) smem = share;
+    }
     dim3 grid;
     int rc;
     double2* out = static_cast<double2*>(jb.vis);
@@ -437,9 +469,13 @@ int run_mixed(const WaveletJob& jb, cudaStream_t s)
 // Launch-shape variants (threads per CTA, visibilities per thread). Which
 // one runs is chosen per (form, sum, J, tree size) by the autotuner, or by
 // stack_fits() when no tuning is available.
-const int kNumWaveletVariants = 8;
-static const Variant kVariants[kNumWaveletVariants] = {{256, 1}, {128, 1}, {128, 2}, {64, 2},
-                                                       {64, 4},  {32, 4},  {32, 2},  {256, 2}};
+// The last one is the explicit float64 sum's, which takes it without tuning
+// wherever it fits: its waves depend on the batch (fp64_resident), not on a
+// sample.
+const int kNumWaveletVariants = 9;
+static const Variant kVariants[kNumWaveletVariants] = {{256, 1}, {128, 1}, {128, 2}, {64, 2}, {64, 4},
+                                                       {32, 4},  {32, 2},  {256, 2}, {64, 1}};
+constexpr int kVariantF64 = 8;
 
 int wavelet_variant_shape(int v, int* nt, int* vpt)
 {
@@ -463,6 +499,7 @@ size_t wavelet_variant_smem(int v, int mode, int which, int J)
 bool wavelet_variant_fits(int v, int mode, int which, int J)
 {
     if (v < 0 || v >= kNumWaveletVariants) return false;
+    if (v == kVariantF64 && !(mode == WT_FP64 && which == WT_SUM_EQ17)) return false;
     return wavelet_variant_smem(v, mode, which, J) <= 220 * 1024;
 }
 
@@ -491,7 +528,8 @@ int launch_wavelet(const WaveletJob& jb, int v, cudaStream_t s)
             case 4: return run_fp64<64, 4>(jb, s);
             case 5: return run_fp64<32, 4>(jb, s);
             case 6: return run_fp64<32, 2>(jb, s);
-            default: return run_fp64<256, 2>(jb, s);
+            case 7: return run_fp64<256, 2>(jb, s);
+            default: return run_fp64<64, 1>(jb, s);
         }
     }
     switch (v) {
@@ -515,10 +553,10 @@ int default_wavelet_variant(int mode, int which, int J)
     // regrouped one, whose stack is small, at 64 x 4 (the per-record work
     // shared by four visibilities), then 128 x 2; Eq. 16 (no stack) on packed
     // pairs of visibilities at 128 x 2
-    static const int order_mixed[kNumWaveletVariants] = {0, 2, 1, 3, 4, 5, 6, 7};
-    static const int order_mixed16[kNumWaveletVariants] = {2, 7, 3, 4, 0, 1, 5, 6};
-    static const int order_mixed_rg[kNumWaveletVariants] = {4, 2, 7, 6, 3, 5, 0, 1};
-    static const int order_fp64[kNumWaveletVariants] = {1, 0, 2, 3, 4, 5, 6, 7};
+    static const int order_mixed[kNumWaveletVariants] = {0, 2, 1, 3, 4, 5, 6, 7, 8};
+    static const int order_mixed16[kNumWaveletVariants] = {2, 7, 3, 4, 0, 1, 5, 6, 8};
+    static const int order_mixed_rg[kNumWaveletVariants] = {4, 2, 7, 6, 3, 5, 0, 1, 8};
+    static const int order_fp64[kNumWaveletVariants] = {8, 1, 0, 2, 3, 4, 5, 6, 7};
     const int* order = (mode == WT_FP64 || mode == WT_FP64_DF) ? order_fp64
                        : (which == WT_SUM_EQ17_REGROUPED) ? order_mixed_rg
                        : (which == WT_SUM_EQ16)           ? order_mixed16
@@ -526,6 +564,11 @@ int default_wavelet_variant(int mode, int which, int J)
     for (int i = 0; i < kNumWaveletVariants; ++i)
         if (wavelet_variant_fits(order[i], mode, which, J)) return order[i];
     return kNumWaveletVariants - 1;
+}
+
+bool wavelet_untuned(int mode, int which, int J)
+{
+    return mode == WT_FP64 && which == WT_SUM_EQ17 && wavelet_variant_fits(kVariantF64, mode, which, J);
 }
 
 int predict_wavelet(wt_tree t, const double* uvw, int64_t n_vis, void* vis, int mode, int sign, int which,
