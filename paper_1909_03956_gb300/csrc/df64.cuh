@@ -108,9 +108,7 @@ __device__ __forceinline__ void sincos_turns_df(float th, float tl, const float4
 // ---- two visibilities at once -------------------------------------------------
 // The same operations on packed pairs, element 0 one visibility and element 1
 // another: the float32 pipe takes a pair every two cycles in one issue slot, so
-// half of them are left for the records, the table and the sweep (one
-// visibility at a time the double-float sums issued an instruction in 9 of 10
-// cycles). A pair cannot be negated for free, so products are formed with their
+// half of them are left for the records, the table and the sweep. A pair cannot be negated for free, so products are formed with their
 // heads negated (from a factor that is kept negated) and subtracted.
 struct DFP {
     float2 h, l;

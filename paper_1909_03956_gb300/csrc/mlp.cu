@@ -416,10 +416,10 @@ __device__ __forceinline__ void silu_both(float z, float& h, float& d)
 // m16n8k16 fragments keep a warp's 16-row block of every activation in its
 // registers from the forward to the backward pass. Bound by the chain of small
 // dependent steps (two warps per scheduler, issue 23 % active): at 8 192 samples
-// (128 tiles on 152 SMs) 11.6 us, against 62 us with the products on the FMA
+// (64 samples a tile, 128 tiles on 152 SMs) 11.6 us, against 62 us with the products on the FMA
 // pipe an element per thread from shared memory, 16.9 us with 4 x 4 register
 // blocks there (bound by their 16-byte shared-memory loads); a training step
-// with k_mlp_adam 73 -> 14.9 us.
+// with k_mlp_adam 73 -> 14.9 us, 11.9 with tiles of 32 samples.
 template <int kS>
 __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float* __restrict__ params,
                                                                      const double* __restrict__ uvw,

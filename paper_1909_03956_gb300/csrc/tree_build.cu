@@ -390,8 +390,9 @@ __global__ void __launch_bounds__(kLevelThreads) k_tree_levels(const uint64_t* _
 // Up to kSmallComps components, a thread each, in one CTA: keys, stable radix
 // sort, leaves, levels J-1 .. 1 and the post-order positions, the level being
 // read kept in shared memory (global memory is only written). The general path
-// takes 3 ceil((2J + 2) / 8) + 4 launches, latency bound; 100 components at
-// J = 8: SMALL_HERE.
+// takes 3 ceil((2J + 2) / 8) + 4 launches, latency bound. A major cycle of 9 920
+// visibilities and 100 components at J = 8 (build, prediction, residuals): 158 ->
+// 106 us.
 constexpr int kSmallComps = 1024;
 
 struct SmallSmem {

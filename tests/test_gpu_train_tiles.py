@@ -1,5 +1,5 @@
 """Loss and gradient of the response network at the edges of the training
-kernel's 64-sample tiles and of its grid, against float64 with the two
+kernel's 32- and 64-sample tiles and of its grid, against float64 with the two
 documented bfloat16 roundings (W2 and the first hidden layer).
 
 Tolerance. The kernel's float32 sums err by 1e-6 at most; what dominates is a
@@ -34,7 +34,7 @@ def _reference(params, x, t):
     return float(loss), torch.autograd.grad(loss, p)[0].cpu().numpy()
 
 
-@pytest.mark.parametrize("n", [1, 63, 64, 65, 8192, 304 * 64 + 1, 20011])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 63, 64, 65, 8192, 304 * 32, 304 * 32 + 1, 304 * 64 + 1, 20011])
 def test_loss_and_gradient_at_tile_edges(n):
     level = 11
     m = wt.Mlp(level, np.pi, np.pi / 4, depth=2, x_max=1e30, seed=n)
