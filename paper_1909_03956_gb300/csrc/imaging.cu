@@ -183,19 +183,19 @@ __global__ void k_image_from_fft(const float2* __restrict__ f, int n, const unsi
 // and the Kaiser-Bessel half-width) for planes uniformly spaced in |w|,
 // from a midpoint sum over kWpSamples^2 points of the field, and interpolated
 // linearly in |w| between the two nearest planes. Each visibility stands for
-// two entries, V at B and conj(V) at -B; the image takes the real part of the
-// transform, and Re F(G + conj G(-.)) = 2 Re F(G), so one of them is gridded,
-// the one at w >= 0, and the image doubled (exact). Each entry is spread over
-// the support its own |w| needs (the same rule at that |w|), not the table's.
+// two entries, V at B and conj(V) at -B, whose taps are each other's conjugates
+// at mirrored cells: the one at w >= 0 is worked out and added to both. Each
+// entry is spread over the support its own |w| needs (the same rule at that
+// |w|), not the table's.
 //
-// The integrand is even in t and in s, and so is the table in x and in y: the
-// midpoint sum runs over the positive quadrant with real cosines, and one
-// quadrant of the table is computed (k_wp_stage1, k_wp_stage2: 16 times less
-// work than complex sums over the whole field, whose two products took 657 +
-// 230 us at 64 planes and h = 11; these take 17 + 17, latency bound, and
-// k_wp_field 19 us where float64 tapers and sincospi at every sample took
-// 420). k_wp_layout writes it out per offset within a cell, so that an entry's
-// taps are whole rows.
+// The table is summed over the whole field in a fixed order, multiplications
+// and additions rounded one by one: its rounding, divided by c(t) c(s) at the
+// image's edges, is most of a small image's error (1e-5 of it), and sums over
+// one quadrant with real cosines (16 times less work, 34 us where this takes
+// 119 at 64 planes and h = 11) move every image by as much. What the symmetry
+// gives exactly is taken: f is even in q, so stage 1 runs over half its rows.
+// 657 + 230 us with a thread per point reading along its own row of tw; the
+// field 18 us, 420 with float64 tapers and sincospi at every sample.
 constexpr int kWpWidth = 7;             // Kaiser-Bessel width (cells)
 constexpr double kWpBeta = 16.25;       // its shape parameter
 constexpr int kWpOversample = 8;        // table points per cell
@@ -224,30 +224,32 @@ __host__ __device__ inline double kb_taper(double t)
 struct WpPlan {
     int P;          // planes
     int h, S;       // half-support, support (cells)
-    int Tc;         // table points at x >= 0: x_c = c / oversample, c = 0 .. (h + 1/2) oversample
+    int T;          // table points per axis (S * oversample + 1)
     double dw;      // plane spacing in |w|
     double ndl;     // n dl: the field width (radians)
     double xc_per_w;   // the field's largest chirp frequency (cells) per unit |w|
 };
 
-__device__ __forceinline__ double wp_sample(int q) { return (q + 0.5) / kWpSamples; }   // t_q > 0
+__device__ __forceinline__ double wp_sample(int q) { return (q + 0.5) / kWpSamples; }   // the q-th t > 0
 
-// The tables of one image: ct[r][c] = cos(2 pi x_c t_r); ft[r] = c(t_r), the
-// field samples' taper; gc[i] = 1 / c((i - n/2) / n), the pixels' grid
-// correction, as a double-float.
-__global__ void k_wp_tables(WpPlan pl, int n, float* __restrict__ ct, double* __restrict__ ft, F2* __restrict__ gc)
+// The tables of one image: tw[r][j] = exp(i 2 pi x_j t_r), x_j = j /
+// oversample - (h + 1/2), for the samples t_r > 0 (at -t_r its conjugate);
+// ft[r] = c(t_r); gc[i] = 1 / c((i - n/2) / n), the pixels' grid correction,
+// as a double-float.
+__global__ void k_wp_tables(WpPlan pl, int n, float2* __restrict__ tw, double* __restrict__ ft, F2* __restrict__ gc)
 {
-    const int nc = pl.Tc * kWpHalf, total = nc + kWpHalf + n;
+    const int nt = pl.T * kWpHalf, total = nt + kWpHalf + n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        if (i < nc) {
-            const int r = i / pl.Tc, c = i % pl.Tc;
-            double ph = static_cast<double>(c) / kWpOversample * wp_sample(r);
-            ph -= rint(ph);
-            ct[i] = static_cast<float>(cospi(2.0 * ph));
-        } else if (i < nc + kWpHalf) {
-            ft[i - nc] = kb_taper(wp_sample(i - nc));
+        if (i < nt) {
+            const int r = i / pl.T, j = i % pl.T;
+            const double x = static_cast<double>(j) / kWpOversample - (pl.h + 0.5);
+            double sn, cs;
+            sincos_turns_f64(x * wp_sample(r), sn, cs);
+            tw[i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+        } else if (i < nt + kWpHalf) {
+            ft[i - nt] = kb_taper(wp_sample(i - nt));
         } else {
-            const int k = i - nc - kWpHalf;
+            const int k = i - nt - kWpHalf;
             gc[k] = split_f64(1.0 / kb_taper(static_cast<double>(k - n / 2) / n));
         }
     }
@@ -256,7 +258,7 @@ __global__ void k_wp_tables(WpPlan pl, int n, float* __restrict__ ct, double* __
 // f[p][q][r] = c(t_q) c(t_r) exp(-i 2 pi w_p (n - 1)) at the field's sample
 // points t > 0 (float64 phase): a thread per (q, r), the planes of a group of
 // kWpFieldPlanes one after the other (n - 1 and the taper are theirs alike).
-constexpr int kWpFieldPlanes = 8;
+constexpr int kWpFieldPlanes = 4;
 
 __global__ void k_wp_field(WpPlan pl, const double* __restrict__ ft, float2* __restrict__ f)
 {
@@ -276,78 +278,98 @@ __global__ void k_wp_field(WpPlan pl, const double* __restrict__ ft, float2* __r
     }
 }
 
-// a[p][q][c] = sum_r f[p][q][r] ct[r][c]: a CTA per (plane, 8 rows q), threads over c.
+// The products' inner step for kWpGroup rows and two columns at once: acc[g] +=
+// x_g b, x_g spread over pairs as (re, re, im, im): fl(re b.re - fl(im b.im))
+// and fl(re b.im + fl(im b.re)), then added, two elements per packed operation
+// (one 16-byte read of shared memory per six of them).
 constexpr int kWpGroup = 8;
 
-__global__ void __launch_bounds__(128) k_wp_stage1(WpPlan pl, const float2* __restrict__ f,
-                                                   const float* __restrict__ ct, float2* __restrict__ a)
+__device__ __forceinline__ void wp_step(float2 (&acc)[kWpGroup][2], const float4* x, float2 b0, float2 b1)
 {
-    __shared__ float2 row[kWpGroup][kWpHalf];
+    const float2 s0 = make_float2(-b0.y, b0.x), s1 = make_float2(-b1.y, b1.x);
+#pragma unroll
+    for (int g = 0; g < kWpGroup; ++g) {
+        const float4 v = x[g];
+        const float2 re = make_float2(v.x, v.y), im = make_float2(v.z, v.w);
+        acc[g][0] = add2(acc[g][0], fma2(re, b0, mul2(im, s0)));
+        acc[g][1] = add2(acc[g][1], fma2(re, b1, mul2(im, s1)));
+    }
+}
+__device__ __forceinline__ float4 wp_pairs(float2 v) { return make_float4(v.x, v.x, v.y, v.y); }
+
+// a[p][q][j] = sum_r f[p][q][r] tw[j][r] for the rows q at t > 0 (those at -t
+// are the same): a CTA per (plane, kWpGroup rows), a thread per two columns.
+__global__ void k_wp_stage1(WpPlan pl, const float2* __restrict__ f, const float2* __restrict__ tw,
+                            float2* __restrict__ a)
+{
+    __shared__ float4 row[kWpHalf][kWpGroup];
     const int p = blockIdx.x, q0 = blockIdx.y * kWpGroup;
     const float2* src = f + (static_cast<int64_t>(p) * kWpHalf + q0) * kWpHalf;
-    for (int i = threadIdx.x; i < kWpGroup * kWpHalf; i += blockDim.x) row[i / kWpHalf][i % kWpHalf] = src[i];
+    for (int i = threadIdx.x; i < kWpGroup * kWpHalf; i += blockDim.x)
+        row[i % kWpHalf][i / kWpHalf] = wp_pairs(src[i]);
     __syncthreads();
-    for (int c = threadIdx.x; c < pl.Tc; c += blockDim.x) {
-        float2 acc[kWpGroup];
+    const int half = (pl.T + 1) / 2;
+    for (int j = threadIdx.x; j < half; j += blockDim.x) {
+        const int j1 = min(j + half, pl.T - 1);   // T odd: the last thread's second column is its neighbour's too
+        float2 acc[kWpGroup][2];
 #pragma unroll
-        for (int g = 0; g < kWpGroup; ++g) acc[g] = make_float2(0.f, 0.f);
-#pragma unroll 8
-        for (int r = 0; r < kWpHalf; ++r) {
-            const float2 t = bcast2(__ldg(ct + r * pl.Tc + c));
-#pragma unroll
-            for (int g = 0; g < kWpGroup; ++g) acc[g] = fma2(row[g][r], t, acc[g]);
+        for (int g = 0; g < kWpGroup; ++g) acc[g][0] = acc[g][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int r = kWpHalf - 1; r >= 0; --r) {   // t < 0
+            const float2 t0 = __ldg(tw + r * pl.T + j), t1 = __ldg(tw + r * pl.T + j1);
+            wp_step(acc, row[r], make_float2(t0.x, -t0.y), make_float2(t1.x, -t1.y));
         }
+#pragma unroll 4
+        for (int r = 0; r < kWpHalf; ++r) wp_step(acc, row[r], __ldg(tw + r * pl.T + j), __ldg(tw + r * pl.T + j1));
 #pragma unroll
-        for (int g = 0; g < kWpGroup; ++g)
-            a[(static_cast<int64_t>(p) * kWpHalf + q0 + g) * pl.Tc + c] = acc[g];
+        for (int g = 0; g < kWpGroup; ++g) {
+            float2* out = a + (static_cast<int64_t>(p) * kWpHalf + q0 + g) * pl.T;
+            out[j] = acc[g][0];
+            out[j1] = acc[g][1];
+        }
     }
 }
 
-// K_q[p][i][c] = (4/M^2) sum_q ct[q][i] a[p][q][c], one quadrant of the
-// table: a CTA per (plane, 8 rows i), threads over c.
-__global__ void __launch_bounds__(128) k_wp_stage2(WpPlan pl, const float2* __restrict__ a,
-                                                   const float* __restrict__ ct, float2* __restrict__ Kq)
+// The table point (i, j), x_i and y_j, of plane p is (1/M^2) sum_q tw[i][q]
+// a[p][q][j]: a CTA per (plane, kWpGroup points i), a thread per two points j.
+// Written as the gridding reads it: K[p][oy][ox][ty][tx], tx, ty = 0 .. S, i =
+// tx oversample + ox, j = ty oversample + oy (an entry's taps are whole rows;
+// the places past the last point, i = S oversample, are never read).
+__global__ void k_wp_stage2(WpPlan pl, const float2* __restrict__ a, const float2* __restrict__ tw,
+                            float2* __restrict__ K)
 {
-    __shared__ float col[kWpHalf][kWpGroup];
+    constexpr int O = kWpOversample;
+    __shared__ float4 neg[kWpHalf][kWpGroup], pos[kWpHalf][kWpGroup];
     const int p = blockIdx.x, i0 = blockIdx.y * kWpGroup;
     for (int k = threadIdx.x; k < kWpGroup * kWpHalf; k += blockDim.x) {
         const int q = k / kWpGroup, g = k % kWpGroup;
-        col[q][g] = i0 + g < pl.Tc ? ct[q * pl.Tc + i0 + g] : 0.0f;
+        const float2 t = i0 + g < pl.T ? tw[q * pl.T + i0 + g] : make_float2(0.f, 0.f);
+        pos[q][g] = wp_pairs(t);
+        neg[q][g] = wp_pairs(make_float2(t.x, -t.y));
     }
     __syncthreads();
-    const float inv = 4.0f / (static_cast<float>(kWpSamples) * static_cast<float>(kWpSamples));
-    for (int c = threadIdx.x; c < pl.Tc; c += blockDim.x) {
-        float2 acc[kWpGroup];
+    const float inv = 1.0f / (static_cast<float>(kWpSamples) * static_cast<float>(kWpSamples));
+    const int half = (pl.T + 1) / 2, R = pl.S + 1;
+    float2* out = K + static_cast<int64_t>(p) * O * O * R * R;
+    for (int j = threadIdx.x; j < half; j += blockDim.x) {
+        const int j1 = min(j + half, pl.T - 1);
+        float2 acc[kWpGroup][2];
 #pragma unroll
-        for (int g = 0; g < kWpGroup; ++g) acc[g] = make_float2(0.f, 0.f);
-        const float2* ap = a + static_cast<int64_t>(p) * kWpHalf * pl.Tc + c;
-#pragma unroll 8
-        for (int q = 0; q < kWpHalf; ++q) {
-            const float2 v = __ldg(ap + q * pl.Tc);
-#pragma unroll
-            for (int g = 0; g < kWpGroup; ++g) acc[g] = fma2(v, bcast2(col[q][g]), acc[g]);
-        }
+        for (int g = 0; g < kWpGroup; ++g) acc[g][0] = acc[g][1] = make_float2(0.f, 0.f);
+        const float2* ap = a + static_cast<int64_t>(p) * kWpHalf * pl.T;
+#pragma unroll 4
+        for (int q = kWpHalf - 1; q >= 0; --q)
+            wp_step(acc, neg[q], __ldg(ap + q * pl.T + j), __ldg(ap + q * pl.T + j1));
+#pragma unroll 4
+        for (int q = 0; q < kWpHalf; ++q) wp_step(acc, pos[q], __ldg(ap + q * pl.T + j), __ldg(ap + q * pl.T + j1));
 #pragma unroll
         for (int g = 0; g < kWpGroup; ++g)
-            if (i0 + g < pl.Tc)
-                Kq[(static_cast<int64_t>(p) * pl.Tc + i0 + g) * pl.Tc + c] =
-                    make_float2(acc[g].x * inv, acc[g].y * inv);
-    }
-}
-
-// The table as the gridding reads it: K[p][oy][ox][ty][tx], ty, tx = 0 .. S,
-// the point x = tx + ox / oversample - (h + 1/2), y likewise (0 beyond the
-// support): a CTA per (p, oy, ox).
-__global__ void k_wp_layout(WpPlan pl, const float2* __restrict__ Kq, float2* __restrict__ K)
-{
-    constexpr int O = kWpOversample;
-    const int R = pl.S + 1, oy = (blockIdx.x / O) % O, ox = blockIdx.x % O;
-    const float2* src = Kq + static_cast<int64_t>(blockIdx.x / (O * O)) * pl.Tc * pl.Tc;
-    float2* dst = K + static_cast<int64_t>(blockIdx.x) * R * R;
-    const int mid = pl.Tc - 1;   // the table index of x = 0
-    for (int i = threadIdx.x; i < R * R; i += blockDim.x) {
-        const int cy = abs(O * (i / R) + oy - mid), cx = abs(O * (i % R) + ox - mid);
-        dst[i] = cy <= mid && cx <= mid ? __ldg(src + cy * pl.Tc + cx) : make_float2(0.f, 0.f);
+            if (i0 + g < pl.T) {
+                const int ox = (i0 + g) % O, tx = (i0 + g) / O;
+                out[((j % O) * O + ox) * R * R + (j / O) * R + tx] = make_float2(acc[g][0].x * inv, acc[g][0].y * inv);
+                out[((j1 % O) * O + ox) * R * R + (j1 / O) * R + tx] =
+                    make_float2(acc[g][1].x * inv, acc[g][1].y * inv);
+            }
     }
 }
 
@@ -370,14 +392,15 @@ __device__ __forceinline__ float2 wp_mix(float2 k0, float2 k1, float a)
 }
 
 // The general form of an entry (V at cell (uc, vc) of the grid, half-support
-// he, offsets fx, fy): every tap finds its table point in both entries of the
-// pair, and where they differ takes their mean, as gridding both would.
+// he, offsets fx, fy): every tap finds its table point in each entry of the
+// pair.
 __device__ __noinline__ void wp_spread_ties(const WpPlan& pl, const float2* __restrict__ K0, float a, float2 V,
                                             int uc, int vc, int he, float fx, float fy, int n,
                                             float2* __restrict__ grid, int lane)
 {
     constexpr int O = kWpOversample;
     const int R = pl.S + 1, last = pl.S * O, Se = 2 * he + 1;
+    const int64_t mirror = static_cast<int64_t>(n / 2 * 2) * (n + 1);   // the sum of two mirrored cells' indices
     const float2* K1 = K0 + static_cast<int64_t>(O) * O * R * R;
     auto index = [&](int d, float f) { return __float2int_rn((static_cast<float>(d) - f + pl.h + 0.5f) * O); };
     auto value = [&](int ix, int iy) {
@@ -388,26 +411,31 @@ __device__ __noinline__ void wp_spread_ties(const WpPlan& pl, const float2* __re
         const int dx = t % Se - he, dy = t / Se - he;
         const float2 k0 = value(index(dx, fx), index(dy, fy));
         const float2 k1 = value(last - index(-dx, -fx), last - index(-dy, -fy));
-        const float sg = ((uc + dx + vc + dy) & 1) ? -0.5f : 0.5f;
-        const float2 e = cmul(V, make_float2(k0.x + k1.x, k0.y + k1.y));
-        atomicAdd(grid + static_cast<int64_t>(vc + dy) * n + uc + dx, make_float2(sg * e.x, sg * e.y));
+        const float sg = ((uc + dx + vc + dy) & 1) ? -1.0f : 1.0f;
+        const int64_t at = static_cast<int64_t>(vc + dy) * n + uc + dx;
+        const float2 e = cmul(V, k0), m = cmul(V, k1);
+        atomicAdd(grid + at, make_float2(sg * e.x, sg * e.y));
+        atomicAdd(grid + (mirror - at), make_float2(sg * m.x, -sg * m.y));
     }
 }
 
-// A warp takes `group` visibilities (unit values if vis is null): each of its
-// first `group` lanes plans one (cell, offset, planes, support: float64 work
-// that a whole warp would repeat), then the warp spreads them one after the
-// other, a lane per aligned pair of cells of a row, 32 / L rows at a time
-// (L lanes cover a row). An entry whose support leaves the grid is dropped;
-// counts two entries per visibility gridded.
-// Bound by L2: per tap 16 bytes of table (two planes, rows of the layout) and
-// an 8-byte addition to the grid, two cells per 16-byte atomic. Medium array,
-// 1 008 000 visibilities, 2048 x 2048, 64 planes: 0.51 ms, against 3.0 ms
-// for both entries of each visibility with 4-byte atomics and a table read
-// across its rows.
+// A warp takes every warps-th visibility (unit values if vis is null), 32 at a
+// time: each lane plans one (cell, offset, planes, support: float64 work that a
+// whole warp would repeat), then the warp spreads them one after the other, a
+// lane per tap, row by row, into both cells of the pair. An entry whose support
+// leaves the grid is dropped; counts two entries per visibility gridded.
+// Bound by the load/store path: per tap 16 bytes of table (two planes, rows of
+// the layout) and two 8-byte additions to the grid, all in whole lines. Medium
+// array, 1 008 000 visibilities, 2048 x 2048, 64 planes: 0.73 ms, against 3.0
+// when each entry read the table across its rows and added 4 bytes at a time.
+// One entry per pair and the image doubled, runs of neighbouring visibilities
+// to a warp, take 0.44 ms, but change the order of the cells' float32 sums: a
+// thousand additions of like sign round to 1.4e-4 of the image (the correction
+// in its corners is 1 / c^2 = 2 900), differently in each order. This order
+// keeps images as they have been, to 4e-5.
 __global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __restrict__ K,
                                                     const double* __restrict__ uvw, const float2* __restrict__ vis,
-                                                    int64_t n_vis, int n, double inv_du, int group,
+                                                    int64_t n_vis, int n, double inv_du,
                                                     float2* __restrict__ grid, unsigned long long* __restrict__ count)
 {
     constexpr int O = kWpOversample;
@@ -416,81 +444,82 @@ __global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __r
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int R = pl.S + 1, half = n / 2;
-    const int64_t k = (static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5)) * group + lane;
-    // the plan of this lane's visibility: its cell, half-support, lower plane,
-    // table row and column of the first tap (-1: near a tie), offset from the
-    // cell's centre and weight between the planes
-    int uc = 0, vc = 0, he = -1, p0 = 0, tab = -1;
-    float fx = 0.0f, fy = 0.0f, a = 0.0f;
-    float2 V = make_float2(0.f, 0.f);
-    if (lane < group && k < n_vis) {
-        double x = uvw[3 * k] * inv_du, y = uvw[3 * k + 1] * inv_du, w = uvw[3 * k + 2];
-        V = vis ? vis[k] : make_float2(1.0f, 0.0f);
-        if (w < 0.0) {               // the conjugate entry
-            x = -x;
-            y = -y;
-            w = -w;
-            V.y = -V.y;
-        }
-        const double icd = rint(x), jcd = rint(y);
-        const double lo = -half + pl.h + 1, hi = half - pl.h - 1;
-        if (icd >= lo && icd <= hi && jcd >= lo && jcd <= hi && w <= 1e30) {   // false for NaN too
-            fx = static_cast<float>(x - icd);
-            fy = static_cast<float>(y - jcd);
-            const double pw = w / pl.dw;
-            p0 = static_cast<int>(floor(pw));
-            if (p0 > pl.P - 2) p0 = pl.P - 2;
-            if (p0 < 0) p0 = 0;
-            a = static_cast<float>(fmin(fmax(pw - p0, 0.0), 1.0));
-            // this entry's own support: the Kaiser-Bessel half-width and the
-            // chirp frequency of its |w| (the kernel is negligible beyond),
-            // within the table's
-            he = static_cast<int>(fmin(ceil(0.5 * kWpWidth + pl.xc_per_w * w) + 1.0, static_cast<double>(pl.h)));
-            uc = static_cast<int>(icd) + half;
-            vc = static_cast<int>(jcd) + half;
-            // tap d's nearest table point is at (d - fx + h + 1/2) oversample:
-            // d + h cells and an offset o = 0 .. oversample alike for every tap
-            // (o = oversample: the next cell's 0)
-            const float gx = (0.5f - fx) * O, gy = (0.5f - fy) * O;
-            const int ox = __float2int_rn(gx), oy = __float2int_rn(gy);
-            if (fabsf(fabsf(gx - ox) - 0.5f) > kWpTie && fabsf(fabsf(gy - oy) - 0.5f) > kWpTie)
-                tab = (((oy % O) * O + ox % O) * R + pl.h - he + oy / O) * R + pl.h - he + ox / O;
-        }
-    }
-    const unsigned todo = __ballot_sync(0xffffffffu, he >= 0);
-    if (lane == 0 && todo) atomicAdd(&blk, 2u * __popc(todo));
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x / 32);
     const int64_t plane = static_cast<int64_t>(O) * O * R * R;
-    for (unsigned left = todo; left; left &= left - 1) {
-        const int src = __ffs(left) - 1;
-        const int su = __shfl_sync(0xffffffffu, uc, src), sv = __shfl_sync(0xffffffffu, vc, src);
-        const int sh = __shfl_sync(0xffffffffu, he, src), st = __shfl_sync(0xffffffffu, tab, src);
-        const int sp = __shfl_sync(0xffffffffu, p0, src);
-        const float sa = __shfl_sync(0xffffffffu, a, src);
-        const float2 sV = make_float2(__shfl_sync(0xffffffffu, V.x, src), __shfl_sync(0xffffffffu, V.y, src));
-        const float2* K0 = K + sp * plane;
-        if (st < 0) {
-            const float sx = __shfl_sync(0xffffffffu, fx, src), sy = __shfl_sync(0xffffffffu, fy, src);
-            wp_spread_ties(pl, K0, sa, sV, su, sv, sh, sx, sy, n, grid, lane);
-            continue;
+    const int64_t mirror = static_cast<int64_t>(half * 2) * (n + 1);   // the sum of two mirrored cells' indices
+    for (int64_t k0 = static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5); k0 < n_vis;
+         k0 += 32 * warps) {
+        const int64_t k = k0 + lane * warps;
+        // the plan of this lane's visibility: its cell, half-support, lower plane,
+        // table row and column of the first tap (-1: near a tie), offset from the
+        // cell's centre and weight between the planes
+        int uc = 0, vc = 0, he = -1, p0 = 0, tab = -1;
+        float fx = 0.0f, fy = 0.0f, a = 0.0f;
+        float2 V = make_float2(0.f, 0.f);
+        if (k < n_vis) {
+            double x = uvw[3 * k] * inv_du, y = uvw[3 * k + 1] * inv_du, w = uvw[3 * k + 2];
+            V = vis ? vis[k] : make_float2(1.0f, 0.0f);
+            if (w < 0.0) {               // the conjugate entry
+                x = -x;
+                y = -y;
+                w = -w;
+                V.y = -V.y;
+            }
+            const double icd = rint(x), jcd = rint(y);
+            const double lo = -half + pl.h + 1, hi = half - pl.h - 1;
+            if (icd >= lo && icd <= hi && jcd >= lo && jcd <= hi && w <= 1e30) {   // false for NaN too
+                fx = static_cast<float>(x - icd);
+                fy = static_cast<float>(y - jcd);
+                const double pw = w / pl.dw;
+                p0 = static_cast<int>(floor(pw));
+                if (p0 > pl.P - 2) p0 = pl.P - 2;
+                if (p0 < 0) p0 = 0;
+                a = static_cast<float>(fmin(fmax(pw - p0, 0.0), 1.0));
+                // this entry's own support: the Kaiser-Bessel half-width and the
+                // chirp frequency of its |w| (the kernel is negligible beyond),
+                // within the table's
+                he = static_cast<int>(fmin(ceil(0.5 * kWpWidth + pl.xc_per_w * w) + 1.0, static_cast<double>(pl.h)));
+                uc = static_cast<int>(icd) + half;
+                vc = static_cast<int>(jcd) + half;
+                // tap d's nearest table point is at (d - fx + h + 1/2) oversample:
+                // d + h cells and an offset o = 0 .. oversample alike for every tap
+                // (o = oversample: the next cell's 0)
+                const float gx = (0.5f - fx) * O, gy = (0.5f - fy) * O;
+                const int ox = __float2int_rn(gx), oy = __float2int_rn(gy);
+                if (fabsf(fabsf(gx - ox) - 0.5f) > kWpTie && fabsf(fabsf(gy - oy) - 0.5f) > kWpTie)
+                    tab = (((oy % O) * O + ox % O) * R + pl.h - he + oy / O) * R + pl.h - he + ox / O;
+            }
         }
-        K0 += st;
-        const float2* K1 = K0 + plane;
-        const int Se = 2 * sh + 1, u0 = su - sh, v0 = sv - sh;   // the first tap's cell
-        const int ua = u0 & ~1;                            // even: a pair of cells is 16-byte aligned
-        const int pairs = (u0 + Se - ua + 1) >> 1;
-        const int lg = pairs <= 8 ? 3 : pairs <= 16 ? 4 : 5;   // log2 of the lanes per row
-        for (int r = lane >> lg; r < Se; r += 32 >> lg) {
-            const float sg = ((v0 + r) & 1) ? -1.0f : 1.0f;    // the index shift (-1)^(iu+iv), iu even
-            float4* out = reinterpret_cast<float4*>(grid + static_cast<int64_t>(v0 + r) * n + ua);
-            for (int q = lane & ((1 << lg) - 1); q < pairs; q += 1 << lg) {
-                float2 e[2];
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int t = 2 * q + j + ua - u0;         // tap -1 and Se: outside the support
-                    e[j] = make_float2(0.f, 0.f);
-                    if (t >= 0 && t < Se) e[j] = cmul(sV, wp_mix(__ldg(K0 + r * R + t), __ldg(K1 + r * R + t), sa));
-                }
-                atomicAdd(out + q, make_float4(sg * e[0].x, sg * e[0].y, -sg * e[1].x, -sg * e[1].y));
+        const unsigned todo = __ballot_sync(0xffffffffu, he >= 0);
+        if (lane == 0 && todo) atomicAdd(&blk, 2u * __popc(todo));
+        for (unsigned left = todo; left; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int su = __shfl_sync(0xffffffffu, uc, src), sv = __shfl_sync(0xffffffffu, vc, src);
+            const int sh = __shfl_sync(0xffffffffu, he, src), st = __shfl_sync(0xffffffffu, tab, src);
+            const int sp = __shfl_sync(0xffffffffu, p0, src);
+            const float sa = __shfl_sync(0xffffffffu, a, src);
+            const float2 sV = make_float2(__shfl_sync(0xffffffffu, V.x, src), __shfl_sync(0xffffffffu, V.y, src));
+            const float2* K0 = K + sp * plane;
+            if (st < 0) {
+                const float sx = __shfl_sync(0xffffffffu, fx, src), sy = __shfl_sync(0xffffffffu, fy, src);
+                wp_spread_ties(pl, K0, sa, sV, su, sv, sh, sx, sy, n, grid, lane);
+                continue;
+            }
+            K0 += st;
+            const float2* K1 = K0 + plane;
+            const int Se = 2 * sh + 1;
+            float2* out = grid + static_cast<int64_t>(sv - sh) * n + su - sh;   // the first tap's cell
+            float2* opp = grid + (mirror - (out - grid));           // the mirrored entry's
+            const int par = su + sv;                               // of (-1)^(iu+iv): that of the first tap's cell
+            const unsigned recip = ((1u << 20) + Se - 1) / Se;     // t / Se = (t recip) >> 20 for t < 65^2
+            for (int t = lane; t < Se * Se; t += 32) {
+                const int r = static_cast<int>((t * recip) >> 20), q = t - r * Se;
+                const int at = r * R + q;
+                const float2 e = cmul(sV, wp_mix(__ldg(K0 + at), __ldg(K1 + at), sa));
+                const float sg = ((par + r + q) & 1) ? -1.0f : 1.0f;
+                const float2 v = make_float2(sg * e.x, sg * e.y);
+                atomicAdd(out + (r * n + q), v);
+                atomicAdd(opp - (r * n + q), make_float2(v.x, -v.y));
             }
         }
     }
@@ -498,15 +527,14 @@ __global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __r
     if (threadIdx.x == 0 && blk) atomicAdd(count, static_cast<unsigned long long>(blk));
 }
 
-// Twice the real part of the transformed grid, times
-// (-1)^(ix+iy) / (W c(t) c(s)), the correction's product in double-float.
+// Real part of the transformed grid, times (-1)^(ix+iy) / (W c(t) c(s)), the correction's product in double-float.
 // Bound by HBM (12 bytes per pixel); with both tapers evaluated per pixel in
 // float64 714 us at 2048 x 2048, 23 us so.
 __global__ void k_image_from_fft_wp(const float2* __restrict__ f, int n, const unsigned long long* __restrict__ count,
                                     const F2* __restrict__ gc, float* __restrict__ image)
 {
     const unsigned long long W = *count;
-    const double inv = W ? 2.0 / static_cast<double>(W) : 0.0;
+    const double inv = W ? 1.0 / static_cast<double>(W) : 0.0;
     for (int iy = blockIdx.x; iy < n; iy += gridDim.x) {
         const int64_t row = static_cast<int64_t>(iy) * n;
         const F2 g = gc[iy];
@@ -1246,19 +1274,18 @@ int dirty_image_w(const double* uvw, const float2* vis, int64_t n_vis, int n, do
     if (2 * pl.h + 2 >= n / 2) return set_error(WT_ERR_RANGE, "%s: a %d-cell kernel does not fit an n = %d grid", fn,
                                                 2 * pl.h + 1, n);
     pl.S = 2 * pl.h + 1;
-    pl.Tc = pl.S * kWpOversample / 2 + 1;
+    pl.T = pl.S * kWpOversample + 1;
     constexpr int H = kWpHalf, O = kWpOversample;
     auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t b_grid = up(nn * sizeof(float2)), b_cnt = 256;
-    const size_t b_ct = up(static_cast<size_t>(pl.Tc) * H * sizeof(float));
+    const size_t b_tw = up(static_cast<size_t>(pl.T) * H * sizeof(float2));
     const size_t b_ft = up(H * sizeof(double)), b_gc = up(static_cast<size_t>(n) * sizeof(F2));
     const size_t b_f = up(static_cast<size_t>(planes) * H * H * sizeof(float2));
-    const size_t b_a = up(static_cast<size_t>(planes) * H * pl.Tc * sizeof(float2));
-    const size_t b_q = up(static_cast<size_t>(planes) * pl.Tc * pl.Tc * sizeof(float2));
+    const size_t b_a = up(static_cast<size_t>(planes) * H * pl.T * sizeof(float2));
     const size_t b_k = up(static_cast<size_t>(planes) * O * O * (pl.S + 1) * (pl.S + 1) * sizeof(float2));
     char* scratch = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch),
-                                    b_grid + b_cnt + b_ct + b_ft + b_gc + b_f + b_a + b_q + b_k, s);
+                                    b_grid + b_cnt + b_tw + b_ft + b_gc + b_f + b_a + b_k, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(WT_ERR_NOMEM, "%s: scratch allocation failed: %s", fn, cudaGetErrorString(e));
@@ -1271,31 +1298,27 @@ int dirty_image_w(const double* uvw, const float2* vis, int64_t n_vis, int n, do
     };
     float2* grid = reinterpret_cast<float2*>(take(b_grid));
     unsigned long long* count = reinterpret_cast<unsigned long long*>(take(b_cnt));
-    float* ct = reinterpret_cast<float*>(take(b_ct));
+    float2* tw = reinterpret_cast<float2*>(take(b_tw));
     double* ft = reinterpret_cast<double*>(take(b_ft));
     F2* gc = reinterpret_cast<F2*>(take(b_gc));
     float2* f = reinterpret_cast<float2*>(take(b_f));
     float2* a = reinterpret_cast<float2*>(take(b_a));
-    float2* Kq = reinterpret_cast<float2*>(take(b_q));
     float2* K = reinterpret_cast<float2*>(take(b_k));
     int rc = WT_OK;
-    k_wp_tables<<<(pl.Tc * H + H + n + 127) / 128, 128, 0, s>>>(pl, n, ct, ft, gc);
+    const int pairs = (pl.T + 1) / 2, turns = (pairs + 255) / 256;
+    const int tj = ((pairs + turns - 1) / turns + 31) / 32 * 32;   // a thread per two table points
+    k_wp_tables<<<(pl.T * H + H + n + 127) / 128, 128, 0, s>>>(pl, n, tw, ft, gc);
     k_wp_field<<<dim3((H * H + 127) / 128, (planes + kWpFieldPlanes - 1) / kWpFieldPlanes), 128, 0, s>>>(pl, ft, f);
-    k_wp_stage1<<<dim3(planes, H / kWpGroup), 128, 0, s>>>(pl, f, ct, a);
-    k_wp_stage2<<<dim3(planes, (pl.Tc + kWpGroup - 1) / kWpGroup), 128, 0, s>>>(pl, a, ct, Kq);
-    k_wp_layout<<<static_cast<unsigned>(planes * O * O), 256, 0, s>>>(pl, Kq, K);
+    k_wp_stage1<<<dim3(planes, H / kWpGroup), tj, 0, s>>>(pl, f, tw, a);
+    k_wp_stage2<<<dim3(planes, (pl.T + kWpGroup - 1) / kWpGroup), tj, 0, s>>>(pl, a, tw, K);
     if (cudaGetLastError() != cudaSuccess) rc = set_error(WT_ERR_CUDA, "%s: kernel tables", fn);
     if (rc == WT_OK && (cudaMemsetAsync(grid, 0, static_cast<size_t>(nn) * sizeof(float2), s) != cudaSuccess ||
                         cudaMemsetAsync(count, 0, sizeof(unsigned long long), s) != cudaSuccess))
         rc = set_error(WT_ERR_CUDA, "%s: clearing the grid", fn);
     if (rc == WT_OK && n_vis > 0) {
-        // 32 visibilities per warp, fewer for a batch that would leave the
-        // chip short of warps (32 per SM)
-        int group = 32;
-        while (group > 4 && n_vis < static_cast<int64_t>(num_sms()) * 32 * group) group /= 2;
-        const int64_t per_cta = 8 * group;
-        k_grid_wproj<<<static_cast<unsigned>((n_vis + per_cta - 1) / per_cta), 256, 0, s>>>(
-            pl, K, uvw, vis, n_vis, n, ndl, group, grid, count);
+        // 8 warps per CTA; a warp per visibility up to 256 warps per SM
+        const int64_t b = std::min<int64_t>((n_vis + 7) / 8, static_cast<int64_t>(num_sms()) * 32);
+        k_grid_wproj<<<static_cast<unsigned>(b), 256, 0, s>>>(pl, K, uvw, vis, n_vis, n, ndl, grid, count);
         if (cudaGetLastError() != cudaSuccess) rc = set_error(WT_ERR_CUDA, "%s: gridding launch", fn);
     }
     if (rc == WT_OK) rc = fft2_forward(grid, n, s);
