@@ -514,11 +514,12 @@ ALG_FLOPS_PER_NODE = 40
 # (record decode, loads, stores, branches, register moves, roundings to
 # integer) is not counted, and the special-function unit's sin and cos are
 # counted separately against that unit's own peak. A complex add is 2 ops.
-#   phase (every leaf): three double-float products (4 each), two
-#     error-free sums (6 each), reduction by the nearest integer (1), tail
-#     (4): 29.
+#   phase (every leaf) on the head grid: per coordinate the head added onto
+#     the grid (1), its remainder (2) and the two cross terms (2); the
+#     reduction (1), the tails' sum (2): 18 (29 with error-free sums, in the
+#     exact pass over tiles beyond the grid's range).
 #   polynomial sin/cos: quadrant reduction and angle (5), sin and cos
-#     polynomials (5 each): 15 (the quadrant selection runs on the ALU).
+#     polynomials (4 each): 13 (the quadrant selection runs on the ALU).
 #   fast sin/cos: the angle (2) and the SFU argument scaling (1): 3, plus
 #     sin and cos on the special-function unit (2 SFU ops).
 #   explicit internal node: butterflies (8), xi (2), three sigma (6),
@@ -529,22 +530,19 @@ ALG_FLOPS_PER_NODE = 40
 #     other internal node adds w xi (plus, at level J - 2, its children's
 #     sum) to V (2, with a Kahan add of 8); every internal node passes xi to
 #     its parent's sum (2).
-OPS_PHASE = 12 + 12 + 1 + 4
-# The regrouped forms' phase on the head grid: per coordinate the head on the
-# grid (2), its remainder (1) and the two cross terms (2); the heads' sum (2),
-# the reduction (1), the tails' sum (2): 20.
-OPS_PHASE_GRID = 3 * 5 + 2 + 1 + 2
-OPS_LEAF = OPS_PHASE + 15
+OPS_PHASE_GRID = 3 * 5 + 1 + 2
+OPS_POLY = 13
+OPS_LEAF = OPS_PHASE_GRID + OPS_POLY
 OPS_NODE = 30
-OPS_LEAF_FAST = OPS_PHASE + 3
+OPS_LEAF_FAST = OPS_PHASE_GRID + 3
 OPS_RG_LEAF = 2 + 2
 OPS_RG_NODE = 2 + 8 + 2
 OPS_RG_LOW = 2 + 2 + 2
 # (form, sum) -> (per leaf, per internal node, per internal node at level J - 1)
 OPS = {("mixed", "explicit"): (OPS_LEAF, OPS_NODE, OPS_NODE),
        ("fast", "explicit"): (OPS_LEAF_FAST, OPS_NODE, OPS_NODE),
-       ("mixed", "regrouped"): (OPS_LEAF - OPS_PHASE + OPS_PHASE_GRID + OPS_RG_LEAF, OPS_RG_NODE, OPS_RG_LOW),
-       ("fast", "regrouped"): (OPS_LEAF_FAST - OPS_PHASE + OPS_PHASE_GRID + OPS_RG_LEAF, OPS_RG_NODE, OPS_RG_LOW)}
+       ("mixed", "regrouped"): (OPS_LEAF + OPS_RG_LEAF, OPS_RG_NODE, OPS_RG_LOW),
+       ("fast", "regrouped"): (OPS_LEAF_FAST + OPS_RG_LEAF, OPS_RG_NODE, OPS_RG_LOW)}
 SFU_OPS_LEAF = {"fast": 2, "mixed": 0}
 # DRAM bytes of one k_wavelet_mixed launch at J = 12, from ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum), per (workload, form, sum);
@@ -552,26 +550,25 @@ SFU_OPS_LEAF = {"fast": 2, "mixed": 0}
 TRAFFIC_BYTES = {("large_256ant_15993600vis_50000comp", "fast", "regrouped"): 388_350_000 + 107_320_000}
 # Double-float form (WT_FP64_DF, regrouped Eq. 17), float32 FMA-pipe ops per
 # (vis, leaf): phase 32 (three double-float products of 5, two error-free
-# sums of 6, reduction 1, tail 4), sin/cos 135 (argument reduction 8, 2 pi f,
-# x^2, x^3 and x^3/6 as double-float products of 7, the float32 tails 6,
-# three double-float sums of 10-11 and one of 11, the rotation by the table
-# entry: four products of 7 and two sums of 11), w eta into V 36, the
-# parent's sum 22; per (vis, internal node): quarter 4, w eta into V 36, the
-# parent's sum 22.
-OPS_DF_LEAF = 32 + 135 + 36 + 22
-OPS_DFT_DF = 32 + 135 + 36   # per (vis, component) of the double-float direct sum
-OPS_DF_NODE = 4 + 36 + 22
+# sums of 6, reduction 1, tail 4), sin/cos 74 (argument reduction 9, 2 pi f 4,
+# x^2 4, sin x and cos x - 1 as double-floats 7, the rotation by the table
+# entry: four products of 4 and sums of 8, two signs), w eta into V 24 (two
+# products and sums), the parent's sum 16; per (vis, internal node): quarter 4,
+# w eta into V 24 and V renormalised 6, the parent's sum 16. The direct sum
+# renormalises every eight components (1).
+OPS_DF_LEAF = 32 + 74 + 24 + 16
+OPS_DFT_DF = 32 + 74 + 24 + 1   # per (vis, component) of the double-float direct sum
+OPS_DF_NODE = 4 + 24 + 6 + 16
 # Direct sum (k_dft_mixed, two visibilities x two components per step), FMA-pipe
-# element ops per (visibility, component): phase 20 on the head grid (the
+# element ops per (visibility, component): phase 18 on the head grid (the
 # grid pass; the exact pass's 29 only for tiles beyond the grid's range),
-# angle and SFU scaling 3 (fast) or polynomial sin/cos 15, the flux times
+# angle and SFU scaling 3 (fast) or polynomial sin/cos 13, the flux times
 # (cos, sin) 2, half a Kahan add of a pair of terms 4. float64 (k_dft_fp64), FP64-pipe instructions per
-# term: phase 3, table reduction and polynomials 14, rotation by the table
-# entry 2 (+2 multiplies), multiply-add into V 2 -> 21 (roundings to integer
-# and the table load not counted).
+# term: phase 3, table reduction 3, polynomials 6, rotation by the table entry
+# 4, multiply-add into V 2 -> 18.
 OPS_DFT_FAST = OPS_PHASE_GRID + 3 + 2 + 4
-OPS_DFT = OPS_PHASE_GRID + 15 + 2 + 4
-OPS_DFT_FP64 = 21
+OPS_DFT = OPS_PHASE_GRID + OPS_POLY + 2 + 4
+OPS_DFT_FP64 = 18
 # Direct sum with the phase on the tensor cores (k_dft_tc), FMA-pipe element
 # ops per (visibility, component) in the epilogue: the accumulators'
 # recombination modulo 1 7, the angle 2, the SFU's scaling 1, the flux times
