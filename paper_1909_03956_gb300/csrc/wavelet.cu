@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(NT) k_wavelet_fp64(const Rec* __restrict__ rec
             b.sgn = sgn;
             b.stk = stk;
             b.maxrow = rows - 1;
-            good = st.sweep(b);
+            good = st.sweep_at(b);
 #pragma unroll
             for (int k = 0; k < VPT; ++k) { vr[k] = b.vr[k]; vi[k] = b.vi[k]; }
         } else {
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT) k_wavelet_fp64(const Rec* __restrict__ rec
 }
 
 // The float64-class double-float form: regrouped Eq. 17 (Eq17DF) on the
-// float32 pipe. Shared memory: the record staging, the 257-entry
+// float32 pipe. Shared memory: the record staging, the 1 024-entry
 // double-float sin/cos table, then the stack.
 template <int NT, int VPT, int SUM>
 __global__ void __launch_bounds__(NT) k_wavelet_df(const RecWDF* __restrict__ recs,

