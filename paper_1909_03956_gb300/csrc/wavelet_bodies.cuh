@@ -26,7 +26,8 @@ __device__ __forceinline__ int clamp_row(uint32_t r, int maxrow) { return min(st
 // the float64 pipe for a node of several children and 2 for an only child,
 // where eta and the three sigma with their factors took 32 and 10; with the
 // sine and cosine's 13 for 18, 201 600 visibilities of 1 115 leaves 16.4 ->
-// 13.6 ms (12.3 with the tiles' waves evened out: fp64_resident).
+// 13.6 ms (12.3 with the tiles' waves evened out: fp64_resident; 11.6 with leaves
+// in groups: at).
 template <int NT, int VPT>
 struct Eq17D {
     double u[VPT], v[VPT], w[VPT];
@@ -37,27 +38,86 @@ struct Eq17D {
 
     __device__ __forceinline__ double2& slot(int row, int k) { return stk[(row * VPT + k) * NT]; }
 
+    __device__ __forceinline__ void wave(const RecD& r, int k, double2& e) const
+    {
+        const double t = fma(w[k], r.c, fma(v[k], r.b, u[k] * r.a));
+        sincos_turns_f64(t, e.y, e.x);
+    }
+
+    // A node of several children, one visibility.
+    __device__ __forceinline__ void node(const RecD& r, bool root, int srow, int k, double2 c0, double2 c1,
+                                         double2 c2, double2 c3)
+    {
+        const double ar = c0.x + c1.x, ai = c0.y + c1.y;   // c0 + c1
+        const double br = c0.x - c1.x, bi = c0.y - c1.y;   // c0 - c1
+        const double cr = c2.x + c3.x, ci = c2.y + c3.y;   // c2 + c3
+        const double dr = c2.x - c3.x, di = c2.y - c3.y;   // c2 - c3
+        const double er = ar + cr, ei = ai + ci;           // Eq. 9 form (times 4^(J-j))
+        // Eq. 10 rows (+ - + -), (+ + - -), (+ - - +), weighted by gamma
+        vr[k] = fma(r.a, br + dr, fma(r.b, ar - cr, fma(r.c, br - dr, vr[k])));
+        vi[k] = fma(r.a, bi + di, fma(r.b, ai - ci, fma(r.c, bi - di, vi[k])));
+        if (root) {
+            vr[k] = fma(r.e, er, vr[k]);
+            vi[k] = fma(r.e, ei, vi[k]);
+        } else {
+            slot(srow, k) = make_double2(er, ei);
+        }
+    }
+
     // One step of the sweep; returns the records it took. Two leaves in a row
     // are siblings (a last sibling is followed by its parent) and independent:
     // their chains of float64 operations run side by side, which an SM's eight
-    // warps alone do not hide: 201 563 visibilities of 1 126 leaves 12.5 -> 11.8
-    // ms, 1.03-1.05x from 50 000 visibilities up.
+    // warps alone do not hide. Where the whole run and its parent are in the
+    // chunk (the run as long as the parent has children), the waves go to the
+    // parent's butterfly in registers, not through the stack. 201 563 visibilities
+    // of 1 126 leaves: 12.49 ms a leaf at a time, 11.81 in pairs, 11.75 so (a
+    // smaller batch, 1.58 ms before: 1.17, 1.12, 1.10).
     __device__ __forceinline__ int at(const RecD* cb, int r, int n)
     {
         const uint32_t m0 = cb[r].meta;
         if ((m0 & (kRecLeaf | kRecRoot)) == kRecLeaf && r + 1 < n && (cb[r + 1].meta & kRecLeaf)) {
+            const int len = r + 2 < n && !(cb[r + 2].meta & kRecLeaf)   ? 2
+                            : r + 3 < n && !(cb[r + 3].meta & kRecLeaf) ? 3
+                            : r + 4 < n && !(cb[r + 4].meta & kRecLeaf) ? 4
+                                                                        : 0;
+            const uint32_t mask = len ? rec_mask(cb[r + len].meta) : 0u;
+            if (len && __popc(mask) == len) {
+                const RecD& par = cb[r + len];
+                const bool root = par.meta & kRecRoot;
+                const int srow = clamp_row(rec_store_row(par.meta), maxrow);
+                const bool b0 = mask & 1u, b1 = mask & 2u, b2 = mask & 4u, b3 = mask & 8u;
+                const int before2 = (b0 ? 1 : 0) + (b1 ? 1 : 0);
+                const double2 zero = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int k = 0; k < VPT; ++k) {
+                    double2 e0, e1, e2 = zero, e3 = zero;
+                    wave(cb[r], k, e0);
+                    wave(cb[r + 1], k, e1);
+                    if (len == 4) {
+                        wave(cb[r + 2], k, e2);
+                        wave(cb[r + 3], k, e3);
+                        node(par, root, srow, k, e0, e1, e2, e3);
+                    } else {
+                        if (len == 3) wave(cb[r + 2], k, e2);
+                        const double2 c0 = b0 ? e0 : zero;
+                        const double2 c1 = !b1 ? zero : b0 ? e1 : e0;
+                        const double2 c2 = !b2 ? zero : before2 == 2 ? e2 : before2 == 1 ? e1 : e0;
+                        const double2 c3 = !b3 ? zero : len == 3 ? e2 : e1;
+                        node(par, root, srow, k, c0, c1, c2, c3);
+                    }
+                }
+                return len + 1;
+            }
             const RecD& p = cb[r];
             const RecD& q = cb[r + 1];
             const int row0 = clamp_row(rec_store_row(m0), maxrow), row1 = clamp_row(rec_store_row(q.meta), maxrow);
 #pragma unroll
             for (int k = 0; k < VPT; ++k) {
-                const double t0 = fma(w[k], p.c, fma(v[k], p.b, u[k] * p.a));
-                const double t1 = fma(w[k], q.c, fma(v[k], q.b, u[k] * q.a));
-                double s0, c0, s1, c1;
-                sincos_turns_f64(t0, s0, c0);
-                sincos_turns_f64(t1, s1, c1);
-                slot(row0, k) = make_double2(c0, s0);
-                slot(row1, k) = make_double2(c1, s1);
+                double2 e0, e1;
+                wave(p, k, e0);
+                wave(q, k, e1);
+                slot(row0, k) = e0;
+                slot(row1, k) = e1;
             }
             return 2;
         }
@@ -107,20 +167,7 @@ struct Eq17D {
                 if (mask & 2u) c1 = slot(crow + 1, k);
                 if (mask & 4u) c2 = slot(crow + 2, k);
                 if (mask & 8u) c3 = slot(crow + 3, k);
-                const double ar = c0.x + c1.x, ai = c0.y + c1.y;   // c0 + c1
-                const double br = c0.x - c1.x, bi = c0.y - c1.y;   // c0 - c1
-                const double cr = c2.x + c3.x, ci = c2.y + c3.y;   // c2 + c3
-                const double dr = c2.x - c3.x, di = c2.y - c3.y;   // c2 - c3
-                const double er = ar + cr, ei = ai + ci;           // Eq. 9 form (times 4^(J-j))
-                // Eq. 10 rows (+ - + -), (+ + - -), (+ - - +), weighted by gamma
-                vr[k] = fma(r.a, br + dr, fma(r.b, ar - cr, fma(r.c, br - dr, vr[k])));
-                vi[k] = fma(r.a, bi + di, fma(r.b, ai - ci, fma(r.c, bi - di, vi[k])));
-                if (root) {
-                    vr[k] = fma(r.e, er, vr[k]);
-                    vi[k] = fma(r.e, ei, vi[k]);
-                } else {
-                    slot(srow, k) = make_double2(er, ei);
-                }
+                node(r, root, srow, k, c0, c1, c2, c3);
             }
         }
     }
