@@ -1,5 +1,5 @@
 """Loss and gradient of the response network at the edges of the training
-kernel's 32- and 64-sample tiles and of its grid, against float64 with the two
+kernel's 64-sample tiles and of its grid, against float64 with the two
 documented bfloat16 roundings (W2 and the first hidden layer).
 
 Tolerance. The kernel's float32 sums err by 1e-6 at most; what dominates is a
