@@ -306,8 +306,7 @@ int set_attr_pass(int shape, size_t smem)
         case 4: fn = reinterpret_cast<const void*>(k_batched<32, 1, KIND, FAST, GRIDPASS>); break;
         default: fn = reinterpret_cast<const void*>(k_batched<32, 2, KIND, FAST, GRIDPASS>); break;
     }
-    WT_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    return WT_OK;
+    return allow_dynamic_smem(fn, smem);
 }
 
 template <int KIND, bool FAST = false>

@@ -326,7 +326,8 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
 template <class K>
 int grid_for(K kernel, int threads, int nt, size_t smem, int64_t n_vis, dim3& grid)
 {
-    WT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    const int rc = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+    if (rc) return rc;
     int per_sm = 0;
     WT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) return set_error(WT_ERR_UNSUPPORTED, "dft kernel does not fit on an SM");

@@ -576,7 +576,8 @@ int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks
     size_t smem = need;
     int per_sm = 0;
     for (;;) {
-        WT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        const int rc = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+        if (rc) return rc;
         WT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTcThreads, smem));
         if (per_sm < 1) return set_error(WT_ERR_UNSUPPORTED, "%s: tensor-core kernel does not fit on an SM", fn);
         if (per_sm * tc_tmem_cols(TILES) <= 512) break;

@@ -1089,8 +1089,9 @@ int persistent_grid(int n, size_t* smem)
     int occ = 0;
     if (cudaFuncGetAttributes(&fa, k_hogbom_persistent) != cudaSuccess ||
         bytes + fa.sharedSizeBytes > static_cast<size_t>(optin) ||
+        // (the same limit from every thread: allow_dynamic_smem)
         cudaFuncSetAttribute(k_hogbom_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(bytes)) != cudaSuccess ||
+                             optin - static_cast<int>(fa.sharedSizeBytes)) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hogbom_persistent, kHogThreads, bytes) != cudaSuccess ||
         static_cast<int64_t>(occ) * sms < G) {
         cudaGetLastError();

@@ -303,7 +303,8 @@ struct Variant {
 template <class K>
 int prepare(K kernel, int nt, size_t smem, int64_t per_tile, int64_t n_vis, dim3& grid)
 {
-    WT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    const int rc = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+    if (rc) return rc;
     int per_sm = 0;
     WT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem));
     if (per_sm < 1) return set_error(WT_ERR_UNSUPPORTED, "wavelet kernel does not fit on an SM (smem %zu)", smem);

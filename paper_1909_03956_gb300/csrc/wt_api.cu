@@ -158,6 +158,13 @@ int num_sms()
     return g_sms[dev];
 }
 
+int allow_dynamic_smem(const void* kernel, size_t smem)
+{
+    const size_t limit = smem > kMostDynamicSmem ? smem : kMostDynamicSmem;
+    WT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(limit)));
+    return WT_OK;
+}
+
 // A pointer the kernels will dereference must be device (or managed) memory
 // of the current device, and [p, p + bytes) must lie inside its allocation.
 int check_device_buffer(const void* p, size_t bytes, const char* fn, const char* name, size_t align)

@@ -769,6 +769,12 @@ int predict_dft(const double* l, const double* m, const double* flux, int64_t n_
 int subtract(const void* obs, const void* model, void* resid, int64_t n_vis, int mode, cudaStream_t s);
 // utilities
 int num_sms();
+// Lets a launch of `kernel` take `smem` bytes of dynamic shared memory. The
+// limit belongs to the function, not to the launch: two host threads that each
+// set their own size could refuse each other's launches. So every caller sets
+// the same, all that a CTA may have beside 1 KB for the kernel's own variables.
+constexpr size_t kMostDynamicSmem = 226 * 1024;
+int allow_dynamic_smem(const void* kernel, size_t smem);
 inline dim3 exact_grid(dim3 grid)
 {
     const unsigned most = static_cast<unsigned>(num_sms()) * kExactCtasPerSm;
