@@ -174,12 +174,20 @@ constexpr int kChunkDirDF = 128;   // records per staging buffer beside the 16 K
 // the terms are then cut into parts, a CTA per (tile, part) on grid.y, each
 // writing its sum to its own row of a workspace, and k_sum_parts adds the rows
 // in order (in float64): 1.46 ms. 780 visibilities x 3 760 components on the
-// special-function unit: 377 -> 40 us. The part's share of the list:
-__device__ __forceinline__ int64_t part_from(int64_t per_part) { return static_cast<int64_t>(blockIdx.y) * per_part; }
-__device__ __forceinline__ int64_t part_count(int64_t n_terms, int64_t per_part)
+// special-function unit: 377 -> 40 us. CUT: the kernel takes its part of the
+// list; a list that is not cut runs the kernel without this (20 components, 3.9 M
+// visibilities: 2.5 % of the double-float form, 1.2 of the polynomial mixed one).
+template <bool CUT, class Rec, class C>
+__device__ __forceinline__ void take_part(const Rec* __restrict__& recs, int64_t& n_terms, int64_t per_part,
+                                          C* __restrict__& vis, int64_t n_vis)
 {
-    const int64_t n = n_terms - part_from(per_part);
-    return n < 0 ? 0 : n < per_part || blockIdx.y + 1 == gridDim.y ? n : per_part;   // the last takes the rest
+    if constexpr (CUT) {
+        const int64_t from = static_cast<int64_t>(blockIdx.y) * per_part;
+        recs += from;
+        n_terms = max(n_terms - from, int64_t(0));
+        if (blockIdx.y + 1 < gridDim.y) n_terms = min(n_terms, per_part);   // the last takes the rest
+        vis += blockIdx.y * n_vis;
+    }
 }
 
 __device__ __forceinline__ double2 to_c128(double2 x) { return x; }
@@ -206,15 +214,15 @@ __global__ void k_sum_parts(const C* __restrict__ partial, int parts, int64_t n_
     from_c128(a, vis[i]);
 }
 
-template <int NT>
+template <int NT, bool CUT>
 __global__ void __launch_bounds__(NT) k_dft_df(const CompF* __restrict__ comps, int64_t n_comp, int64_t per_part,
                                                const double* __restrict__ uvw, int64_t n_vis,
                                                double2* __restrict__ vis, double sgn, int* status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    vis += blockIdx.y * n_vis;
+    take_part<CUT>(comps, n_comp, per_part, vis, n_vis);
     Stager<CompF> st;
-    stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunkDirDF);
+    stager_setup(st, smem, comps, n_comp, kChunkDirDF);
     float4* tab = reinterpret_cast<float4*>(smem + stager_bytes<CompF>(kChunkDirDF));
     load_sincos_table_df(tab);
     __syncthreads();
@@ -240,15 +248,15 @@ __global__ void __launch_bounds__(NT) k_dft_df(const CompF* __restrict__ comps, 
     }
 }
 
-template <int NT>
+template <int NT, bool CUT>
 __global__ void __launch_bounds__(NT) k_dft_fp64(const CompD* __restrict__ comps, int64_t n_comp, int64_t per_part,
                                                  const double* __restrict__ uvw, int64_t n_vis,
                                                  double2* __restrict__ vis, double sgn, int* status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    vis += blockIdx.y * n_vis;
+    take_part<CUT>(comps, n_comp, per_part, vis, n_vis);
     Stager<CompD> st;
-    stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunk);
+    stager_setup(st, smem, comps, n_comp, kChunk);
     const int64_t ntiles = (n_vis + NT - 1) / NT;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t n = tile * NT + threadIdx.x;
@@ -268,7 +276,7 @@ __global__ void __launch_bounds__(NT) k_dft_fp64(const CompD* __restrict__ comps
 // the head grid is swept too, its results discarded, and marked for the
 // exact pass); else the exact pass (only the marked tiles). bound: the
 // records' coordinate bounds (k_pack_components).
-template <int NT, bool FAST, bool GRIDPASS>
+template <int NT, bool FAST, bool GRIDPASS, bool CUT>
 __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comps, int64_t n_comp, int64_t per_part,
                                                   const uint32_t* __restrict__ bound,
                                                   const double* __restrict__ uvw, int64_t n_vis,
@@ -278,9 +286,9 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
     if constexpr (!GRIDPASS) {
         if (!any_deferred(reinterpret_cast<const float*>(bound))) return;
     }
-    vis += blockIdx.y * n_vis;
+    take_part<CUT>(comps, n_comp, per_part, vis, n_vis);
     Stager<CompF> st;
-    stager_setup(st, smem, comps + part_from(per_part), part_count(n_comp, per_part), kChunk);
+    stager_setup(st, smem, comps, n_comp, kChunk);
     const int64_t ntiles = (n_vis + 2 * NT - 1) / (2 * NT);
     const double sg = static_cast<double>(sgn);       // sign folded into the baseline (exact)
     float smax[3] = {0.f, 0.f, 0.f};
@@ -401,7 +409,7 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
     if (mode == WT_FP64) {
         constexpr int NT = 128;
         const size_t smem = static_cast<size_t>(stager_bytes<CompD>(kChunk));
-        auto k = k_dft_fp64<NT>;
+        auto k = tp.parts > 1 ? k_dft_fp64<NT, true> : k_dft_fp64<NT, false>;
         int rc = grid_for(k, NT, NT, smem, n_vis, grid);
         if (rc) return rc;
         grid.y = static_cast<unsigned>(tp.parts);
@@ -410,7 +418,7 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
     } else if (mode == WT_FP64_DF) {
         constexpr int NT = 64;
         const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunkDirDF)) + kDfTableEntries * sizeof(float4);
-        auto k = k_dft_df<NT>;
+        auto k = tp.parts > 1 ? k_dft_df<NT, true> : k_dft_df<NT, false>;
         int rc = grid_for(k, NT, 2 * NT, smem, n_vis, grid);
         if (rc) return rc;
         grid.y = static_cast<unsigned>(tp.parts);
@@ -421,8 +429,13 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
         constexpr int NT = 256;
         const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunk));
         const bool fast = mode == WT_MIXED_FAST;
-        auto kg = fast ? k_dft_mixed<NT, true, true> : k_dft_mixed<NT, false, true>;
-        auto ke = fast ? k_dft_mixed<NT, true, false> : k_dft_mixed<NT, false, false>;
+        const bool cut = tp.parts > 1;
+        auto kg = fast ? cut ? k_dft_mixed<NT, true, true, true> : k_dft_mixed<NT, true, true, false>
+                  : cut ? k_dft_mixed<NT, false, true, true>
+                        : k_dft_mixed<NT, false, true, false>;
+        auto ke = fast ? cut ? k_dft_mixed<NT, true, false, true> : k_dft_mixed<NT, true, false, false>
+                  : cut ? k_dft_mixed<NT, false, false, true>
+                        : k_dft_mixed<NT, false, false, false>;
         dim3 grid_e;
         int rc = grid_for(kg, NT, 2 * NT, smem, n_vis, grid);   // two visibilities per thread
         if (!rc) rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid_e);
@@ -448,7 +461,7 @@ int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, 
 {
     constexpr int NT = 64;
     const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunk));
-    auto ke = k_dft_mixed<NT, true, false>;
+    auto ke = tp.parts > 1 ? k_dft_mixed<NT, true, false, true> : k_dft_mixed<NT, true, false, false>;
     dim3 grid;
     int rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid);
     if (rc) return rc;
