@@ -22,7 +22,7 @@ namespace wt {
 // dft_tc.cu: the tensor-core form (WT_MIXED_TC)
 size_t dft_tc_scratch_bytes(int64_t n_comp);
 int dft_tc_launch(const double* l, const double* m, const double* flux, int64_t n_comp, const void* recs,
-                  const uint32_t* bound, void* tc, const TermParts& tp, const double* uvw, int64_t n_vis, float2* vis,
+                  const uint32_t* bound, void* tc, const TermParts& tp, const double* uvw, int64_t n_vis, void* vis,
                   int sign, int* status, cudaStream_t s);
 int64_t dft_tc_tiles(int64_t n_vis, int64_t n_comp);
 
@@ -190,28 +190,21 @@ __device__ __forceinline__ void take_part(const Rec* __restrict__& recs, int64_t
     }
 }
 
-__device__ __forceinline__ double2 to_c128(double2 x) { return x; }
-__device__ __forceinline__ double2 to_c128(float2 x) { return make_double2(x.x, x.y); }
-__device__ __forceinline__ void from_c128(double2 x, double2& y) { y = x; }
-__device__ __forceinline__ void from_c128(double2 x, float2& y)
-{
-    y = make_float2(static_cast<float>(x.x), static_cast<float>(x.y));
-}
-
 // vis[i] = sum over p of partial[p][i], in order, in float64.
 template <class C>
-__global__ void k_sum_parts(const C* __restrict__ partial, int parts, int64_t n_vis, C* __restrict__ vis)
+__global__ void k_sum_parts(const double2* __restrict__ partial, int parts, int64_t n_vis, C* __restrict__ vis)
 {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n_vis) return;
     double2 a = make_double2(0.0, 0.0);
 #pragma unroll 4
     for (int p = 0; p < parts; ++p) {
-        const double2 x = to_c128(partial[p * n_vis + i]);
+        const double2 x = partial[p * n_vis + i];
         a.x += x.x;
         a.y += x.y;
     }
-    from_c128(a, vis[i]);
+    vis[i].x = static_cast<decltype(vis[i].x)>(a.x);
+    vis[i].y = static_cast<decltype(vis[i].y)>(a.y);
 }
 
 template <int NT, bool CUT>
@@ -280,7 +273,7 @@ template <int NT, bool FAST, bool GRIDPASS, bool CUT>
 __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comps, int64_t n_comp, int64_t per_part,
                                                   const uint32_t* __restrict__ bound,
                                                   const double* __restrict__ uvw, int64_t n_vis,
-                                                  float2* __restrict__ vis, float sgn, int* status)
+                                                  MixedOut<CUT>* __restrict__ vis, float sgn, int* status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     if constexpr (!GRIDPASS) {
@@ -298,7 +291,7 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
         smax[2] = __uint_as_float(bound[2]);
     }
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        float2* first_vis = vis + tile * 2 * NT;
+        float2* first_vis = reinterpret_cast<float2*>(vis + tile * 2 * NT);
         if constexpr (!GRIDPASS) {
             if (!tile_deferred(first_vis)) continue;   // done by the grid pass
         }
@@ -326,8 +319,8 @@ __global__ void __launch_bounds__(NT) k_dft_mixed(const CompF* __restrict__ comp
             mark_deferred(first_vis, reinterpret_cast<const float*>(bound));
             continue;
         }
-        if (ok0) vis[n0] = sub2(b.acc[0], b.comp[0]);
-        if (ok1) vis[n1] = sub2(b.acc[1], b.comp[1]);
+        if (ok0) store_sum(vis[n0], b.acc[0], b.comp[0]);
+        if (ok1) store_sum(vis[n1], b.acc[1], b.comp[1]);
     }
 }
 
@@ -389,19 +382,17 @@ int sum_parts(const void* partial, const TermParts& tp, int64_t n_vis, void* vis
 {
     const unsigned blocks = static_cast<unsigned>((n_vis + 127) / 128);
     const int parts = static_cast<int>(tp.parts);
-    if (c128)
-        k_sum_parts<<<blocks, 128, 0, s>>>(static_cast<const double2*>(partial), parts, n_vis,
-                                           static_cast<double2*>(vis));
-    else
-        k_sum_parts<<<blocks, 128, 0, s>>>(static_cast<const float2*>(partial), parts, n_vis,
-                                           static_cast<float2*>(vis));
+    const double2* x = static_cast<const double2*>(partial);
+    if (c128) k_sum_parts<<<blocks, 128, 0, s>>>(x, parts, n_vis, static_cast<double2*>(vis));
+    else k_sum_parts<<<blocks, 128, 0, s>>>(x, parts, n_vis, static_cast<float2*>(vis));
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;
 }
 
 // Launch the DFT on component records already packed in `scratch`
 // (n_comp records of 32 bytes, 256-byte aligned) with their coordinate
-// bounds at `bound` (mixed forms); errors go to `status`. vis: [tp.parts][n_vis].
+// bounds at `bound` (mixed forms); errors go to `status`. vis: the
+// visibilities, or the parts' sums [tp.parts][n_vis], complex128 in every mode.
 int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp, const TermParts& tp,
                       const double* uvw, int64_t n_vis, void* vis, int mode, int sign, int* status, cudaStream_t s)
 {
@@ -428,25 +419,29 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
         // the grid pass, then the exact pass over the tiles it left marked
         constexpr int NT = 256;
         const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunk));
-        const bool fast = mode == WT_MIXED_FAST;
-        const bool cut = tp.parts > 1;
-        auto kg = fast ? cut ? k_dft_mixed<NT, true, true, true> : k_dft_mixed<NT, true, true, false>
-                  : cut ? k_dft_mixed<NT, false, true, true>
-                        : k_dft_mixed<NT, false, true, false>;
-        auto ke = fast ? cut ? k_dft_mixed<NT, true, false, true> : k_dft_mixed<NT, true, false, false>
-                  : cut ? k_dft_mixed<NT, false, false, true>
-                        : k_dft_mixed<NT, false, false, false>;
-        dim3 grid_e;
-        int rc = grid_for(kg, NT, 2 * NT, smem, n_vis, grid);   // two visibilities per thread
-        if (!rc) rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid_e);
-        if (rc) return rc;
-        grid.y = grid_e.y = static_cast<unsigned>(tp.parts);
         const CompF* recs = static_cast<const CompF*>(scratch);
-        float2* out = static_cast<float2*>(vis);
-        kg<<<grid, NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign), status);
-        WT_CUDA_TRY(cudaGetLastError());
-        ke<<<exact_grid(grid_e), NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign),
-                                    status);
+        auto both = [&](auto kg, auto ke, auto* out) {
+            dim3 grid_e;
+            int rc = grid_for(kg, NT, 2 * NT, smem, n_vis, grid);   // two visibilities per thread
+            if (!rc) rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid_e);
+            if (rc) return rc;
+            grid.y = grid_e.y = static_cast<unsigned>(tp.parts);
+            kg<<<grid, NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out, static_cast<float>(sign),
+                                      status);
+            WT_CUDA_TRY(cudaGetLastError());
+            ke<<<exact_grid(grid_e), NT, smem, s>>>(recs, n_comp, tp.per_part, bound, uvw, n_vis, out,
+                                                    static_cast<float>(sign), status);
+            return static_cast<int>(WT_OK);
+        };
+        const bool fast = mode == WT_MIXED_FAST;
+        auto* sums = static_cast<double2*>(vis);
+        auto* out = static_cast<float2*>(vis);
+        const int rc =
+            tp.parts > 1 ? fast ? both(k_dft_mixed<NT, true, true, true>, k_dft_mixed<NT, true, false, true>, sums)
+                                : both(k_dft_mixed<NT, false, true, true>, k_dft_mixed<NT, false, false, true>, sums)
+            : fast ? both(k_dft_mixed<NT, true, true, false>, k_dft_mixed<NT, true, false, false>, out)
+                   : both(k_dft_mixed<NT, false, true, false>, k_dft_mixed<NT, false, false, false>, out);
+        if (rc) return rc;
     }
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;
@@ -455,19 +450,24 @@ int dft_launch_packed(const void* scratch, const uint32_t* bound, int64_t n_comp
 // The exact pass of the mixed fast direct sum over 128-visibility tiles
 // (64 threads, two visibilities each): only the tiles whose first
 // visibility carries kDeferredMark are evaluated (the tensor-core form's
-// tiles beyond its range). vis: [tp.parts][n_vis].
+// tiles beyond its range). vis: as dft_launch_packed.
 int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, const TermParts& tp, const double* uvw,
-                       int64_t n_vis, float2* vis, int sign, int* status, cudaStream_t s)
+                       int64_t n_vis, void* vis, int sign, int* status, cudaStream_t s)
 {
     constexpr int NT = 64;
     const size_t smem = static_cast<size_t>(stager_bytes<CompF>(kChunk));
-    auto ke = tp.parts > 1 ? k_dft_mixed<NT, true, false, true> : k_dft_mixed<NT, true, false, false>;
-    dim3 grid;
-    int rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid);
+    auto exact = [&](auto ke, auto* out) {
+        dim3 grid;
+        const int rc = grid_for(ke, NT, 2 * NT, smem, n_vis, grid);
+        if (rc) return rc;
+        grid.y = static_cast<unsigned>(tp.parts);
+        ke<<<exact_grid(grid), NT, smem, s>>>(static_cast<const CompF*>(recs), n_comp, tp.per_part, bound, uvw, n_vis,
+                                              out, static_cast<float>(sign), status);
+        return static_cast<int>(WT_OK);
+    };
+    const int rc = tp.parts > 1 ? exact(k_dft_mixed<NT, true, false, true>, static_cast<double2*>(vis))
+                                : exact(k_dft_mixed<NT, true, false, false>, static_cast<float2*>(vis));
     if (rc) return rc;
-    grid.y = static_cast<unsigned>(tp.parts);
-    ke<<<exact_grid(grid), NT, smem, s>>>(static_cast<const CompF*>(recs), n_comp, tp.per_part, bound, uvw, n_vis, vis,
-                              static_cast<float>(sign), status);
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;
 }
@@ -502,7 +502,7 @@ int predict_dft(const double* l, const double* m, const double* flux, int64_t n_
     const size_t tc_bytes = tc ? (dft_tc_scratch_bytes(n_comp) + 255) / 256 * 256 : 0;
     const size_t base_bytes = rec_bytes + 256 + tc_bytes;
     const size_t part_bytes =
-        tp.parts > 1 ? static_cast<size_t>(tp.parts) * static_cast<size_t>(n_vis) * (c128 ? 16 : 8) : 0;
+        tp.parts > 1 ? static_cast<size_t>(tp.parts) * static_cast<size_t>(n_vis) * sizeof(double2) : 0;
     void* scratch = nullptr;
     cudaError_t e = cudaMallocAsync(&scratch, base_bytes + part_bytes, s);
     if (e != cudaSuccess) {
@@ -521,7 +521,7 @@ int predict_dft(const double* l, const double* m, const double* flux, int64_t n_
     if (rc == WT_OK) {
         if (tc)
             rc = dft_tc_launch(l, m, flux, n_comp, scratch, bound, static_cast<unsigned char*>(scratch) + rec_bytes + 256,
-                               tp, uvw, n_vis, static_cast<float2*>(out), sign, status, s);
+                               tp, uvw, n_vis, out, sign, status, s);
         else
             rc = dft_launch_packed(scratch, bound, n_comp, tp, uvw, n_vis, out, mode, sign, status, s);
     }

@@ -62,7 +62,7 @@ namespace wt {
 // dft.cu: the exact pass of the mixed direct sum over 128-visibility tiles
 // marked by mark_deferred.
 int dft_exact_pass_128(const void* recs, const uint32_t* bound, int64_t n_comp, const TermParts& tp, const double* uvw,
-                       int64_t n_vis, float2* vis, int sign, int* status, cudaStream_t s);
+                       int64_t n_vis, void* vis, int sign, int* status, cudaStream_t s);
 
 namespace {
 
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kTcThreads) k_dft_tc(const unsigned char* __re
                                                       const int64_t* __restrict__ n_dev,
                                                       const uint32_t* __restrict__ bound,
                                                       const double* __restrict__ uvw, int64_t n_vis,
-                                                      float2* __restrict__ vis, float sgn, int* status)
+                                                      MixedOut<CUT>* __restrict__ vis, float sgn, int* status)
 {
     constexpr int kTcCtaVis = kTcRows * kTcTiles;                 // visibilities per CTA
     constexpr int kTcAcc = tc_acc_cols(kTcTiles);
@@ -386,7 +386,8 @@ __global__ void __launch_bounds__(kTcThreads) k_dft_tc(const unsigned char* __re
 #pragma unroll
             for (int q = 0; q < kTcTiles; ++q) {
                 const int64_t first = tile * kTcCtaVis + q * kTcRows;
-                if (first < n_vis) mark_deferred(vis + first, reinterpret_cast<const float*>(bound));
+                if (first < n_vis)
+                    mark_deferred(reinterpret_cast<float2*>(vis + first), reinterpret_cast<const float*>(bound));
             }
         }
         return;
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(kTcThreads) k_dft_tc(const unsigned char* __re
 #pragma unroll
             for (int q = 0; q < kTcTiles; ++q) {
                 const int64_t n = tile * kTcCtaVis + q * kTcRows + t;
-                if (n < n_vis) vis[n] = sub2(acc[q], cmp[q]);
+                if (n < n_vis) store_sum(vis[n], acc[q], cmp[q]);
             }
         }
     }
@@ -564,12 +565,12 @@ size_t dft_tc_scratch_bytes(int64_t n_comp)
 
 namespace {
 
-template <int TILES>
+template <int TILES, bool CUT>
 int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks, int64_t stages,
-                    const TermParts& tp, const int64_t* n_dev, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
-                    int sign, int* status, cudaStream_t s, const char* fn)
+                    const TermParts& tp, const int64_t* n_dev, const uint32_t* bound, const double* uvw, int64_t n_vis,
+                    void* vis, int sign, int* status, cudaStream_t s, const char* fn)
 {
-    auto kernel = tp.parts > 1 ? k_dft_tc<TILES, true> : k_dft_tc<TILES, false>;
+    auto kernel = k_dft_tc<TILES, CUT>;
     // no more CTAs per SM than their tensor memory allows (a CTA beyond
     // that would wait in tcgen05.alloc)
     const size_t need = 1024 + TILES * kTcRows * 128 + 2 * kTcStageBytes + 2 * kTcStageComps * 4;
@@ -587,8 +588,8 @@ int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks
     const int64_t tiles = (n_vis + cta_vis - 1) / cta_vis;
     if (tiles > 0x7fffffff) return set_error(WT_ERR_RANGE, "%s: too many visibilities for one launch", fn);
     kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(tp.parts)), kTcThreads, smem, s>>>(
-        bsl, bfl, n_chunks, stages, tp.per_part / kTcStageComps, n_dev, bound, uvw, n_vis, vis,
-        static_cast<float>(sign), status);
+        bsl, bfl, n_chunks, stages, tp.per_part / kTcStageComps, n_dev, bound, uvw, n_vis,
+        static_cast<MixedOut<CUT>*>(vis), static_cast<float>(sign), status);
     WT_CUDA_TRY(cudaGetLastError());
     return WT_OK;
 }
@@ -598,12 +599,14 @@ int tc_launch_tiles(const unsigned char* bsl, const float* bfl, int64_t n_chunks
 // need, when n_dev is given); chunks_hint, the chunks the host expects,
 // picks two tiles per CTA for a few hundred terms.
 int tc_main_launch(const unsigned char* bsl, const float* bfl, int64_t n_chunks, int64_t stages, const TermParts& tp,
-                   const int64_t* n_dev, int64_t chunks_hint, const uint32_t* bound, const double* uvw, int64_t n_vis, float2* vis,
-                   int sign, int* status, cudaStream_t s, const char* fn)
+                   const int64_t* n_dev, int64_t chunks_hint, const uint32_t* bound, const double* uvw, int64_t n_vis,
+                   void* vis, int sign, int* status, cudaStream_t s, const char* fn)
 {
-    if (chunks_hint <= kTcTwoTileMaxChunks)
-        return tc_launch_tiles<2>(bsl, bfl, n_chunks, stages, tp, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
-    return tc_launch_tiles<1>(bsl, bfl, n_chunks, stages, tp, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
+    const bool two = chunks_hint <= kTcTwoTileMaxChunks, cut = tp.parts > 1;
+    auto launch = two ? cut ? tc_launch_tiles<2, true> : tc_launch_tiles<2, false>
+                  : cut ? tc_launch_tiles<1, true>
+                        : tc_launch_tiles<1, false>;
+    return launch(bsl, bfl, n_chunks, stages, tp, n_dev, bound, uvw, n_vis, vis, sign, status, s, fn);
 }
 
 }  // namespace
@@ -621,7 +624,7 @@ static_assert(kTcStageComps == kPartTerms, "a part is whole stages");
 // 256-byte aligned) for the slices; then the exact pass over the tiles left
 // to it.
 int dft_tc_launch(const double* l, const double* m, const double* flux, int64_t n_comp, const void* recs,
-                  const uint32_t* bound, void* tc, const TermParts& tp, const double* uvw, int64_t n_vis, float2* vis,
+                  const uint32_t* bound, void* tc, const TermParts& tp, const double* uvw, int64_t n_vis, void* vis,
                   int sign, int* status, cudaStream_t s)
 {
     if (n_vis == 0) return WT_OK;
@@ -660,7 +663,7 @@ int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t
     // few visibilities: the terms cut by the count the host expects (the last
     // part takes whatever more there is)
     const TermParts tp = term_parts(dft_tc_tiles(n_vis, n_hint), n_hint, 4);
-    const size_t bytes = base + (tp.parts > 1 ? sizeof(float2) * static_cast<size_t>(tp.parts * n_vis) : 0);
+    const size_t bytes = base + (tp.parts > 1 ? sizeof(double2) * static_cast<size_t>(tp.parts * n_vis) : 0);
     unsigned char* scratch = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, s);
     if (e != cudaSuccess) {
@@ -669,7 +672,7 @@ int eq16_tc_launch(const RecF* recs, const TreeHeader* hdr, int64_t cap, int64_t
                          cudaGetErrorString(e));
     }
     CompF* exact = reinterpret_cast<CompF*>(scratch);
-    float2* out = tp.parts > 1 ? reinterpret_cast<float2*>(scratch + base) : vis;
+    void* out = tp.parts > 1 ? static_cast<void*>(scratch + base) : vis;
     unsigned char* bsl = scratch + ((exact_bytes + 255) / 256) * 256;
     float* bfl = reinterpret_cast<float*>(bsl + stages * kTcStageBytes);
     int rc = WT_OK;

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/wtvis.h"
 
 namespace wt {
@@ -502,6 +504,19 @@ constexpr int kSumBlock = 8;
 // stage of the tensor-core form's operand).
 constexpr int kPartTerms = 128;
 
+// What a mixed direct sum stores of a visibility's compensated sum: the sum
+// rounded to float32, or all of it where it is one part of several (CUT), which
+// are added in float64 and rounded once. A part's mark (mark_deferred) is the
+// float64 2^1021 or so, which no sum of float32 terms reaches.
+template <bool CUT>
+using MixedOut = std::conditional_t<CUT, double2, float2>;
+__device__ __forceinline__ void store_sum(float2& out, float2 sum, float2 comp) { out = sub2(sum, comp); }
+__device__ __forceinline__ void store_sum(double2& out, float2 sum, float2 comp)
+{
+    out = make_double2(static_cast<double>(sum.x) - static_cast<double>(comp.x),
+                       static_cast<double>(sum.y) - static_cast<double>(comp.y));
+}
+
 // Kahan-compensated sum of pairs (each element as kahan_add).
 __device__ __forceinline__ void kahan_add2(float2& sum, float2& comp, float2 x)
 {
@@ -764,6 +779,7 @@ struct TermParts {
     int64_t per_part;     // terms per part, a multiple of kPartTerms
 };
 TermParts term_parts(int64_t tiles, int64_t n_terms, int fill);
+// vis (complex128 or complex64) = the sum of partial[tp.parts][n_vis] (complex128)
 int sum_parts(const void* partial, const TermParts& tp, int64_t n_vis, void* vis, bool c128, cudaStream_t s);
 int predict_dft(const double* l, const double* m, const double* flux, int64_t n_comp, const double* uvw,
                 int64_t n_vis, void* vis, int mode, int sign, cudaStream_t s);
