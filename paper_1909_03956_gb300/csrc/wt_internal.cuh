@@ -180,7 +180,7 @@ __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, f
     c = ((qi + 1) & 2) ? -cc : cc;
 }
 
-// ---- float64 sin/cos of 2 pi t (t in turns, |t| < 2^40) ---------------------
+// ---- float64 sin/cos of 2 pi t (t in turns) ----------------------------------
 // Table-driven reduction (the table-lookup method of P. T. P. Tang, ACM TOMS
 // 15(2), 1989): k = rint(1024 t), f = t - k/1024 (exact, |f| <= 1/2048), and
 // exp(i 2 pi t) = exp(i 2 pi (k mod 1024)/1024) exp(i 2 pi f). The table holds
@@ -192,13 +192,32 @@ __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, f
 // neither a conversion nor a separate reduction of t by its nearest integer.
 // 13 operations of the float64 pipe, which bounds every kernel that calls it
 // (256 entries, with rint, a conversion to integer and one more term each: 18
-// and two conversions).
+// and two conversions). The sum holds k's low bits while |t| < 2^41; beyond,
+// t is brought down to 2^40 .. 2^41 first (turns_below_2_41).
 static __device__ const double2 kSinCos1024[1024] =
 #include "sincos_table.inc"
     ;
 
+// t modulo whole turns, exactly: from 2^41 up the bits worth 2^40 and more are
+// shifted out of the significand and the exponent set to 2^40's. Integer steps:
+// they cost the explicit Eq. 17 0.5 % and the other float64 sums nothing, where
+// two operations of the float64 pipe, which those fill (t - rint(t), taken or
+// not), cost the direct sum 12 %.
+__device__ __forceinline__ double turns_below_2_41(double t)
+{
+    const uint32_t over = (static_cast<uint32_t>(__double2hiint(t)) & 0x7fffffffu) - 0x42800000u;
+    if (over < 0x7ff00000u - 0x42800000u) {   // 2^41 <= |t|, finite
+        const int by = min(static_cast<int>(over >> 20) + 1, 52);
+        const uint64_t b = static_cast<uint64_t>(__double_as_longlong(t));
+        t = __longlong_as_double(static_cast<long long>((b & 0x8000000000000000ull) | 0x4270000000000000ull |
+                                                        ((b << by) & 0x000fffffffffffffull)));
+    }
+    return t;
+}
+
 __device__ __forceinline__ void sincos_turns_f64(double t, double& s, double& c)
 {
+    t = turns_below_2_41(t);
     constexpr double kMagic = 6597069766656.0;                      // 1.5 * 2^42
     const double m = __dadd_rn(t, kMagic);
     const double f = t - __dsub_rn(m, kMagic);                      // t - k/1024, exact
