@@ -26,7 +26,7 @@
 //   WT_FP64   float64 throughout; sin/cos by table-driven reduction
 //             (sincos_turns_f64, wt_internal.cuh).
 //   WT_MIXED  phase in double-float turns (float64-accurate), sin/cos of the
-//             reduced phase in float32 (Taylor series, wt_internal.cuh),
+//             reduced phase in float32 (polynomials, wt_internal.cuh),
 //             recursion in float32, Kahan-compensated float32 V.
 //   WT_MIXED_FAST  as WT_MIXED with sin/cos from the special-function unit.
 //   WT_FP64_DF     float64-class: phase, sin/cos (table method) and every

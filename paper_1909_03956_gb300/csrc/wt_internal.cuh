@@ -2,7 +2,7 @@
 //
 // Device helpers used by more than one kernel file: PTX wrappers for the
 // mbarrier / bulk-copy staging path, double-float arithmetic for the mixed
-// precision forms, a float32 sin/cos of 2*pi*t written from the Taylor series,
+// precision forms, a float32 sin/cos of 2*pi*t as polynomials,
 // the per-device status word, and the host-side error plumbing.
 #pragma once
 
@@ -150,14 +150,17 @@ __device__ __forceinline__ void phase_turns_df(F2 u, F2 v, F2 w, F2 su, F2 sv, F
 
 // sin and cos of 2*pi*(th + tl) for |th| <= 1/2 and small tl (turns),
 // float32. Quadrant reduction q = rint(4 th), f = (4 th - q) + 4 tl, the
-// first difference exact, so |f| <= 1/2 + 4|tl|; angle x = f * pi/2 (pi/2
-// rounded to float32: relative error 3e-8, below the float32 result's own
-// rounding); then sin to x^7 and cos to x^8 with the coefficients that
-// minimise the largest error on |x| <= 0.84 (Remez exchange; 7e-9 and 7e-10
-// with the coefficients rounded to float32, below float32 rounding; the
-// Taylor series need a term more each for as much).
-constexpr float kSinC3 = -0.1666664332151413f, kSinC5 = 0.00833156332373619f, kSinC7 = -0.0001944637333508581f;
-constexpr float kCosC4 = 0.04166663810610771f, kCosC6 = -0.0013886900851503015f, kCosC8 = 2.43866270466242e-05f;
+// first difference exact, so |f| <= 1/2 + 4|tl|; angle x = f * p with p = pi/2
+// rounded to float32 (2.8e-8 too large); then sin to x^7 and cos to x^8. Their
+// coefficients are the least-squares fit of sin and cos of f pi/2 over |f| <= 1/2
+// (a little beyond, for the tail) in powers of x, so that they take up p's
+// rounding where they can, moved by units in the last place to the smallest
+// error of the float32 evaluation. Over all quadrants the sine and cosine err by
+// 1.86e-8 RMS, 8.5e-8 at most; Taylor's coefficients with a term more in each
+// 2.03e-8 and 9.97e-8, minimax ones of these degrees for x itself 2.04e-8.
+constexpr float kSinC3 = -0.16666679084300995f, kSinC5 = 0.0083328485488891602f, kSinC7 = -0.00019572142628021538f;
+constexpr float kCosC2 = -0.49999997019767761f, kCosC4 = 0.041666626930236816f;
+constexpr float kCosC6 = -0.0013886927627027035f, kCosC8 = 2.4401293558184989e-05f;
 
 __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, float& c)
 {
@@ -170,7 +173,7 @@ __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, f
     const float sx = __fmaf_rn(__fmul_rn(x, x2), ps, x);
     float pc = __fmaf_rn(x2, kCosC8, kCosC6);
     pc = __fmaf_rn(x2, pc, kCosC4);
-    pc = __fmaf_rn(x2, pc, -0.5f);
+    pc = __fmaf_rn(x2, pc, kCosC2);
     const float cx = __fmaf_rn(x2, pc, 1.0f);
     const int qi = static_cast<int>(q) & 3;
     // angle = q * pi/2 + x
@@ -486,7 +489,7 @@ __device__ __forceinline__ void sincos_turns_f32x2(float2 h, float2 tl, float2& 
     const float2 sx = fma2(mul2(x, x2), ps, x);
     float2 pc = fma2(x2, bcast2(kCosC8), bcast2(kCosC6));
     pc = fma2(x2, pc, bcast2(kCosC4));
-    pc = fma2(x2, pc, bcast2(-0.5f));
+    pc = fma2(x2, pc, bcast2(kCosC2));
     const float2 cx = fma2(x2, pc, bcast2(1.0f));
     const int q0 = static_cast<int>(q.x) & 3, q1 = static_cast<int>(q.y) & 3;
     const float ss0 = (q0 & 1) ? cx.x : sx.x, cc0 = (q0 & 1) ? sx.x : cx.x;
