@@ -139,30 +139,41 @@ struct BodyDF {
     DF2 U, V, W;
     DFP vr, vi;
     const float4* tab;
-    __device__ __forceinline__ void term(const CompF& c)
+    static constexpr int kBlock = 4;   // (df_accumulate)
+    template <bool FIRST>
+    __device__ __forceinline__ void term(const CompF& c, DFP& br, DFP& bi) const
     {
         float2 th, tl;
         phase_turns_dfp(U, V, W, F2{c.lh, c.ll}, F2{c.mh, c.ml}, F2{c.nh, c.nl}, th, tl);
         DFP s, co;
         sincos_turns_dfp(th, tl, tab, s, co);
         const DFS f = dfs(c.flux, c.flux_lo);
-        dfp_accumulate_product(vr, f, co);
-        dfp_accumulate_product(vi, f, s);
+        if constexpr (FIRST) {
+            br = dfp_product(f, co);
+            bi = dfp_product(f, s);
+        } else {
+            dfp_accumulate_product(br, f, co);
+            dfp_accumulate_product(bi, f, s);
+        }
     }
-    // a block of components (kSumBlock, or what is left of a chunk), then the
-    // sums renormalised; returns how many
+    // a block of components (kBlock, or what is left of a chunk) into the sums;
+    // returns how many
     __device__ __forceinline__ int at(const CompF* cb, int r, int n)
     {
-        int taken = kSumBlock;
-        if (r + kSumBlock <= n) {
-#pragma unroll 4
-            for (int j = 0; j < kSumBlock; ++j) term(cb[r + j]);
+        DFP br, bi;
+        int taken = kBlock;
+        term<true>(cb[r], br, bi);
+        if (r + kBlock <= n) {
+#pragma unroll
+            for (int j = 1; j < kBlock; ++j) term<false>(cb[r + j], br, bi);
         } else {
             taken = n - r;
-            for (int j = r; j < n; ++j) term(cb[j]);
+            for (int j = r + 1; j < n; ++j) term<false>(cb[j], br, bi);
         }
-        dfp_renorm(vr);
-        dfp_renorm(vi);
+        dfp_renorm(br);
+        dfp_renorm(bi);
+        dfp_add_block(vr, br);
+        dfp_add_block(vi, bi);
         return taken;
     }
 };
