@@ -11,6 +11,7 @@
 #include <mutex>
 #include <vector>
 
+#include "kept.h"
 #include "wt_internal.cuh"
 
 namespace wt {
@@ -221,48 +222,20 @@ namespace {
 
 // Pinned header copies of freed trees, kept for the next ones (allocating and
 // freeing pinned memory, with a second wait for the stream, took 340 of the 500
-// us of a small major cycle): at most kKeptHeaders, each of the context it was
-// allocated in; one of a context that is gone is dropped with it. A header is
-// given back only after its tree's stream has been waited for, so no copy into
-// it is pending.
-constexpr size_t kKeptHeaders = 32;
-struct KeptHeader {
-    TreeHeader* p;
-    uint64_t ctx;
-};
-std::mutex g_hdr_mu;
-std::vector<KeptHeader> g_hdrs;
+// us of a small major cycle). A header is given back only after its tree's stream
+// has been waited for, so no copy into it is pending. `device` is current.
+wt::Kept g_hdrs;
 
-TreeHeader* take_header(cudaError_t* e)
+TreeHeader* take_header(int device, cudaError_t* e)
 {
-    const uint64_t ctx = wt::current_context_id();
-    {
-        std::lock_guard<std::mutex> lk(g_hdr_mu);
-        for (size_t i = g_hdrs.size(); i-- > 0;)
-            if (g_hdrs[i].ctx == ctx) {
-                TreeHeader* p = g_hdrs[i].p;
-                g_hdrs.erase(g_hdrs.begin() + static_cast<std::ptrdiff_t>(i));
-                return p;
-            }
-    }
-    TreeHeader* p = nullptr;
-    *e = cudaMallocHost(reinterpret_cast<void**>(&p), sizeof(TreeHeader));
-    return *e == cudaSuccess ? p : nullptr;
+    void* p = g_hdrs.take(device, wt::current_context_id());
+    if (!p) *e = cudaMallocHost(&p, sizeof(TreeHeader));
+    return *e == cudaSuccess ? static_cast<TreeHeader*>(p) : nullptr;
 }
 
-void give_back_header(TreeHeader* p)
+void give_back_header(int device, TreeHeader* p)
 {
-    if (!p) return;
-    const uint64_t ctx = wt::current_context_id();
-    if (ctx != 0) {
-        std::lock_guard<std::mutex> lk(g_hdr_mu);
-        if (g_hdrs.size() == kKeptHeaders && g_hdrs.front().ctx != ctx) g_hdrs.erase(g_hdrs.begin());
-        if (g_hdrs.size() < kKeptHeaders) {
-            g_hdrs.push_back(KeptHeader{p, ctx});
-            return;
-        }
-    }
-    cudaFreeHost(p);
+    if (p && !g_hdrs.keep(device, wt::current_context_id(), p)) cudaFreeHost(p);
 }
 
 // A new tree handle built from `src` (checked by the caller).
@@ -283,7 +256,7 @@ int new_tree(const char* fn, const wt::KeySource& src, const double* flux, int64
     t->n_comp = n_comp;
     t->stream = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
-    t->host_hdr = take_header(&e);
+    t->host_hdr = take_header(t->device, &e);
     if (!t->host_hdr) {
         t->magic = 0;
         delete t;
@@ -292,7 +265,7 @@ int new_tree(const char* fn, const wt::KeySource& src, const double* flux, int64
     rc = wt::build_tree(src, flux, n_comp, ra0, dec0, J, t, t->stream);
     if (rc != WT_OK) {
         if (t->block) cudaFreeAsync(t->block, t->stream);
-        if (cudaStreamSynchronize(t->stream) == cudaSuccess) give_back_header(t->host_hdr);
+        if (cudaStreamSynchronize(t->stream) == cudaSuccess) give_back_header(t->device, t->host_hdr);
         else cudaFreeHost(t->host_hdr);
         t->magic = 0;
         delete t;
@@ -476,7 +449,7 @@ void wt_free_tree(wt_tree t)
     wt::batch_forget_tree(t);
     const bool quiet = cudaStreamSynchronize(t->stream) == cudaSuccess;
     if (t->block) cudaFreeAsync(t->block, t->stream);
-    if (quiet) give_back_header(t->host_hdr);
+    if (quiet) give_back_header(t->device, t->host_hdr);
     else if (t->host_hdr) cudaFreeHost(t->host_hdr);
     cudaGetLastError();
     if (prev >= 0 && prev != t->device) cudaSetDevice(prev);
