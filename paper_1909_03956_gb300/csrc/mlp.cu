@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train_grad(const float
     if (tid < 2) sm.b3[tid] = params[ob3 + tid];
     // gradients this thread sums over the CTA's tiles: its block of gW2; one
     // element of gW1 (tid < 192) or gb1 (the rest); one of gW3 (tid < 128) or
-    // gb2 (tid - 128 < 64) or gb3 (tid - 192 < 2); thread 0 the loss
+    // gb2 (tid - 128 < 64) or gb3 (tid - 192 < 2); thread 224 the loss
     float2 gW2[4][2];
 #pragma unroll
     for (int i = 0; i < 4; ++i) gW2[i][0] = gW2[i][1] = make_float2(0.f, 0.f);
