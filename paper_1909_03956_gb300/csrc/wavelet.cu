@@ -324,18 +324,22 @@ int prepare(K kernel, int nt, size_t smem, int64_t per_tile, int64_t n_vis, dim3
 // float64 pipe busy for the whole sweep. All the tiles take alike, so they run
 // in waves of SMs x resident CTAs and a wave's time goes with its CTAs per SM:
 // the last one, however few tiles are left to it, costs as much as the others.
-// More CTAs hide latency (a wave's time per CTA, measured: 1.09, 1.035 and 1 at
-// two, three and four), fewer make finer waves; the count with the smallest
-// product. 201 563 visibilities (3 150 tiles; J = 12): four CTAs 13.6 ms in six
-// waves, three 12.3 in seven.
+// More CTAs hide latency (a wave's time per CTA, measured over many whole waves:
+// 2.2 to 2.5, 1.16 to 1.36 and 1.01 to 1.07 at one, two and three of four's time,
+// from J = 14 and 12 to J = 6, and 1.00 to 0.97 from five up), fewer make finer
+// waves; the count, up to what fits (three at J = 14, eight at J = 6), with the
+// smallest product. Over J = 6 .. 14 and 344 .. 18 240 tiles it comes within 0.6 %
+// of the best count on average, 6 % at worst; always the most that fit, 2.1 % and
+// 26 %. 3 150 tiles at J = 12: four CTAs 4.56 ms, three 4.48; 1 000 tiles at J = 14:
+// three 2.12 ms, two 2.59.
 int fp64_resident(int64_t tiles, int most)
 {
-    static const double per_cta[] = {0.0, 2.04, 1.088, 1.035, 1.0};
+    static const double per_cta[] = {0.0, 2.3, 1.22, 1.02};   // 1 from four up
     int best = most;
     double least = 1e300;
-    for (int r = most < 4 ? most : 4; r >= 1; --r) {
+    for (int r = most; r >= 1; --r) {
         const int64_t wave = static_cast<int64_t>(num_sms()) * r;
-        const double time = static_cast<double>((tiles + wave - 1) / wave * r) * per_cta[r];
+        const double time = static_cast<double>((tiles + wave - 1) / wave * r) * (r < 4 ? per_cta[r] : 1.0);
         if (time < least) {
             least = time;
             best = r;
