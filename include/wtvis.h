@@ -367,7 +367,7 @@ int wt_dirty_image_w(const double* uvw, const void* vis, int64_t n_vis, int n, d
  *   n_comp     device int32: the number of components recorded
  * gain in (0, 1]. Asynchronous. When the image's rows fit in shared memory
  * across the GPU's CTAs (n up to about 2700 on 152 SMs) the whole clean is
- * one cooperative launch whose CTAs meet at a grid barrier per iteration
+ * one cooperative launch whose CTAs meet once for up to 64 components
  * (bounded waits: WT_ERR_TIMEOUT in the device status word if one runs out,
  * the image and the components then undefined); otherwise one launch per
  * iteration. WT_HOGBOM=launches in the environment forces the latter. The
@@ -557,7 +557,7 @@ int wt_selftest_bounded_wait(uint32_t spin_limit, void* stream);
 
 /* Failure-detection self-test of the grid barrier of the persistent Hogbom
  * clean (wt_hogbom): a two-CTA cooperative launch meets at a barrier that
- * never opens (its arrival count starts past the grid size); each CTA gives
+ * never opens (it waits for one arrival more than the grid makes); each CTA gives
  * up after spin_limit (1..65536) polls and WT_ERR_TIMEOUT is recorded in the
  * device status word. The kernel returns normally; read the outcome with
  * wt_device_status(). WT_ERR_UNSUPPORTED without cooperative launches. */

@@ -428,11 +428,14 @@ __device__ __noinline__ void wp_spread_ties(const WpPlan& pl, const float2* __re
 // the layout) and two 8-byte additions to the grid, all in whole lines. Medium
 // array, 1 008 000 visibilities, 2048 x 2048, 64 planes: 0.73 ms, against 3.0
 // when each entry read the table across its rows and added 4 bytes at a time.
-// One entry per pair and the image doubled, runs of neighbouring visibilities
-// to a warp, take 0.44 ms, but change the order of the cells' float32 sums: a
-// thousand additions of like sign round to 1.4e-4 of the image (the correction
-// in its corners is 1 / c^2 = 2 900), differently in each order. This order
-// keeps images as they have been, to 4e-5.
+// The visibilities are dealt to the warps in a fixed interleaving, but a cell's
+// float32 sum takes them as the warps reach it: two runs on the same input differ
+// (by 1.5e-5 of the image, RMS; 2e-7 to 3.4e-5 over other sizes, where the error
+// against float64 is 7e-5, and 1e-5 to 2.2e-4: a thousand additions of like sign
+// under a correction of 1 / c^2 = 2 900 in the corners). One entry per pair and the
+// image doubled, runs of neighbouring visibilities to a warp, take 0.44 ms and are
+// no less accurate, but put like visibilities next to one another in the sums and
+// so move images by up to 1.4e-4, beyond what runs differ by: not taken.
 __global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __restrict__ K,
                                                     const double* __restrict__ uvw, const float2* __restrict__ vis,
                                                     int64_t n_vis, int n, double inv_du,
@@ -527,9 +530,11 @@ __global__ void __launch_bounds__(256) k_grid_wproj(WpPlan pl, const float2* __r
     if (threadIdx.x == 0 && blk) atomicAdd(count, static_cast<unsigned long long>(blk));
 }
 
-// Real part of the transformed grid, times (-1)^(ix+iy) / (W c(t) c(s)), the correction's product in double-float.
-// Bound by HBM (12 bytes per pixel); with both tapers evaluated per pixel in
-// float64 714 us at 2048 x 2048, 23 us so.
+// Real part of the transformed grid, times (-1)^(ix+iy) / (W c(t) c(s)), the
+// correction's product in double-float: of 2e8 pixels four round to a float32
+// other than the float64 quotient's, by a unit in the last place. Bound by HBM (12
+// bytes per pixel): 23 us at 2048 x 2048, 46 with the product in float64, 714 with
+// both tapers evaluated per pixel.
 __global__ void k_image_from_fft_wp(const float2* __restrict__ f, int n, const unsigned long long* __restrict__ count,
                                     const F2* __restrict__ gc, float* __restrict__ image)
 {

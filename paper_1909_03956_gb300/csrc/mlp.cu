@@ -407,9 +407,10 @@ __device__ __forceinline__ void gemm_rows(const float (*a)[kLd], const float (*b
 // 4 ub .. 4 ub + 3, and units 4 sb .. by units 4 ub .. of gW2), so a summed
 // row costs a warp two 16-byte shared-memory wavefronts for 8 packed FMAs and
 // the products run on the FMA pipe; the activations of a block stay in its
-// thread from the forward to the backward pass. Bound by that pipe (3 x 2 048
-// cycles of a tile) and the barriers between the small steps: at 8 192
-// samples (128 tiles on 152 SMs) 16.9 us, against 62 us an element per thread.
+// thread from the forward to the backward pass. Bound by
+// the waits at the barriers between the small steps, with eight warps on an SM:
+// at 8 192 samples (128 tiles on 152 SMs) 16.9 us, of which that pipe is busy 3
+// (3 x 2 048 cycles of a tile); 62 us an element per thread.
 // Every sum keeps its order, so training is as it was, bit for bit. Tensor-core
 // fragments on exact bfloat16 operands, tiles of 32 samples and overlapping
 // launches make a step 11.9 us instead of 26 and the gradients as accurate, but
