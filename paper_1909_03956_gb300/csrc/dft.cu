@@ -139,7 +139,8 @@ struct BodyDF {
     DF2 U, V, W;
     DFP vr, vi;
     const float4* tab;
-    static constexpr int kBlock = 4;   // (df_accumulate)
+    // a block's terms (df_accumulate): kBlock, or fewer
+    static constexpr int kBlock = 4;
     template <bool FIRST>
     __device__ __forceinline__ void term(const CompF& c, DFP& br, DFP& bi) const
     {
@@ -156,22 +157,33 @@ struct BodyDF {
             dfp_accumulate_product(bi, f, s);
         }
     }
-    // a block of components (kBlock, or what is left of a chunk) into the sums;
-    // returns how many
+    // Two blocks side by side, or one of what is left of a chunk, into the sums;
+    // returns how many components.
     __device__ __forceinline__ int at(const CompF* cb, int r, int n)
     {
         DFP br, bi;
-        int taken = kBlock;
+        int taken = 2 * kBlock;
         term<true>(cb[r], br, bi);
-        if (r + kBlock <= n) {
+        if (r + 2 * kBlock <= n) {
+            DFP cr, ci;
+            term<true>(cb[r + kBlock], cr, ci);
 #pragma unroll
-            for (int j = 1; j < kBlock; ++j) term<false>(cb[r + j], br, bi);
+            for (int j = 1; j < kBlock; ++j) {
+                term<false>(cb[r + j], br, bi);
+                term<false>(cb[r + kBlock + j], cr, ci);
+            }
+            dfp_renorm(br);
+            dfp_renorm(bi);
+            dfp_renorm(cr);
+            dfp_renorm(ci);
+            dfp_accumulate(br, cr);
+            dfp_accumulate(bi, ci);
         } else {
-            taken = n - r;
-            for (int j = r + 1; j < n; ++j) term<false>(cb[j], br, bi);
+            taken = n - r < kBlock ? n - r : kBlock;
+            for (int j = 1; j < taken; ++j) term<false>(cb[r + j], br, bi);
+            dfp_renorm(br);
+            dfp_renorm(bi);
         }
-        dfp_renorm(br);
-        dfp_renorm(bi);
         dfp_add_block(vr, br);
         dfp_add_block(vi, bi);
         return taken;

@@ -631,10 +631,12 @@ struct Eq16DF<1> {
 
 // Regrouped Eq. 17 in double-float (WT_FP64_DF, RecWDF): V = sum_n w_n eta_n
 // with every quantity a double-float on the float32 pipe. Each node adds
-// its w eta to V as soon as its eta is known, sibling leaves and their parent as
-// one block (df_accumulate; the block itself not renormalised: over random trees
-// the error is 0.95e-15 of Sigma |w eta| RMS, 1.40 when every addition was
-// renormalised, 1.60 without blocks). Per visibility a thread keeps
+// its w eta to V as soon as its eta is known, in blocks (df_accumulate): a run of
+// sibling leaves and what follows it, up to the next run's first leaf, where the
+// block joins V beside that leaf's phase, which does not wait for it. Over random
+// trees the error is 0.70e-15 of Sigma |w eta| RMS (1.0 for 50 leaves, 1.3 for
+// isolated components at J = 12), 1.40 (1.36, 2.3) when every addition was
+// renormalised. Per visibility a thread keeps
 // the sum of the children's eta of the open level-j node (j = 1 .. J-2) in
 // shared-memory row j - 1; that of the open level-(J-1) node lives in
 // registers, so a leaf never touches shared memory. A node's eta is a quarter
@@ -648,8 +650,8 @@ struct Eq17DF {
     static constexpr int NP = VPT / 2;
     DF2 U[NP], V[NP], W[NP];
     DFP vr[NP], vi[NP];    // V
-    DFP br[NP], bi[NP];    // w eta of the open level-(J-1) node's children
-    DFP lr[NP], li[NP];    // their eta
+    DFP br[NP], bi[NP];    // the block's part of V
+    DFP lr[NP], li[NP];    // children's eta sum of the open level-(J-1) node
     float4* stk;           // shared stack + threadIdx.x; row stride VPT * NT
     const float4* tab;     // exp(i 2 pi k/1024), sincos_turns_dfp
     int J;
@@ -667,7 +669,11 @@ struct Eq17DF {
             vr[p] = vi[p] = br[p] = bi[p] = lr[p] = li[p] = dfp_zero();
         }
     }
-    __device__ __forceinline__ double2 result(int k) const { return dfp_vis(vr[k / 2], vi[k / 2], k & 1); }
+    __device__ __forceinline__ double2 result(int k) const
+    {
+        const double2 v = dfp_vis(vr[k / 2], vi[k / 2], k & 1), b = dfp_vis(br[k / 2], bi[k / 2], k & 1);
+        return make_double2(v.x + b.x, v.y + b.y);
+    }
 
     __device__ void operator()(const RecWDF& r)
     {
@@ -683,10 +689,9 @@ struct Eq17DF {
                 phase_turns_dfp(U[p], V[p], W[p], su, sv, sw, th, tl);
                 DFP s, c;
                 sincos_turns_dfp(th, tl, tab, s, c);
-                if (root) {
-                    dfp_add_block(vr[p], dfp_product(wgt, c));
-                    dfp_add_block(vi[p], dfp_product(wgt, s));
-                } else if (first) {
+                if (first) {           // (every leaf of level 1 is one)
+                    dfp_add_block(vr[p], br[p]);
+                    dfp_add_block(vi[p], bi[p]);
                     br[p] = dfp_product(wgt, c);
                     bi[p] = dfp_product(wgt, s);
                     lr[p] = c;
@@ -717,17 +722,8 @@ struct Eq17DF {
             }
             er = DFP{mul2(er.h, quarter), mul2(er.l, quarter)};
             ei = DFP{mul2(ei.h, quarter), mul2(ei.l, quarter)};
-            if (in_regs) {
-                dfp_accumulate_product(br[p], wgt, er);
-                dfp_accumulate_product(bi[p], wgt, ei);
-                dfp_add_block(vr[p], br[p]);
-                dfp_add_block(vi[p], bi[p]);
-            } else {
-                dfp_accumulate_product(vr[p], wgt, er);
-                dfp_accumulate_product(vi[p], wgt, ei);
-                dfp_renorm(vr[p]);
-                dfp_renorm(vi[p]);
-            }
+            dfp_accumulate_product(br[p], wgt, er);
+            dfp_accumulate_product(bi[p], wgt, ei);
             if (root) continue;
             float4& A = slot(par, 2 * p);
             float4& B = slot(par, 2 * p + 1);
@@ -765,7 +761,10 @@ struct Eq17DF<NT, 1> {
         w = w1[0];
         vr = vi = br = bi = lr = li = DF{0.f, 0.f};
     }
-    __device__ __forceinline__ double2 result(int) const { return make_double2(df_to_double(vr), df_to_double(vi)); }
+    __device__ __forceinline__ double2 result(int) const
+    {
+        return make_double2(df_to_double(vr) + df_to_double(br), df_to_double(vi) + df_to_double(bi));
+    }
 
     __device__ void operator()(const RecWDF& r)
     {
@@ -774,24 +773,24 @@ struct Eq17DF<NT, 1> {
         const bool root = meta & kRwRoot, first = meta & kRwFirst;
         const DF wgt{r.wh, r.wl};
         if (meta & kRwLeaf) {
+            // no branch (few visibilities, a warp or two per scheduler: a run's
+            // later leaves add an empty block beside the phase, which costs less
+            // than waiting for a branch's chain)
+            const DF none{0.f, 0.f};
+            df_add_block(vr, first ? br : none);
+            df_add_block(vi, first ? bi : none);
+            br = first ? none : br;
+            bi = first ? none : bi;
+            lr = first ? none : lr;
+            li = first ? none : li;
             float th, tl;
             phase_turns_df(u, v, w, F2{r.ah, r.al}, F2{r.bh, r.bl}, F2{r.ch, r.cl}, th, tl);
             DF s, c;
             sincos_turns_df(th, tl, tab, s, c);
-            if (root) {
-                df_add_block(vr, df_product(wgt, c));
-                df_add_block(vi, df_product(wgt, s));
-            } else if (first) {
-                br = df_product(wgt, c);
-                bi = df_product(wgt, s);
-                lr = c;
-                li = s;
-            } else {
-                df_accumulate_product(br, wgt, c);
-                df_accumulate_product(bi, wgt, s);
-                df_accumulate(lr, c.h, c.l);
-                df_accumulate(li, s.h, s.l);
-            }
+            df_accumulate_product(br, wgt, c);
+            df_accumulate_product(bi, wgt, s);
+            df_accumulate(lr, c.h, c.l);
+            df_accumulate(li, s.h, s.l);
             return;
         }
         const int own = clamp_row(static_cast<uint32_t>(lev > 1 ? lev - 1 : 0), maxrow);
@@ -800,17 +799,13 @@ struct Eq17DF<NT, 1> {
         if (lev == J - 1) {
             er = df_scale(lr, 0.25f);
             ei = df_scale(li, 0.25f);
-            df_accumulate_product(br, wgt, er);
-            df_accumulate_product(bi, wgt, ei);
-            df_add_block(vr, br);
-            df_add_block(vi, bi);
         } else {
             const float4 S = slot(own);
             er = DF{0.25f * S.x, 0.25f * S.y};
             ei = DF{0.25f * S.z, 0.25f * S.w};
-            df_add_block(vr, df_product(wgt, er));
-            df_add_block(vi, df_product(wgt, ei));
         }
+        df_accumulate_product(br, wgt, er);
+        df_accumulate_product(bi, wgt, ei);
         if (root) return;
         float4& P = slot(par);
         if (first) {
