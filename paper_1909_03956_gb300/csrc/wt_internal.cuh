@@ -195,36 +195,31 @@ __device__ __forceinline__ void sincos_turns_f32(float th, float tl, float& s, f
 // neither a conversion nor a separate reduction of t by its nearest integer.
 // 13 operations of the float64 pipe, which bounds every kernel that calls it
 // (256 entries, with rint, a conversion to integer and one more term each: 18
-// and two conversions). The sum holds k's low bits while |t| < 2^41; beyond,
-// t is brought down to 2^40 .. 2^41 first (turns_below_2_41).
+// and two conversions). The sum holds k's low bits while |t| < 2^41; beyond, t is
+// a multiple of 2^-11 and k and f are read off its own bits, in integer steps
+// beside the sum: two operations more on the float64 pipe (t - rint(t), taken or
+// not) cost the direct sum 12 %, integer steps before the sum an explicit Eq. 17
+// over few visibilities 4 %, these 2 % there, 0.2 on a full batch and nothing on
+// the other float64 sums.
 static __device__ const double2 kSinCos1024[1024] =
 #include "sincos_table.inc"
     ;
 
-// t modulo whole turns, exactly: from 2^41 up the bits worth 2^40 and more are
-// shifted out of the significand and the exponent set to 2^40's. Integer steps:
-// they cost the explicit Eq. 17 0.5 % and the other float64 sums nothing, where
-// two operations of the float64 pipe, which those fill (t - rint(t), taken or
-// not), cost the direct sum 12 %.
-__device__ __forceinline__ double turns_below_2_41(double t)
-{
-    const uint32_t over = (static_cast<uint32_t>(__double2hiint(t)) & 0x7fffffffu) - 0x42800000u;
-    if (over < 0x7ff00000u - 0x42800000u) {   // 2^41 <= |t|, finite
-        const int by = min(static_cast<int>(over >> 20) + 1, 52);
-        const uint64_t b = static_cast<uint64_t>(__double_as_longlong(t));
-        t = __longlong_as_double(static_cast<long long>((b & 0x8000000000000000ull) | 0x4270000000000000ull |
-                                                        ((b << by) & 0x000fffffffffffffull)));
-    }
-    return t;
-}
-
 __device__ __forceinline__ void sincos_turns_f64(double t, double& s, double& c)
 {
-    t = turns_below_2_41(t);
     constexpr double kMagic = 6597069766656.0;                      // 1.5 * 2^42
     const double m = __dadd_rn(t, kMagic);
-    const double f = t - __dsub_rn(m, kMagic);                      // t - k/1024, exact
-    const double2 e = __ldg(&kSinCos1024[__double2loint(m) & 1023]);
+    double f = t - __dsub_rn(m, kMagic);                            // t - k/1024, exact
+    uint32_t k = static_cast<uint32_t>(__double2loint(m));
+    const int hi = __double2hiint(t), lo = __double2loint(t);
+    const uint32_t over = (static_cast<uint32_t>(hi) & 0x7fffffffu) - 0x42800000u;
+    if (over < 0x7ff00000u - 0x42800000u) {   // 2^41 <= |t|, finite: |t| = (2^52 + ...) 2^(by - 11), k its low bits
+        const uint32_t by = over >> 20;
+        k = by == 0 ? static_cast<uint32_t>(lo) >> 1 : by < 11 ? static_cast<uint32_t>(lo) << (by - 1) : 0u;
+        if (hi < 0) k = 0u - k;
+        f = __hiloint2double(by == 0 && (lo & 1) ? (hi & 0x80000000) | 0x3f400000 : 0, 0);
+    }
+    const double2 e = __ldg(&kSinCos1024[k & 1023u]);
     const double f2 = f * f;
     // sin 2 pi f = f (2 pi - (2 pi)^3/3! f^2 + (2 pi)^5/5! f^4)
     const double sx = f * fma(f2, fma(f2, 81.60524927607505, -41.34170224039976), 6.283185307179586);
