@@ -105,7 +105,7 @@ static int64_t sample_size(int v, const WaveletJob& jb)
 
 int choose_wavelet_variant(wt_tree t, const WaveletJob& jb, cudaStream_t s)
 {
-    const int fallback = default_wavelet_variant(jb.mode, jb.which, jb.J);
+    const int fallback = default_wavelet_variant(jb.mode, jb.which, jb.J, jb.n_vis);
     const char* pin = getenv("WT_WAVELET_VARIANT");
     if (pin && *pin) {
         const int v = atoi(pin);

@@ -551,13 +551,19 @@ int launch_wavelet(const WaveletJob& jb, int v, cudaStream_t s)
 
 // Default when nothing is tuned: the first variant that fits in a measured
 // preference order.
-int default_wavelet_variant(int mode, int which, int J)
+int default_wavelet_variant(int mode, int which, int J, int64_t n_vis)
 {
     // measured on the medium and large workloads (J = 12): the explicit
     // mixed sum runs best at 256 x 1 (its stack limits the CTAs per SM), the
     // regrouped one, whose stack is small, at 64 x 4 (the per-record work
     // shared by four visibilities), then 128 x 2; Eq. 16 (no stack) on packed
-    // pairs of visibilities at 128 x 2
+    // pairs of visibilities at 128 x 2. The double-float regrouped sum: at 128 x 1
+    // while that leaves an SM no more than two CTAs (10 000 visibilities, 1 880
+    // leaves: 523 us, 675 as pairs), then as pairs at 128 x 2 (60 000: 934 against
+    // 1 062; a million: 10.1 ms against 12.5).
+    if (mode == WT_FP64_DF && which == WT_SUM_EQ17_REGROUPED &&
+        n_vis > 2 * 128 * static_cast<int64_t>(num_sms()) && wavelet_variant_fits(2, mode, which, J))
+        return 2;
     static const int order_mixed[kNumWaveletVariants] = {0, 2, 1, 3, 4, 5, 6, 7, 8};
     static const int order_mixed16[kNumWaveletVariants] = {2, 7, 3, 4, 0, 1, 5, 6, 8};
     static const int order_mixed_rg[kNumWaveletVariants] = {4, 2, 7, 6, 3, 5, 0, 1, 8};

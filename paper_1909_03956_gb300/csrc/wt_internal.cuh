@@ -772,7 +772,7 @@ int wavelet_variant_shape(int v, int* nt, int* vpt);
 bool wavelet_variant_fits(int v, int mode, int which, int J);
 size_t wavelet_variant_smem(int v, int mode, int which, int J);
 int launch_wavelet(const WaveletJob& jb, int v, cudaStream_t s);
-int default_wavelet_variant(int mode, int which, int J);
+int default_wavelet_variant(int mode, int which, int J, int64_t n_vis = 0);
 bool wavelet_untuned(int mode, int which, int J);   // the default shape without timing
 // autotune.cu
 int choose_wavelet_variant(wt_tree t, const WaveletJob& jb, cudaStream_t s);

@@ -11,6 +11,9 @@ import math
 import numpy as np
 import pytest
 
+import oracle as O
+import synth
+
 torch = pytest.importorskip("torch")
 wt = pytest.importorskip("paper_1909_03956_gb300")
 
@@ -54,3 +57,22 @@ def test_blocks_are_no_worse(n):
         got[k] = float(v[0].real)
     err = got - exact
     assert np.sqrt(np.mean((err / exact) ** 2)) <= np.sqrt(np.mean((bar / exact) ** 2))
+
+
+@pytest.mark.parametrize("which", [wt.WT_SUM_EQ17_REGROUPED, wt.WT_SUM_EQ16])
+@pytest.mark.parametrize("beyond", [-1, 0, 1, 70])
+def test_shapes_without_tuning(which, beyond, monkeypatch):
+    """At the line where the default turns to pairs of visibilities; the form's
+    bar, 1e-10 of the fluxes' sum, against the oracle's sums."""
+    monkeypatch.setenv("WT_AUTOTUNE", "0")
+    n = 2 * 128 * torch.cuda.get_device_properties(0).multi_processor_count + beyond
+    g = np.random.default_rng(3)
+    l, m = g.uniform(-0.01, 0.01, (2, 40))
+    f = g.uniform(0.5, 1.5, 40)
+    dev = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    t = wt.wt_build_tree(dev(l), dev(m), dev(f), synth.RA0, synth.DEC0, 9)
+    uvw = g.uniform(-1000, 1000, (n, 3))
+    v = wt.wt_predict_vis(t, dev(uvw), mode=wt.WT_FP64_DF, which=which).cpu().numpy()
+    at = np.r_[0:300, n - 300:n]
+    ref = O.Tree(l, m, f, synth.RA0, synth.DEC0, 9).vis_eq17(uvw[at], 1)
+    assert np.max(np.abs(v[at] - ref)) <= 1e-10 * f.sum()
