@@ -554,12 +554,12 @@ TRAFFIC_BYTES = {("large_256ant_15993600vis_50000comp", "fast", "regrouped"): 38
 # x^2 4, sin x and cos x - 1 as double-floats 7, the rotation by the table
 # entry: four products of 4 and sums of 8, two signs), w eta into V 24 (two
 # products and sums), the parent's sum 16; per (vis, internal node): quarter 4,
-# w eta into V 24 and V renormalised 6 (a node of leaves: their block into V, 2
-# more), the parent's sum 16. The direct sum adds and renormalises a block every
-# four components (14 a block beside the products and sums, one sum saved: 3.5).
+# w eta into V 24, the parent's sum 16, and for each run of leaves its block into
+# V, 8 more than a leaf's sum (two nodes in three have one: 5). The direct sum
+# takes two blocks of four components at a time: 22 beside the products and sums.
 OPS_DF_LEAF = 32 + 74 + 24 + 16
-OPS_DFT_DF = 32 + 74 + 24 + 3.5   # per (vis, component) of the double-float direct sum
-OPS_DF_NODE = 4 + 24 + 6 + 16
+OPS_DFT_DF = 32 + 74 + 24 + 22 / 8   # per (vis, component) of the double-float direct sum
+OPS_DF_NODE = 4 + 24 + 16 + 5
 # Direct sum (k_dft_mixed, two visibilities x two components per step), FMA-pipe
 # element ops per (visibility, component): phase 18 on the head grid (the
 # grid pass; the exact pass's 29 only for tiles beyond the grid's range),
